@@ -161,6 +161,14 @@ struct GSeg {
 struct GTile {
   int g, m0, n0, pad;
 };
+// One T x T output tile of the FP64 GEMM (tt_gemm64.cu), with what the kernel
+// needs of its group: C at the tile's corner, rows x cols of it in use.
+struct FTile {
+  Ref C;
+  int m0, n0, rows, cols;
+  int seg0, seg1;
+  int ldc, flags;
+};
 struct GemmPlan {
   std::vector<GGroup> groups;
   std::vector<GSeg> segs;

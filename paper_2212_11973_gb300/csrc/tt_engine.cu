@@ -112,6 +112,7 @@ void upload(tt_ctx* c, const GemmPlan& p, DevGemmBuf& o) {
   o.checked = false;
   o.tc_checked = o.tc_ok = false;
   o.ntiles128 = o.ntilesp = 0;
+  o.d.ntilesf = o.d.tf = 0;
   o.choice = -1;
   for (int i = 0; i < 8; ++i) { o.key_p[i] = nullptr; o.key_lo[i] = 0; }
 }
@@ -150,6 +151,7 @@ void release(tt_ctx* c, DevGemmBuf& o) {
   dfree(c, o.maps);
   dfree(c, o.tiles128);
   dfree(c, o.tilesp);
+  dfree(c, o.tilesf);
   o.d = DevGemm();
   o.host = GemmPlan();
   o.checked = o.tc_checked = o.tc_ok = false;
@@ -718,6 +720,22 @@ struct Eng {
     return true;
   }
 
+  // FP64 launch of a plan; its tile list is built and uploaded the first time
+  // (in the uncaptured step, as for the tensor maps)
+  void f64(DevGemmBuf& g, const Bases& b) {
+    if (g.d.tf == 0) {
+      if (r->capturing) throw Err{TT_ERR_STATE, "FP64 tile list missing during graph capture"};
+      g.d.tf = f64_tile_size(g.host);
+      const std::vector<FTile> t = f64_tiles(g.host, g.d.tf);
+      ensure(c, g.tilesf, t.size() * sizeof(FTile) + 16);
+      if (!t.empty()) CK(cudaMemcpyAsync(g.tilesf.p, t.data(), t.size() * sizeof(FTile), cudaMemcpyHostToDevice, st));
+      CK(cudaStreamSynchronize(st));
+      g.d.tilesf = (FTile*)g.tilesf.p;
+      g.d.ntilesf = (int)t.size();
+    }
+    CK(launch_gemm_f64(g.d, b, st));
+  }
+
   // one launch of a split-BF16 plan on kernel k (tcgen05 kernels need prep_tc)
   void launch_split(DevGemmBuf& g, const Bases& b, int k) {
     if (k != TK_MMA64 && !r->tcerr.p) {
@@ -827,7 +845,7 @@ struct Eng {
     } else if (f64_kernel == 2) {
       CK(launch_gemm_df(g.d, b, st));
     } else {
-      CK(launch_gemm_f64(g.d, b, st));
+      f64(g, b);
     }
     prof_end(e);
     count();
@@ -1115,7 +1133,10 @@ struct Eng {
     CK(cudaMemsetAsync(q.fail.p, 0, q.h.jobs.size() * sizeof(int), st));
     // the mixed modes run the Gram and apply GEMMs in double-float on the
     // FP32 pipe (their error budget is far above ~2^-46), FP64 mode in FP64
-    auto qr_gemm = [&](const DevGemmBuf& g) { CK(mixed() ? launch_gemm_df(g.d, b, st) : launch_gemm_f64(g.d, b, st)); };
+    auto qr_gemm = [&](DevGemmBuf& g) {
+      if (mixed()) CK(launch_gemm_df(g.d, b, st));
+      else f64(g, b);
+    };
     for (int p = 0; p < 3; ++p) {
       long e = prof_begin(11, q.gram[p].d.flops);
       qr_gemm(q.gram[p]);
@@ -1131,8 +1152,8 @@ struct Eng {
       count(3);
     }
     const long e2 = prof_begin(11, q.tt.d.flops + q.rf.d.flops);
-    CK(launch_gemm_f64(q.tt.d, b, st));
-    CK(launch_gemm_f64(q.rf.d, b, st));
+    f64(q.tt, b);
+    f64(q.rf, b);
     prof_end(e2);
     count(2);
     if (!r->qrfb.p) {
@@ -1480,7 +1501,7 @@ struct Eng {
       b2.p[S_X] = r->A[j - 1].p;
       b2.p[S_AUX] = r->Sb.p;
       b2.p[S_Y] = newP.p;
-      CK(launch_gemm_f64(abd.d, b2, st));
+      f64(abd, b2);
       CK(cudaStreamSynchronize(st));
       std::swap(r->A[j], newA);
       std::swap(r->A[j - 1], newP);
@@ -1625,7 +1646,7 @@ struct Eng {
       b3.p[S_X] = r->A[j + 1].p;
       b3.p[S_AUX] = Sm.p;
       b3.p[S_Y] = newN.p;
-      CK(launch_gemm_f64(abd.d, b3, st));
+      f64(abd, b3);
       CK(cudaStreamSynchronize(st));
       release(c, abd);
       std::swap(r->A[j], newA);
@@ -1839,9 +1860,9 @@ struct Eng {
       b.p[S_T1] = r->T1.p;
       b.p[S_AUX] = r->el0.p;
       b.p[S_AUX2] = r->el1.p;
-      CK(launch_gemm_f64(md.t.d, b, st));
+      f64(md.t, b);
       CK(launch_local_obs((const ObsItem*)md.items.p, md.nitems, dptr(r->A[j]), dptr(r->T1), dptr(part2), ob, st));
-      CK(launch_gemm_f64(md.el.d, b, st));
+      f64(md.el, b);
       std::swap(r->el0, r->el1);
     }
     double hv[4];
@@ -1912,7 +1933,7 @@ struct Eng {
     b.p[S_AUX] = r->A[j + 1].p;
     b.p[S_T1] = r->T1.p;
     b.p[S_Y] = Cbuf.p;
-    CK(launch_gemm_f64(gd.d, b, st));
+    f64(gd, b);
     CK(launch_copy(cd.d, b, st));
     CK(cudaStreamSynchronize(st));
     release(c, gd);
@@ -2191,9 +2212,9 @@ struct Eng {
         b.p[S_X] = (void*)x;
         b.p[S_L] = r->L[j].p;
         b.p[S_R] = r->R[j + 2].p;
-        CK(launch_gemm_f64(s1.d, b, st));
+        f64(s1, b);
         CK(launch_gather(s2.d, b, 0, 0, st));
-        CK(launch_gemm_f64(s3.d, b, st));
+        f64(s3, b);
       }
     };
     lanczos(dptr(Cbuf), n, t, apply);

@@ -56,6 +56,7 @@ struct DevGemmBuf {
   // tcgen05 path: eligibility, 128 x 128 tile list, per-segment tensor maps
   bool tc_checked = false, tc_ok = false;
   DBuf maps, tiles128, tilesp;
+  DBuf tilesf;  // FP64 kernel's tiles (built for its first launch)
   int ntiles128 = 0, ntilesp = 0;  // 128 x 128 tiles (tc), 128 x 64 tiles (persistent tc)
   // autotuned kernel of a split-BF16 plan: -1 not chosen yet, else a TcKernel
   int choice = -1;

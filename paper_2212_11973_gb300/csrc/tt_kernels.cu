@@ -1,6 +1,7 @@
 // Device kernels of the tanTRG hot path (sm_103a).
 //
-//  * grouped, segmented GEMM (FP64 FMA; split-BF16 x3 on the tensor cores):
+//  * grouped, segmented GEMM (double-float on the FP32 pipe; split-BF16 on the
+//    tensor cores; FP64 in tt_gemm64.cu):
 //    every contraction of the H_eff apply (Supplement, Fig. "Lanczos": L_i A_i,
 //    then H_i, then R_i), the bond apply (Fig. "optimalB"(d)), the environment
 //    updates and the absorb step is a list of groups C_g = sum_seg A_seg B_seg;
@@ -38,85 +39,12 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// ---------------------------------------------------------------------------
-// FP64 grouped GEMM: one 64 x 64 output tile per CTA, 256 threads, 4 x 4 per
-// thread, K staged through shared memory in chunks of 16.
-// ---------------------------------------------------------------------------
 constexpr int FBM = 64, FBN = 64, FBK = 16;
 
-__global__ void __launch_bounds__(256) gemm_f64_kernel(const GGroup* __restrict__ groups,
-                                                       const GSeg* __restrict__ segs,
-                                                       const GTile* __restrict__ tiles, Bases bs) {
-  __shared__ double As[FBK][FBM + 1];
-  __shared__ double Bs[FBK][FBN + 1];
-  const GTile tl = tiles[blockIdx.x];
-  const GGroup g = groups[tl.g];
-  const int tid = threadIdx.x;
-  const int tx = tid % 16, ty = tid / 16;  // 16 x 16 threads, each 4 x 4 outputs
-  double acc[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-
-  for (int si = g.seg0; si < g.seg1; ++si) {
-    const GSeg sg = segs[si];
-    const double* A = rptr<const double>(bs, sg.A);
-    const double* B = rptr<const double>(bs, sg.B);
-    for (int k0 = 0; k0 < sg.K; k0 += FBK) {
-      // load A tile: FBM x FBK logical (m, k)
-      for (int e = tid; e < FBM * FBK; e += 256) {
-        int mm, kk;
-        if (sg.tA) { mm = e % FBM; kk = e / FBM; } else { kk = e % FBK; mm = e / FBK; }
-        int gm = tl.m0 + mm, gk = k0 + kk;
-        double v = 0.0;
-        if (gm < g.M && gk < sg.K)
-          v = sg.tA ? A[(long long)gk * sg.lda + gm] : A[(long long)gm * sg.lda + gk];
-        As[kk][mm] = v;
-      }
-      for (int e = tid; e < FBN * FBK; e += 256) {
-        int nn, kk;
-        if (sg.tB) { kk = e % FBK; nn = e / FBK; } else { nn = e % FBN; kk = e / FBN; }
-        int gn = tl.n0 + nn, gk = k0 + kk;
-        double v = 0.0;
-        if (gn < g.N && gk < sg.K)
-          v = sg.tB ? B[(long long)gn * sg.ldb + gk] : B[(long long)gk * sg.ldb + gn];
-        Bs[kk][nn] = v;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int kk = 0; kk < FBK; ++kk) {
-        double a[4], b[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-      }
-      __syncthreads();
-    }
-  }
-  double* C = rptr<double>(bs, g.C);
-  const bool accum = g.flags & 1;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    int gm = tl.m0 + ty + 16 * i;
-    if (gm >= g.M) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      int gn = tl.n0 + tx + 16 * j;
-      if (gn >= g.N) continue;
-      double* c = C + (long long)gm * g.ldc + gn;
-      *c = accum ? *c + acc[i][j] : acc[i][j];
-    }
-  }
-}
-
 // ---------------------------------------------------------------------------
-// The same grouped GEMM in double-float arithmetic on the FP32 pipe (GB300
+// Grouped GEMM in double-float arithmetic on the FP32 pipe: one 64 x 64 output
+// tile per CTA, 256 threads, 4 x 4 per thread, K staged through shared memory
+// in chunks of 16 (GB300
 // issues ~2 FP64 FMA per clock per SM against 128 FP32): FP64 operands split
 // into float pairs (hi, lo) as they are staged, every product by the FMA
 // TwoProduct with the cross terms, every sum by TwoSum into an unnormalised
@@ -1138,12 +1066,6 @@ inline int grid_for(long long n) {
 // host wrappers
 // ---------------------------------------------------------------------------
 int lanczos_nblk() { return NBLK; }
-
-cudaError_t launch_gemm_f64(const DevGemm& g, const Bases& b, cudaStream_t s) {
-  if (g.ntiles64 == 0) return cudaSuccess;
-  gemm_f64_kernel<<<g.ntiles64, 256, 0, s>>>(g.groups, g.segs, g.tiles64, b);
-  return cudaGetLastError();
-}
 
 cudaError_t launch_gemm_df(const DevGemm& g, const Bases& b, cudaStream_t s) {
   if (g.ntiles64 == 0) return cudaSuccess;
