@@ -1088,18 +1088,13 @@ struct Eng {
     double* part = dptr(r->partial);
     KrylovState* ks = (KrylovState*)r->ks.p;
     const int64_t ldq = r->ldq;
-    CK(k_norm_init(x, n, part, ks, Q, st)); count(3);
+    CK(k_lanczos_begin(x, n, part, ks, Q, st)); count(2);
     for (int k = 0; k < K; ++k) {
       apply(Q + (int64_t)k * ldq, w);
-      CK(k_dots_alpha(Q, ldq, k, w, n, part, ks, st)); count(2);
-      CK(k_three_term(Q, ldq, k, w, n, ks, st)); count();
-      CK(k_cgs_pass(Q, ldq, k, w, n, part, ks, 0, BREAKDOWN_TOL, K, nullptr, st)); count(3);
-      CK(k_cgs_pass(Q, ldq, k, w, n, part, ks, 1, BREAKDOWN_TOL, K, k + 1 < K ? Q + (int64_t)(k + 1) * ldq : nullptr, st));
-      count(k + 1 < K ? 5 : 4);
+      CK(k_lanczos_step(Q, ldq, k, K, w, n, part, ks, (RhoScalars*)r->rs.p, BREAKDOWN_TOL, t, st));
+      count(k + 1 < K ? 3 : 2);
     }
-    CK(k_krylov_exp(ks, t, K, st)); count();
-    CK(k_combine(Q, ldq, ks, x, n, part, nullptr, st)); count();
-    CK(k_finish_normalise(x, n, part, ks, (RhoScalars*)r->rs.p, st)); count(2);
+    CK(k_lanczos_end(Q, ldq, ks, x, n, st)); count();
   }
 
   void site_exp(int j, double t) {
@@ -2341,6 +2336,7 @@ void alloc_rho_arrays(tt_rho* r) {
   tt_ctx* c = r->ctx;
   ensure(c, r->partial, (size_t)lanczos_nblk() * 17 * 8);
   ensure(c, r->ks, sizeof(KrylovState));
+  CK(cudaMemsetAsync(r->ks.p, 0, sizeof(KrylovState), c->st));
   ensure(c, r->rs, sizeof(RhoScalars));
   CK(cudaMemsetAsync(r->rs.p, 0, sizeof(RhoScalars), c->st));
 }

@@ -6,10 +6,7 @@
 //    then H_i, then R_i), the bond apply (Fig. "optimalB"(d)), the environment
 //    updates and the absorb step is a list of groups C_g = sum_seg A_seg B_seg;
 //  * W gather: applies the sparse MPO tensor between the two GEMM stages;
-//  * Lanczos vector kernels in FP64 (Supplement, "Lanczos-based exponential
-//    method"), with deterministic two-stage reductions;
-//  * the small Krylov exponential exp(t T) e_1 by scaling and squaring of a
-//    Taylor polynomial (Moler & Van Loan);
+//  * norms and dot products with deterministic two-stage reductions;
 //  * Householder QR (FP64) of the per-sector gauge matrices.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -407,37 +404,8 @@ __global__ void split_bf16_kernel(const double* __restrict__ x, long long n, int
 
 
 // ---------------------------------------------------------------------------
-// Lanczos vector kernels
+// Norms and dot products of flat vectors (the Lanczos steps: tt_lanczos.cu)
 // ---------------------------------------------------------------------------
-// partial[blk * 17 + j] = sum over this block's chunk of Q_j . w   (j < nv)
-template <int MAXV>
-__global__ void __launch_bounds__(VT) multidot_kernel(const double* __restrict__ Q, long long ldq, int j0, int nv,
-                                                      const double* __restrict__ w, long long n,
-                                                      double* __restrict__ partial) {
-  double acc[MAXV];
-#pragma unroll
-  for (int j = 0; j < MAXV; ++j) acc[j] = 0.0;
-  for (long long i = blockIdx.x * (long long)VT + threadIdx.x; i < n; i += (long long)gridDim.x * VT) {
-    double wi = w[i];
-#pragma unroll
-    for (int j = 0; j < MAXV; ++j)
-      if (j < nv) acc[j] = fma(Q[(long long)(j0 + j) * ldq + i], wi, acc[j]);
-  }
-  __shared__ double red[VT / 32][MAXV];
-  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-#pragma unroll
-  for (int j = 0; j < MAXV; ++j) {
-    double v = warp_sum(acc[j]);
-    if (lane == 0) red[wp][j] = v;
-  }
-  __syncthreads();
-  if (threadIdx.x < nv) {
-    double s = 0.0;
-    for (int q = 0; q < VT / 32; ++q) s += red[q][threadIdx.x];
-    partial[blockIdx.x * 17 + threadIdx.x] = s;
-  }
-}
-
 __global__ void sumsq_kernel(const double* __restrict__ v, long long n, double* __restrict__ partial) {
   double acc = 0.0;
   for (long long i = blockIdx.x * (long long)VT + threadIdx.x; i < n; i += (long long)gridDim.x * VT)
@@ -465,22 +433,6 @@ __device__ void finalize_sums(const double* partial, int nblk, int nv, double* o
   }
 }
 
-__global__ void norm_init_finalize(const double* partial, int nblk, KrylovState* ks) {
-  __shared__ double s;
-  finalize_sums(partial, nblk, 1, &s);
-  __syncwarp();
-  if (threadIdx.x == 0) {
-    double nb = sqrt(s);
-    ks->nb = nb;
-    ks->hscale = 0.0;
-    ks->resid = 0.0;
-    ks->kdim = 0;
-    ks->broken = 0;
-    ks->bad = !isfinite(nb) ? 1 : 0;
-    for (int j = 0; j < 17; ++j) { ks->alpha[j] = 0; ks->beta[j] = 0; ks->h[j] = 0; ks->c[j] = 0; }
-  }
-}
-
 __global__ void scale_kernel(const double* __restrict__ v, long long n, const double* __restrict__ denom,
                              const int* __restrict__ dead, double* __restrict__ out) {
   const double d = *denom;
@@ -488,179 +440,6 @@ __global__ void scale_kernel(const double* __restrict__ v, long long n, const do
   const double inv = z ? 0.0 : 1.0 / d;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     out[i] = v[i] * inv;
-}
-
-__global__ void alpha_finalize(const double* partial, int nblk, int k, KrylovState* ks) {
-  __shared__ double s;
-  finalize_sums(partial, nblk, 1, &s);
-  __syncwarp();
-  if (threadIdx.x == 0 && !ks->broken) ks->alpha[k] = s;
-}
-
-__global__ void three_term_kernel(const double* __restrict__ Q, long long ldq, int k, double* __restrict__ w,
-                                  long long n, const KrylovState* __restrict__ ks) {
-  const double a = ks->alpha[k];
-  const double b = (k > 0) ? ks->beta[k - 1] : 0.0;
-  const double* qk = Q + (long long)k * ldq;
-  const double* qp = Q + (long long)(k > 0 ? k - 1 : 0) * ldq;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    double v = w[i] - a * qk[i];
-    if (k > 0) v -= b * qp[i];
-    w[i] = v;
-  }
-}
-
-__global__ void h_finalize(const double* partial, int nblk, int nv, KrylovState* ks) {
-  finalize_sums(partial, nblk, nv, ks->h);
-}
-
-// w -= sum_j h_j Q_j ; optional partial ||w||^2
-__global__ void __launch_bounds__(VT) axpy_multi_kernel(const double* __restrict__ Q, long long ldq, int nv,
-                                                        const KrylovState* __restrict__ ks, double* __restrict__ w,
-                                                        long long n, double* __restrict__ partial) {
-  __shared__ double h[17];
-  if (threadIdx.x < 17) h[threadIdx.x] = ks->h[threadIdx.x];
-  __syncthreads();
-  double acc = 0.0;
-  for (long long i = blockIdx.x * (long long)VT + threadIdx.x; i < n; i += (long long)gridDim.x * VT) {
-    double v = w[i];
-    for (int j = 0; j < nv; ++j) v -= h[j] * Q[(long long)j * ldq + i];
-    w[i] = v;
-    acc = fma(v, v, acc);
-  }
-  if (partial) {
-    __shared__ double red[VT / 32];
-    double s = warp_sum(acc);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double t = 0.0;
-      for (int q = 0; q < VT / 32; ++q) t += red[q];
-      partial[blockIdx.x * 17] = t;
-    }
-  }
-}
-
-// beta_k = ||w||; breakdown test of the oracle; stores beta (or 0 if broken).
-__global__ void beta_finalize(const double* partial, int nblk, int k, int K, double tol, KrylovState* ks) {
-  __shared__ double s;
-  finalize_sums(partial, nblk, 1, &s);
-  __syncwarp();
-  if (threadIdx.x != 0) return;
-  if (ks->broken) {
-    ks->beta[k] = 0.0;
-    return;
-  }
-  double b = sqrt(s);
-  if (!isfinite(b) || !isfinite(ks->alpha[k])) ks->bad = 1;
-  double hs = fmax(ks->hscale, fabs(ks->alpha[k]) + b);
-  ks->hscale = hs;
-  ks->kdim = k + 1;
-  if (k == K - 1) {
-    ks->beta[k] = b;  // residual norm, not part of T
-    return;
-  }
-  if (b <= tol * hs) {
-    ks->broken = 1;
-    ks->beta[k] = 0.0;
-    return;
-  }
-  ks->beta[k] = b;
-}
-
-// c = exp(t T) e_1 for the kdim x kdim tridiagonal T, by scaling and squaring
-// with a degree-18 Taylor polynomial (Moler & Van Loan, "Nineteen dubious
-// ways", method 3): M = t T / 2^s with ||M||_1 <= 1/4, E = sum_k M^k / k!
-// (Horner), then E <- E^2 s times.  One thread per matrix entry (kdim <= 16).
-__global__ void __launch_bounds__(256) krylov_exp_kernel(KrylovState* ks, double t, int K) {
-  __shared__ double M[16][16], E[16][16], P[16][16];
-  __shared__ int m_s, s_s;
-  const int tid = threadIdx.x, i = tid / 16, j = tid % 16;
-  if (tid == 0) {
-    const int m = ks->kdim;
-    double nrm = 0.0;  // ||t T||_1 (T symmetric tridiagonal)
-    for (int c = 0; c < m; ++c) {
-      double col = fabs(ks->alpha[c]);
-      if (c > 0) col += fabs(ks->beta[c - 1]);
-      if (c + 1 < m) col += fabs(ks->beta[c]);
-      nrm = fmax(nrm, fabs(t) * col);
-    }
-    int sq = 0;
-    while (nrm > 0.25 && sq < 60) { nrm *= 0.5; ++sq; }
-    m_s = m;
-    s_s = sq;
-  }
-  __syncthreads();
-  const int m = m_s, sq = s_s;
-  const double scale = ldexp(t, -sq);
-  double mij = 0.0;
-  if (i < m && j < m) {
-    if (i == j) mij = ks->alpha[i];
-    else if (j == i + 1) mij = ks->beta[i];
-    else if (i == j + 1) mij = ks->beta[j];
-    mij *= scale;
-  }
-  M[i][j] = mij;
-  E[i][j] = (i == j && i < m) ? 1.0 : 0.0;  // Horner: E = I + M/18, then E = I + M E / k
-  __syncthreads();
-  for (int k = 18; k >= 1; --k) {
-    double acc = 0.0;
-    for (int q = 0; q < m; ++q) acc = fma(M[i][q], E[q][j], acc);
-    __syncthreads();
-    E[i][j] = (i < m && j < m) ? ((i == j ? 1.0 : 0.0) + acc / (double)k) : 0.0;
-    __syncthreads();
-  }
-  for (int r = 0; r < sq; ++r) {
-    double acc = 0.0;
-    for (int q = 0; q < m; ++q) acc = fma(E[i][q], E[q][j], acc);
-    P[i][j] = acc;
-    __syncthreads();
-    E[i][j] = P[i][j];
-    __syncthreads();
-  }
-  if (tid < 17) ks->c[tid] = (tid < m) ? E[tid][0] : 0.0;
-  if (tid == 0) ks->resid = (!ks->broken && m == K) ? ks->nb * ks->beta[K - 1] * fabs(E[K - 1][0]) : 0.0;
-}
-
-__global__ void __launch_bounds__(VT) combine_kernel(const double* __restrict__ Q, long long ldq,
-                                                     const KrylovState* __restrict__ ks, double* __restrict__ y,
-                                                     long long n, double* __restrict__ partial) {
-  __shared__ double c[17];
-  __shared__ int m;
-  if (threadIdx.x < 17) c[threadIdx.x] = ks->c[threadIdx.x] * ks->nb;
-  if (threadIdx.x == 0) m = ks->kdim;
-  __syncthreads();
-  double acc = 0.0;
-  for (long long i = blockIdx.x * (long long)VT + threadIdx.x; i < n; i += (long long)gridDim.x * VT) {
-    double v = 0.0;
-    for (int j = 0; j < m; ++j) v = fma(c[j], Q[(long long)j * ldq + i], v);
-    y[i] = v;
-    acc = fma(v, v, acc);
-  }
-  __shared__ double red[VT / 32];
-  double s = warp_sum(acc);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int q = 0; q < VT / 32; ++q) t += red[q];
-    partial[blockIdx.x * 17] = t;
-  }
-}
-
-__global__ void nrm_finalize(const double* partial, int nblk, KrylovState* ks, RhoScalars* rs) {
-  __shared__ double s;
-  finalize_sums(partial, nblk, 1, &s);
-  __syncwarp();
-  if (threadIdx.x != 0) return;
-  double nrm = sqrt(s);
-  ks->nrm = nrm;
-  if (!isfinite(nrm) || nrm == 0.0 || ks->bad) {
-    rs->bad = 1;
-    return;
-  }
-  rs->logscale += log(nrm);
-  rs->resid_max = fmax(rs->resid_max, ks->resid);
 }
 
 // ---------------------------------------------------------------------------
@@ -1112,55 +891,6 @@ cudaError_t launch_split_copy(const DevCopy& c, const Bases& b, int nsplit, cuda
   return cudaGetLastError();
 }
 
-cudaError_t k_norm_init(const double* v, int64_t n, double* partial, KrylovState* ks, double* q0, cudaStream_t s) {
-  int g = grid_for(n);
-  sumsq_kernel<<<g, VT, 0, s>>>(v, n, partial);
-  norm_init_finalize<<<1, 32, 0, s>>>(partial, g, ks);
-  scale_kernel<<<g, VT, 0, s>>>(v, n, &ks->nb, nullptr, q0);
-  return cudaGetLastError();
-}
-
-cudaError_t k_dots_alpha(const double* Q, int64_t ldq, int k, const double* w, int64_t n, double* partial,
-                         KrylovState* ks, cudaStream_t s) {
-  int g = grid_for(n);
-  multidot_kernel<1><<<g, VT, 0, s>>>(Q, ldq, k, 1, w, n, partial);
-  alpha_finalize<<<1, 32, 0, s>>>(partial, g, k, ks);
-  return cudaGetLastError();
-}
-
-cudaError_t k_three_term(const double* Q, int64_t ldq, int k, double* w, int64_t n, KrylovState* ks, cudaStream_t s) {
-  three_term_kernel<<<grid_for(n), VT, 0, s>>>(Q, ldq, k, w, n, ks);
-  return cudaGetLastError();
-}
-
-cudaError_t k_cgs_pass(const double* Q, int64_t ldq, int k, double* w, int64_t n, double* partial, KrylovState* ks,
-                       int last, double tol, int K, double* qnext, cudaStream_t s) {
-  int g = grid_for(n);
-  int nv = k + 1;
-  if (nv <= 4) multidot_kernel<4><<<g, VT, 0, s>>>(Q, ldq, 0, nv, w, n, partial);
-  else if (nv <= 8) multidot_kernel<8><<<g, VT, 0, s>>>(Q, ldq, 0, nv, w, n, partial);
-  else multidot_kernel<17><<<g, VT, 0, s>>>(Q, ldq, 0, nv, w, n, partial);
-  h_finalize<<<1, 32, 0, s>>>(partial, g, nv, ks);
-  axpy_multi_kernel<<<g, VT, 0, s>>>(Q, ldq, nv, ks, w, n, last ? partial : nullptr);
-  if (last) {
-    beta_finalize<<<1, 32, 0, s>>>(partial, g, k, K, tol, ks);
-    if (k < K - 1) scale_kernel<<<g, VT, 0, s>>>(w, n, &ks->beta[k], &ks->broken, qnext);
-  }
-  return cudaGetLastError();
-}
-
-cudaError_t k_krylov_exp(KrylovState* ks, double t, int K, cudaStream_t s) {
-  krylov_exp_kernel<<<1, 256, 0, s>>>(ks, t, K);
-  return cudaGetLastError();
-}
-
-cudaError_t k_combine(const double* Q, int64_t ldq, const KrylovState* ks, double* y, int64_t n, double* partial,
-                      KrylovState* ksw, cudaStream_t s) {
-  (void)ksw;
-  combine_kernel<<<grid_for(n), VT, 0, s>>>(Q, ldq, ks, y, n, partial);
-  return cudaGetLastError();
-}
-
 cudaError_t k_dot_plain(const double* x, const double* y, int64_t n, double* partial, double* out, cudaStream_t s) {
   int g = grid_for(n);
   dot_kernel<<<g, VT, 0, s>>>(x, y, n, partial);
@@ -1236,15 +966,6 @@ cudaError_t k_normalise_inplace(double* v, int64_t n, double* partial, KrylovSta
   sumsq_kernel<<<g, VT, 0, s>>>(v, n, partial);
   plain_nrm_finalize<<<1, 32, 0, s>>>(partial, g, ks, rs);
   scale_kernel<<<g, VT, 0, s>>>(v, n, &ks->nrm, nullptr, v);
-  return cudaGetLastError();
-}
-
-// Normalisation after the Krylov combination: finalize ||y|| then y /= ||y||.
-cudaError_t k_finish_normalise(double* y, int64_t n, double* partial, KrylovState* ks, RhoScalars* rs,
-                               cudaStream_t s) {
-  int g = grid_for(n);
-  nrm_finalize<<<1, 32, 0, s>>>(partial, g, ks, rs);
-  scale_kernel<<<g, VT, 0, s>>>(y, n, &ks->nrm, nullptr, y);
   return cudaGetLastError();
 }
 

@@ -65,7 +65,8 @@ struct DevDigit {
 struct KrylovState {
   double alpha[17];
   double beta[17];
-  double h[17];
+  double h[17];     // first Gram-Schmidt pass
+  double h2[17];    // second
   double c[17];
   double nb;        // ||v||
   double hscale;    // max(|alpha_j| + beta_j)
@@ -74,7 +75,7 @@ struct KrylovState {
   int kdim;         // Krylov dimension in use
   int broken;       // breakdown seen
   int bad;          // NaN / Inf seen
-  int pad;
+  unsigned ticket;  // CTAs arrived at the current reduction (zero between launches)
 };
 
 // Global accumulators of a state (device).
@@ -133,21 +134,19 @@ int gather_digits_max_contribs();
 cudaError_t launch_gemm_tc(const GGroup* groups, const GSeg* segs, const GTile* tiles128, int ntiles,
                            const void* maps, const Bases& b, int nsplit, int* err, long long wait_ns, cudaStream_t s);
 
-// Lanczos exponential steps on flat FP64 vectors of length n.  Q holds the
-// Krylov basis with leading dimension ldq.  `partial` is scratch of
-// nblk * 17 doubles.
+// Lanczos exponential on flat FP64 vectors of length n (tt_lanczos.cu).  Q holds
+// the Krylov basis with leading dimension ldq; `partial` is scratch of
+// lanczos_nblk() * 17 doubles; ks->ticket must be zero before the first use.
 int lanczos_nblk();
-cudaError_t k_norm_init(const double* v, int64_t n, double* partial, KrylovState* ks, double* q0, cudaStream_t s);
-cudaError_t k_dots_alpha(const double* Q, int64_t ldq, int k, const double* w, int64_t n, double* partial,
-                         KrylovState* ks, cudaStream_t s);
-cudaError_t k_three_term(const double* Q, int64_t ldq, int k, double* w, int64_t n, KrylovState* ks, cudaStream_t s);
-cudaError_t k_cgs_pass(const double* Q, int64_t ldq, int k, double* w, int64_t n, double* partial, KrylovState* ks,
-                       int last, double breakdown_tol, int K, double* qnext, cudaStream_t s);
-cudaError_t k_krylov_exp(KrylovState* ks, double t, int K, cudaStream_t s);
-cudaError_t k_combine(const double* Q, int64_t ldq, const KrylovState* ks, double* y, int64_t n, double* partial,
-                      KrylovState* ksw, cudaStream_t s);
-// after k_combine (same n): finalize ||y||, logscale += ln ||y||, y /= ||y||
-cudaError_t k_finish_normalise(double* y, int64_t n, double* partial, KrylovState* ks, RhoScalars* rs, cudaStream_t s);
+// ks reset, ks->nb = |x|, q0 = x / |x|
+cudaError_t k_lanczos_begin(const double* x, int64_t n, double* partial, KrylovState* ks, double* q0, cudaStream_t s);
+// step k of K after w = H q_k: alpha_k, beta_k and q_{k+1} (in Q); the last
+// step leaves the normalised coefficients of exp(t T) e_1 in ks and adds the
+// log of the norm to rs.  Three launches, two for the last step.
+cudaError_t k_lanczos_step(double* Q, int64_t ldq, int k, int K, double* w, int64_t n, double* partial, KrylovState* ks,
+                           RhoScalars* rs, double breakdown_tol, double t, cudaStream_t s);
+// y = sum_j ks->c[j] q_j
+cudaError_t k_lanczos_end(const double* Q, int64_t ldq, const KrylovState* ks, double* y, int64_t n, cudaStream_t s);
 
 // v /= ||v||, logscale += ln ||v|| (rs->bad set on zero / non-finite norm)
 cudaError_t k_normalise_inplace(double* v, int64_t n, double* partial, KrylovState* ks, RhoScalars* rs, cudaStream_t s);
