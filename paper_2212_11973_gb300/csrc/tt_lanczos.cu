@@ -91,12 +91,16 @@ __device__ __forceinline__ bool publish(double* acc, double extra, double* __res
     if (lane == 0) red[wp][V] = x;
   }
   __syncthreads();
-  if (threadIdx.x < V + (EXTRA ? 1 : 0)) {
-    double t = red[0][threadIdx.x];
+  {  // the warps' sums: LW lanes per value
+    constexpr int NV = V + (EXTRA ? 1 : 0);
+    const int j = threadIdx.x / LW, q = threadIdx.x % LW;
+    double t = j < NV ? red[q][j] : 0.0;
 #pragma unroll
-    for (int q = 1; q < LW; ++q) t += red[q][threadIdx.x];
-    partial[blockIdx.x * LMAX + threadIdx.x] = t;
-    __threadfence();
+    for (int o = LW / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (j < NV && q == 0) {
+      partial[blockIdx.x * LMAX + j] = t;
+      __threadfence();
+    }
   }
   __syncthreads();
   if (threadIdx.x == 0) last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;
@@ -106,15 +110,15 @@ __device__ __forceinline__ bool publish(double* acc, double extra, double* __res
 }
 
 // out[j] (shared, j < nv <= LMAX) = sum over the CTAs of partial[. * LMAX + j]
-// in a fixed order: 8 lanes per value, 32 values' worth of threads
+// in a fixed order: a warp per value
 __device__ __forceinline__ void total(const double* __restrict__ partial, int nblk, int nv, double* out) {
-  const int j = threadIdx.x >> 3, q = threadIdx.x & 7;
-  double s = 0.0;
-  if (j < nv)
-    for (int b = q; b < nblk; b += 8) s += __ldcg(&partial[b * LMAX + j]);
-#pragma unroll
-  for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (j < nv && q == 0) out[j] = s;
+  const int wp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int j = wp; j < nv; j += LW) {
+    double s = 0.0;
+    for (int b = lane; b < nblk; b += 32) s += __ldcg(&partial[b * LMAX + j]);
+    s = warp_sum1(s);
+    if (lane == 0) out[j] = s;
+  }
   __syncthreads();
 }
 
