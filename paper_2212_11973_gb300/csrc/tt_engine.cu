@@ -725,7 +725,9 @@ struct Eng {
   void f64(DevGemmBuf& g, const Bases& b) {
     if (g.d.tf == 0) {
       if (r->capturing) throw Err{TT_ERR_STATE, "FP64 tile list missing during graph capture"};
-      g.d.tf = f64_tile_size(g.host);
+      const F64Shape sh = f64_shape(g.host);
+      g.d.tf = sh.T;
+      g.d.wkf = sh.wk;
       const std::vector<FTile> t = f64_tiles(g.host, g.d.tf);
       ensure(c, g.tilesf, t.size() * sizeof(FTile) + 16);
       if (!t.empty()) CK(cudaMemcpyAsync(g.tilesf.p, t.data(), t.size() * sizeof(FTile), cudaMemcpyHostToDevice, st));

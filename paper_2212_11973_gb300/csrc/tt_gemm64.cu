@@ -16,13 +16,17 @@
 // steps ahead across segment boundaries; no shared memory, no barrier in the
 // loop.
 //
-// The tile size T is chosen per plan (f64_tile_size): the largest of 32, 16, 8
-// whose longest tile is at most a quarter of one SM's share of the plan.
+// T and the number of warps on a tile are chosen per plan (f64_shape): the
+// largest of 32, 16, 8 whose longest tile is at most a quarter of one SM's (or,
+// for one-warp tiles, one sub-partition's) share of the plan.  Where no K is
+// above 128 a tile belongs to one warp: splitting 3 to 12 K steps over four
+// warps leaves some of them idle, and the sum of the four shares costs as much
+// FP64 work as 3 of the K steps' multiply-adds per output.
 //
 // Measured against 64 x 64 DFMA tiles with a K loop per CTA (which padded a
 // sector of 12 to 64 and left most SMs idle behind a few long tiles): FP64
-// beta-step of a 4x8 cylinder at D = 256 961 -> 162 ms, of the 2x2 cluster at
-// D = 64 24.3 -> 5.4 ms; measurement and QR factors of a D = 300 exact-split
+// beta-step of a 4x8 cylinder at D = 256 961 -> 162 ms (140 -> 135 ms by the
+// one-warp tiles later), of the 2x2 cluster at D = 64 24.3 -> 5.4 ms; measurement and QR factors of a D = 300 exact-split
 // step 249 -> 217 ms.
 #include <cuda_runtime.h>
 
@@ -44,7 +48,7 @@ __device__ __forceinline__ void dmma(double* c, double a, double b) {
                : "d"(a), "d"(b));
 }
 
-// K steps (4 deep) of one warp: steps wk, wk + 4, ... counted through all
+// K steps (4 deep) of one warp: steps wk, wk + WK, ... counted through all
 // segments of the tile
 struct KIter {
   const GSeg* segs;
@@ -54,6 +58,7 @@ struct KIter {
   long long ars, brs, aks, bks;   // strides along the tile row / column and K
   int lr, lk, m0, n0;
 
+  template <int WK>
   __device__ __forceinline__ void open() {
     const GSeg sg = segs[si];
     K = sg.K;
@@ -64,14 +69,15 @@ struct KIter {
     bks = sg.tB ? 1 : sg.ldb;
     pa = reinterpret_cast<const double*>(sel_base(*bs, slot_of(sg.A))) + off_of(sg.A) + (m0 + lr) * ars + lk * aks;
     pb = reinterpret_cast<const double*>(sel_base(*bs, slot_of(sg.B))) + off_of(sg.B) + (n0 + lr) * brs + lk * bks;
-    t = (wk - s0) & 3;
+    t = (wk - s0) & (WK - 1);
   }
   // position on this warp's next step; false past the end
+  template <int WK>
   __device__ __forceinline__ bool settle() {
     while (t >= n4) {
       s0 += n4;
       if (++si >= seg1) return false;
-      open();
+      open<WK>();
     }
     return true;
   }
@@ -82,14 +88,16 @@ struct Frag {
   double a[NB], b[NB];
 };
 
-template <int T, int PF>
-__global__ void __launch_bounds__(128) gemm_f64_kernel(const FTile* __restrict__ tiles, const GSeg* __restrict__ segs,
-                                                       Bases bs) {
+template <int T, int PF, int WK>
+__global__ void __launch_bounds__(128) gemm_f64_kernel(const FTile* __restrict__ tiles, int ntiles,
+                                                       const GSeg* __restrict__ segs, Bases bs) {
   constexpr int NB = T / 8;
   constexpr int LD = T + (T > 8 ? 4 : 0);  // staging row (bank spread of the double2 stores)
-  __shared__ __align__(16) double red[4][T * LD];
-  const FTile tl = tiles[blockIdx.x];
+  __shared__ __align__(16) double red[WK == 1 ? 1 : 4][WK == 1 ? 2 : T * LD];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int ti = WK == 1 ? blockIdx.x * 4 + warp : blockIdx.x;
+  if (WK == 1 && ti >= ntiles) return;
+  const FTile tl = tiles[ti];
   const int lr = lane >> 2, lk = lane & 3;
   const int mb = (tl.rows + 7) >> 3, nb = (tl.cols + 7) >> 3;  // 8 x 8 blocks in use (uniform)
   double acc[NB][NB][2];
@@ -105,12 +113,12 @@ __global__ void __launch_bounds__(128) gemm_f64_kernel(const FTile* __restrict__
     it.si = tl.seg0;
     it.seg1 = tl.seg1;
     it.s0 = 0;
-    it.wk = warp;
+    it.wk = WK == 1 ? 0 : warp;
     it.lr = lr;
     it.lk = lk;
     it.m0 = tl.m0;
     it.n0 = tl.n0;
-    it.open();
+    it.open<WK>();
     Frag<NB> f[PF];
     bool ok[PF];
     auto load = [&](Frag<NB>& q) {
@@ -121,11 +129,11 @@ __global__ void __launch_bounds__(128) gemm_f64_kernel(const FTile* __restrict__
       for (int i = 0; i < NB; ++i) q.a[i] = (kin && 8 * i + lr < tl.rows) ? a[8 * i * it.ars] : 0.0;
 #pragma unroll
       for (int j = 0; j < NB; ++j) q.b[j] = (kin && 8 * j + lr < tl.cols) ? b[8 * j * it.brs] : 0.0;
-      it.t += 4;
+      it.t += WK;
     };
 #pragma unroll
     for (int p = 0; p < PF; ++p) {
-      ok[p] = it.si < it.seg1 && it.settle();
+      ok[p] = it.si < it.seg1 && it.settle<WK>();
       if (ok[p]) load(f[p]);
     }
     bool more = ok[0];
@@ -141,10 +149,26 @@ __global__ void __launch_bounds__(128) gemm_f64_kernel(const FTile* __restrict__
 #pragma unroll
           for (int j = 0; j < NB; ++j)
             if (i < mb && j < nb) dmma(acc[i][j], f[p].a[i], f[p].b[j]);
-        ok[p] = it.si < it.seg1 && it.settle();
+        ok[p] = it.si < it.seg1 && it.settle<WK>();
         if (ok[p]) load(f[p]);
       }
     }
+  }
+  double* C = reinterpret_cast<double*>(sel_base(bs, slot_of(tl.C))) + off_of(tl.C);
+  const bool accum = tl.flags & 1;
+  if (WK == 1) {
+#pragma unroll
+    for (int i = 0; i < NB; ++i)
+#pragma unroll
+      for (int j = 0; j < NB; ++j)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int r = 8 * i + lr, c = 8 * j + 2 * lk + h;
+          if (r >= tl.rows || c >= tl.cols) continue;
+          double* p = C + (long long)r * tl.ldc + c;
+          *p = accum ? *p + acc[i][j][h] : acc[i][j][h];
+        }
+    return;
   }
   // the four K shares summed in warp order, rows written along their columns
 #pragma unroll
@@ -154,8 +178,6 @@ __global__ void __launch_bounds__(128) gemm_f64_kernel(const FTile* __restrict__
       *reinterpret_cast<double2*>(&red[warp][(8 * i + lr) * LD + 8 * j + 2 * lk]) =
           make_double2(acc[i][j][0], acc[i][j][1]);
   __syncthreads();
-  double* C = reinterpret_cast<double*>(sel_base(bs, slot_of(tl.C))) + off_of(tl.C);
-  const bool accum = tl.flags & 1;
   for (int e = threadIdx.x; e < T * T; e += 128) {
     const int r = e / T, c = e % T;
     if (r >= tl.rows || c >= tl.cols) continue;
@@ -168,7 +190,7 @@ __global__ void __launch_bounds__(128) gemm_f64_kernel(const FTile* __restrict__
 
 }  // namespace
 
-int f64_tile_size(const GemmPlan& p) {
+F64Shape f64_shape(const GemmPlan& p) {
   // clocks of one SM: 2 multiply-adds each
   double total = 0, kmax = 0;
   for (const GGroup& g : p.groups) {
@@ -178,9 +200,12 @@ int f64_tile_size(const GemmPlan& p) {
     kmax = std::max(kmax, k);
   }
   const double share = total / 152;
+  if (kmax <= 128)
+    for (int T : {16, 8})
+      if (4 * 4 * 0.5 * T * T * kmax <= share) return {T, 1};
   for (int T : {32, 16})
-    if (4 * 0.5 * T * T * kmax <= share) return T;
-  return 8;
+    if (4 * 0.5 * T * T * kmax <= share) return {T, 4};
+  return {8, 4};
 }
 
 std::vector<FTile> f64_tiles(const GemmPlan& p, int T) {
@@ -204,9 +229,12 @@ std::vector<FTile> f64_tiles(const GemmPlan& p, int T) {
 
 cudaError_t launch_gemm_f64(const DevGemm& g, const Bases& b, cudaStream_t s) {
   if (g.ntilesf == 0) return cudaSuccess;
-  if (g.tf == 32) gemm_f64_kernel<32, 1><<<g.ntilesf, 128, 0, s>>>(g.tilesf, g.segs, b);
-  else if (g.tf == 16) gemm_f64_kernel<16, 2><<<g.ntilesf, 128, 0, s>>>(g.tilesf, g.segs, b);
-  else if (g.tf == 8) gemm_f64_kernel<8, 4><<<g.ntilesf, 128, 0, s>>>(g.tilesf, g.segs, b);
+  const int gw = (g.ntilesf + 3) / 4;
+  if (g.tf == 32) gemm_f64_kernel<32, 1, 4><<<g.ntilesf, 128, 0, s>>>(g.tilesf, g.ntilesf, g.segs, b);
+  else if (g.tf == 16 && g.wkf == 1) gemm_f64_kernel<16, 2, 1><<<gw, 128, 0, s>>>(g.tilesf, g.ntilesf, g.segs, b);
+  else if (g.tf == 16) gemm_f64_kernel<16, 2, 4><<<g.ntilesf, 128, 0, s>>>(g.tilesf, g.ntilesf, g.segs, b);
+  else if (g.tf == 8 && g.wkf == 1) gemm_f64_kernel<8, 4, 1><<<gw, 128, 0, s>>>(g.tilesf, g.ntilesf, g.segs, b);
+  else if (g.tf == 8) gemm_f64_kernel<8, 4, 4><<<g.ntilesf, 128, 0, s>>>(g.tilesf, g.ntilesf, g.segs, b);
   else return cudaErrorInvalidValue;
   return cudaGetLastError();
 }

@@ -40,8 +40,8 @@ struct DevGemm {
   GGroup* groups = nullptr;
   GSeg* segs = nullptr;
   GTile* tiles64 = nullptr;   // 64 x 64 output tiles
-  FTile* tilesf = nullptr;    // FP64 kernel: tf x tf output tiles
-  int ngroups = 0, nsegs = 0, ntiles64 = 0, ntilesf = 0, tf = 0;
+  FTile* tilesf = nullptr;    // FP64 kernel: tf x tf output tiles on wkf warps
+  int ngroups = 0, nsegs = 0, ntiles64 = 0, ntilesf = 0, tf = 0, wkf = 0;
   double flops = 0;
 };
 struct DevGather {
@@ -86,8 +86,12 @@ struct RhoScalars {
   int pad;
 };
 
-// FP64 GEMM (tt_gemm64.cu) on the tile list f64_tiles(plan, T), T = f64_tile_size(plan).
-int f64_tile_size(const GemmPlan& p);
+// FP64 GEMM (tt_gemm64.cu) on the tile list f64_tiles(plan, T): T x T tiles, each
+// on wk warps that share its K steps.
+struct F64Shape {
+  int T, wk;
+};
+F64Shape f64_shape(const GemmPlan& p);
 std::vector<FTile> f64_tiles(const GemmPlan& p, int T);
 cudaError_t launch_gemm_f64(const DevGemm& g, const Bases& b, cudaStream_t s);
 // The same in double-float arithmetic on the FP32 pipe (~2^-46 per operation).
