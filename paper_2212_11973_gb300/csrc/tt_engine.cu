@@ -3076,6 +3076,20 @@ tt_status tt_qr_device(tt_ctx* ctx, const double* A, int m, int n, double* Q, do
   DBuf ws, job;
   tt_status st = guarded(ctx, nullptr, [&] {
     const int64_t mn = (int64_t)m * n;
+    auto apart = [](const double* a, int64_t na, const double* b, int64_t nb) { return a + na <= b || b + nb <= a; };
+    if (apart(A, mn, Q, mn) && apart(A, mn, R, (int64_t)n * n) && apart(Q, mn, R, (int64_t)n * n)) {
+      ensure(ctx, ws, qr_grid_scratch(m, n));
+      int *err = nullptr, timed_out = 0;
+      bool done = false;
+      // a budget of its own: the factorisation is accepted under every wait limit of the context
+      CK(launch_qr_grid(A, m, n, Q, R, ws.p, 2000000000ll, ctx->st, &err, &done));
+      if (done) {
+        CK(cudaMemcpyAsync(&timed_out, err, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
+        CK(cudaStreamSynchronize(ctx->st));
+        if (timed_out) throw Err{TT_ERR_TIMEOUT, "tt_qr_device: a wait between the columns' CTAs ran out"};
+        return;
+      }
+    }
     ensure(ctx, ws, (size_t)(2 * mn + (int64_t)n * n) * sizeof(double));
     ensure(ctx, job, sizeof(QrJob));
     QrJob J{0, mn, 2 * mn, m, n};
