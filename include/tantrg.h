@@ -63,8 +63,9 @@ typedef enum {
                                 float sum.  In both modes the Lanczos vectors,
                                 Krylov exponential, SVD, absorb step,
                                 measurements and log-norm stay FP64; the
-                                CholeskyQR gauge runs in double-float (~2^-46)
-                                with a FP64 Householder fallback */
+                                CholeskyQR gauge has its GEMMs in FP64 and its
+                                factorisation in double-float (~2^-46), with a
+                                FP64 Householder fallback */
   TT_PREC_SPLIT_EXACT = 3    /* exact-accumulation split (Ozaki scheme): the
                                 H_eff and bond applies' operands as four
                                 fixed-point BF16 digits with one exponent per
@@ -77,8 +78,8 @@ typedef enum {
                                 have at most 256 states and a gather item at
                                 most 64 MPO terms (TT_ERR_INVALID_ARG
                                 otherwise).  Environment updates per
-                                env_precision; the CholeskyQR gauge in
-                                double-float; Lanczos, Krylov exponential,
+                                env_precision; the CholeskyQR gauge as above;
+                                Lanczos, Krylov exponential,
                                 absorb, measurements and log-norm in FP64 */
 } tt_precision;
 

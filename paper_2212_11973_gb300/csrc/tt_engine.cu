@@ -1128,15 +1128,9 @@ struct Eng {
       return;
     }
     CK(cudaMemsetAsync(q.fail.p, 0, q.h.jobs.size() * sizeof(int), st));
-    // the mixed modes run the Gram and apply GEMMs in double-float on the
-    // FP32 pipe (their error budget is far above ~2^-46), FP64 mode in FP64
-    auto qr_gemm = [&](DevGemmBuf& g) {
-      if (mixed()) CK(launch_gemm_df(g.d, b, st));
-      else f64(g, b);
-    };
     for (int p = 0; p < 3; ++p) {
       long e = prof_begin(11, q.gram[p].d.flops);
-      qr_gemm(q.gram[p]);
+      f64(q.gram[p], b);
       prof_end(e);
       e = prof_begin(12, 0);
       // the mixed modes factorise in double-float (their error budget is far
@@ -1144,7 +1138,7 @@ struct Eng {
       CK(launch_chol_inv((const CholJob*)q.cjobs[p].p, q.ncj[p], dptr(r->ws), (int*)q.fail.p, st, q.maxn[p], mixed()));
       prof_end(e);
       e = prof_begin(11, q.app[p].d.flops);
-      qr_gemm(q.app[p]);
+      f64(q.app[p], b);
       prof_end(e);
       count(3);
     }

@@ -47,7 +47,7 @@ constexpr int FBM = 64, FBN = 64, FBK = 16;
 // TwoProduct with the cross terms, every sum by TwoSum into an unnormalised
 // (hi, lo) accumulator (Dekker; Knuth TAOCP vol. 2, 4.2.2): ~2^-46 relative
 // per operation, K 2^-46 of sum |a| |b| per output.  Output FP64.  Used by the
-// mixed modes' CholeskyQR Gram and apply GEMMs.
+// environment updates with env_precision 2.
 // ---------------------------------------------------------------------------
 // v = hi + lo: hi the top 24 significant bits of v (truncated), lo the other
 // 29 rounded to 24 (error <= 2^-47 |v|), by integer operations on the FP64 bit
@@ -600,7 +600,7 @@ __device__ __forceinline__ double dbl_of_float(float f) {
 
 struct CholDF {
   using T = float2;  // value x + y, |y| <= ulp(x) / 2
-  // unit roundoff of the double-float Gram (gemm_df_kernel) and factor
+  // unit roundoff of the double-float factor (its input rounded to it)
   static constexpr double u = 1.4210854715202004e-14;  // 2^-46
   static __device__ __forceinline__ T of(double v) { return df_split(v); }
   // one FP64 addition (the conversions are integer operations)
