@@ -14,6 +14,7 @@
 #include <cmath>
 #include <cstdint>
 
+#include "tt_df.h"
 #include "tt_kernels.h"
 
 namespace tt {
@@ -49,26 +50,6 @@ constexpr int FBM = 64, FBN = 64, FBK = 16;
 // per operation, K 2^-46 of sum |a| |b| per output.  Output FP64.  Used by the
 // environment updates with env_precision 2.
 // ---------------------------------------------------------------------------
-// v = hi + lo: hi the top 24 significant bits of v (truncated), lo the other
-// 29 rounded to 24 (error <= 2^-47 |v|), by integer operations on the FP64 bit
-// pattern (no FP64 arithmetic); zero for zero and FP64 subnormals, FP64
-// conversions for |v| outside [2^-97, 2^127]
-__device__ __forceinline__ float2 df_split(double v) {
-  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(v));
-  const int e = (int)((b >> 52) & 0x7FF);
-  if (e == 0) return make_float2(0.f, 0.f);
-  if (e < 926 || e > 1150) {
-    const float h = __double2float_rn(v);
-    return make_float2(h, __double2float_rn(v - (double)h));
-  }
-  const unsigned sg = (unsigned)(b >> 32) & 0x80000000u;
-  const float hi = __uint_as_float(sg | ((unsigned)(e - 896) << 23) | (unsigned)((b >> 29) & 0x7FFFFFu));
-  // low 29 mantissa bits times 2^(e - 1075) = (ml 2^-29) 2^(e - 1046), e - 1046 >= -120
-  const float lo = ((float)(unsigned)(b & 0x1FFFFFFFull) * 1.862645149230957e-09f) *
-                   __uint_as_float((unsigned)(e - 1046 + 127) << 23);
-  return make_float2(hi, __uint_as_float(__float_as_uint(lo) | sg));
-}
-
 __global__ void __launch_bounds__(256) gemm_df_kernel(const GGroup* __restrict__ groups, const GSeg* __restrict__ segs,
                                                       const GTile* __restrict__ tiles, Bases bs) {
   __shared__ float2 As[FBK][FBM + 1];
@@ -547,224 +528,6 @@ __device__ __forceinline__ void qr_one(const QrJob J, double* __restrict__ ws) {
   }
 }
 
-// Cholesky G = R^T R (R upper; G the sum of the job's partial Gram matrices,
-// row-major n x n at ws + g) and R^-1, one CTA per job.  Optional diagonal
-// shift s = 11 (m n + n (n + 1)) u tr(G) (shifted CholeskyQR, Fukaya, Kannan,
-// Nakatsukasa, Yamamoto, Yanagisawa 2020).  A non-positive or non-finite pivot
-// marks fail[sec] and leaves the job to the Householder fallback.
-//
-// The upper triangle is packed row by row (row i holds columns i..n-1) in
-// shared memory, or for n > CHOL_SMEM_MAXN in the job's workspace scratch,
-// factorised in place (right-looking: pivot row scaled, then every trailing
-// row updated, a warp per row, lanes along the columns), R written out, then
-// inverted in place, also right-looking: rows k = n-1 .. 0 of R^-1 are
-// finalised in turn (row k divided by R(k, k)) and every row above takes its
-// rank-1 update, R^-1(i, c) -= R(i, k) R^-1(k, c) (back substitution of
-// R X = I, with R(i, k) read just before its slot becomes R^-1(i, k)).  Every
-// step is parallel over a whole trailing block.
-//
-// Element arithmetic: FP64, or double-float (a pair of floats, the error-free
-// TwoSum / FMA TwoProduct transformations of Dekker and Knuth; ~2^-46
-// relative), which runs on the FP32 pipe: GB300 executes ~2 FP64 FMA per clock
-// per SM against 128 FP32, and one CTA factorises one sector.
-constexpr int CHOL_SMEM_MAXN = 230;
-constexpr int CHOL_T = 512;
-
-__device__ __forceinline__ int pk(int i, int j, int n) { return i * n - (i * (i - 1)) / 2 + (j - i); }
-
-struct CholF64 {
-  using T = double;
-  static constexpr double u = 1.1102230246251565e-16;  // unit roundoff 2^-53
-  static __device__ __forceinline__ T of(double x) { return x; }
-  static __device__ __forceinline__ double dbl(T a) { return a; }
-  static __device__ __forceinline__ T zero() { return 0.0; }
-  static __device__ __forceinline__ T add(T a, double v) { return a + v; }
-  // |a - target| (a test against a threshold)
-  static __device__ __forceinline__ double dev(T a, double target) { return fabs(a - target); }
-  // a - b c
-  static __device__ __forceinline__ T fnms(T a, T b, T c) { return fma(-b, c, a); }
-  static __device__ __forceinline__ T mul(T a, T b) { return a * b; }
-};
-
-// FP64 value of a normal float by integer operations (exponent rebias and
-// mantissa shift); zero for zero and float subnormals
-__device__ __forceinline__ double dbl_of_float(float f) {
-  const unsigned u = __float_as_uint(f);
-  const unsigned e = (u >> 23) & 0xFF;
-  if (e == 0) return 0.0;
-  const unsigned long long b = ((unsigned long long)(u & 0x80000000u) << 32) |
-                               ((unsigned long long)(e - 127 + 1023) << 52) |
-                               ((unsigned long long)(u & 0x7FFFFFu) << 29);
-  return __longlong_as_double((long long)b);
-}
-
-struct CholDF {
-  using T = float2;  // value x + y, |y| <= ulp(x) / 2
-  // unit roundoff of the double-float factor (its input rounded to it)
-  static constexpr double u = 1.4210854715202004e-14;  // 2^-46
-  static __device__ __forceinline__ T of(double v) { return df_split(v); }
-  // one FP64 addition (the conversions are integer operations)
-  static __device__ __forceinline__ double dbl(T a) { return dbl_of_float(a.x) + dbl_of_float(a.y); }
-  static __device__ __forceinline__ T zero() { return make_float2(0.f, 0.f); }
-  static __device__ __forceinline__ T two_sum(float s, float t) {
-    const float h = s + t;
-    const float bp = h - s;
-    return make_float2(h, (s - (h - bp)) + (t - bp));
-  }
-  static __device__ __forceinline__ T add(T a, double v) {
-    const float2 b = df_split(v);
-    const float s = a.x + b.x;
-    const float bp = s - a.x;
-    const float t = ((a.x - (s - bp)) + (b.x - bp)) + (a.y + b.y);
-    return two_sum(s, t);
-  }
-  static __device__ __forceinline__ double dev(T a, double target) {
-    return (double)fabsf((a.x - (float)target) + a.y);
-  }
-  static __device__ __forceinline__ T fnms(T a, T b, T c) {
-    const float p = b.x * c.x;
-    float e = fmaf(b.x, c.x, -p);  // b.x c.x = p + e exactly
-    e = fmaf(b.x, c.y, e);
-    e = fmaf(b.y, c.x, e);
-    const float s = a.x - p;       // a.x - p = s + t exactly
-    const float bp = s - a.x;
-    float t = (a.x - (s - bp)) + (-p - bp);
-    t += a.y - e;
-    return two_sum(s, t);
-  }
-  static __device__ __forceinline__ T mul(T a, T b) {
-    const float p = a.x * b.x;
-    float e = fmaf(a.x, b.x, -p);
-    e = fmaf(a.x, b.y, e);
-    e = fmaf(a.y, b.x, e);
-    return two_sum(p, e);
-  }
-};
-
-template <class A>
-__global__ void __launch_bounds__(CHOL_T, 1) chol_inv_smem_kernel(const CholJob* __restrict__ jobs, double* __restrict__ ws,
-                                                               int* __restrict__ fail) {
-  using T = typename A::T;
-  extern __shared__ __align__(16) unsigned char chol_raw[];
-  const CholJob J = jobs[blockIdx.x];
-  const int n = J.n;
-  // the packed triangle: shared memory, or the job's workspace scratch (L2
-  // resident) for the sectors too large for it
-  T* sm = n <= CHOL_SMEM_MAXN ? reinterpret_cast<T*>(chol_raw) : reinterpret_cast<T*>(ws + J.pk);
-  if (J.shift == 3) {
-    if (threadIdx.x == 0) fail[J.sec] = 1;
-    return;
-  }
-  if (fail[J.sec]) return;
-  double* G = ws + J.g;
-  double* R = ws + J.r;
-  double* Ri = ws + J.ri;
-  const long long nn = (long long)n * n;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = blockDim.x >> 5;
-  __shared__ double red[CHOL_T / 32];
-  __shared__ T piv_t, ipiv_t;  // the current pivot and its reciprocal
-  __shared__ int bad;
-  // G = sum of the partial Gram matrices, upper triangle into shared memory
-  for (int i = warp; i < n; i += nw)
-    for (int j = i + lane; j < n; j += 32) {
-      const long long e = (long long)i * n + j;
-      T acc = A::of(G[e]);
-      for (int s = 1; s < J.parts; ++s) acc = A::add(acc, G[s * nn + e]);
-      sm[pk(i, j, n)] = acc;
-    }
-  __syncthreads();
-  if (J.shift == 2) {
-    // last pass: G = I + E; first-order factor when n max|E| <= 1e-8, else a
-    // full factorisation; far from I (> 1e-3): Householder fallback
-    double mx = 0.0;
-    for (int i = warp; i < n; i += nw)
-      for (int j = i + lane; j < n; j += 32) {
-        const double dev = A::dev(sm[pk(i, j, n)], i == j ? 1.0 : 0.0);
-        mx = (dev <= mx) ? mx : (dev == dev ? dev : 1e300);
-      }
-    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if (lane == 0) red[warp] = mx;
-    __syncthreads();
-    double all = 0.0;
-    for (int q = 0; q < nw; ++q) all = fmax(all, red[q]);
-    if (!(all <= 1e-3)) {
-      if (tid == 0) fail[J.sec] = 1;
-      return;
-    }
-    if ((double)n * all <= 1e-8) {
-      for (int i = warp; i < n; i += nw)
-        for (int j = lane; j < n; j += 32) {
-          const long long e = (long long)i * n + j;
-          if (j < i) {
-            R[e] = 0.0;
-            Ri[e] = 0.0;
-          } else if (j == i) {
-            const double h = 0.5 * (A::dbl(sm[pk(i, i, n)]) - 1.0);
-            R[e] = 1.0 + h;
-            Ri[e] = 1.0 - h;
-          } else {
-            const double g = A::dbl(sm[pk(i, j, n)]);
-            R[e] = g;
-            Ri[e] = -g;
-          }
-        }
-      return;
-    }
-  }
-  if (tid == 0) {
-    bad = 0;
-    if (J.shift == 1) {
-      // shift s = 11 (m n + n (n + 1)) u ||X||^2 with ||X||^2 <= tr(G), u the
-      // unit roundoff of the arithmetic that formed G and factorises it
-      double tr = 0.0;
-      for (int i = 0; i < n; ++i) tr += A::dbl(sm[pk(i, i, n)]);
-      const double sft = 11.0 * ((double)J.m * n + (double)n * (n + 1)) * A::u * tr;
-      for (int i = 0; i < n; ++i) sm[pk(i, i, n)] = A::of(A::dbl(sm[pk(i, i, n)]) + sft);
-    }
-  }
-  __syncthreads();
-  for (int k = 0; k < n; ++k) {
-    if (tid == 0) {
-      const double d = A::dbl(sm[pk(k, k, n)]);
-      if (!(d > 0.0) || !isfinite(d)) {
-        bad = 1;
-        fail[J.sec] = 1;
-      }
-      const double p = bad ? 1.0 : sqrt(d);
-      piv_t = A::of(p);
-      ipiv_t = A::of(1.0 / p);
-    }
-    __syncthreads();
-    if (bad) return;
-    for (int j = k + tid; j < n; j += blockDim.x) sm[pk(k, j, n)] = j == k ? piv_t : A::mul(sm[pk(k, j, n)], ipiv_t);
-    __syncthreads();
-    for (int i = k + 1 + warp; i < n; i += nw) {
-      const T rki = sm[pk(k, i, n)];
-      for (int j = i + lane; j < n; j += 32) sm[pk(i, j, n)] = A::fnms(sm[pk(i, j, n)], rki, sm[pk(k, j, n)]);
-    }
-    __syncthreads();
-  }
-  for (int i = warp; i < n; i += nw)
-    for (int j = lane; j < n; j += 32) R[(long long)i * n + j] = (j >= i) ? A::dbl(sm[pk(i, j, n)]) : 0.0;
-  // in-place inverse, rows from the bottom
-  for (int k = n - 1; k >= 0; --k) {
-    __syncthreads();
-    if (tid == 0) ipiv_t = A::of(1.0 / A::dbl(sm[pk(k, k, n)]));
-    __syncthreads();
-    for (int c = k + tid; c < n; c += blockDim.x) sm[pk(k, c, n)] = c == k ? ipiv_t : A::mul(sm[pk(k, c, n)], ipiv_t);
-    __syncthreads();
-    for (int i = warp; i < k; i += nw) {
-      const T rik = sm[pk(i, k, n)];
-      __syncwarp();
-      for (int c = k + lane; c < n; c += 32)
-        sm[pk(i, c, n)] = A::fnms(c == k ? A::zero() : sm[pk(i, c, n)], rik, sm[pk(k, c, n)]);
-    }
-  }
-  __syncthreads();
-  for (int i = warp; i < n; i += nw)
-    for (int j = lane; j < n; j += 32) Ri[(long long)i * n + j] = (j >= i) ? A::dbl(sm[pk(i, j, n)]) : 0.0;
-}
-
 __global__ void dot_finalize(const double* partial, int nblk, double* out) {
   __shared__ double s;
   finalize_sums(partial, nblk, 1, &s);
@@ -927,23 +690,6 @@ cudaError_t launch_qr_job(const QrJob& job, double* ws, cudaStream_t s) {
 cudaError_t launch_qr_masked(const QrJob* jobs, int njobs, double* ws, const int* only, int* nrun, cudaStream_t s) {
   if (njobs == 0) return cudaSuccess;
   qr_kernel<<<njobs, QRT, 0, s>>>(jobs, ws, only, nrun);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_chol_inv(const CholJob* jobs, int njobs, double* ws, int* fail, cudaStream_t s, int maxn, bool df) {
-  if (njobs == 0) return cudaSuccess;
-  const int ns = maxn < CHOL_SMEM_MAXN ? maxn : CHOL_SMEM_MAXN;
-  const size_t smem = ((size_t)ns * (ns + 1) / 2) * 8;
-  const int smax = (int)(((size_t)CHOL_SMEM_MAXN * (CHOL_SMEM_MAXN + 1) / 2) * 8);
-  // once per process (thread-safe static initialisation): the largest size
-  static const cudaError_t e1 =
-      cudaFuncSetAttribute(chol_inv_smem_kernel<CholF64>, cudaFuncAttributeMaxDynamicSharedMemorySize, smax);
-  static const cudaError_t e2 =
-      cudaFuncSetAttribute(chol_inv_smem_kernel<CholDF>, cudaFuncAttributeMaxDynamicSharedMemorySize, smax);
-  if (e1 != cudaSuccess) return e1;
-  if (e2 != cudaSuccess) return e2;
-  if (df) chol_inv_smem_kernel<CholDF><<<njobs, CHOL_T, smem, s>>>(jobs, ws, fail);
-  else chol_inv_smem_kernel<CholF64><<<njobs, CHOL_T, smem, s>>>(jobs, ws, fail);
   return cudaGetLastError();
 }
 
