@@ -625,6 +625,15 @@ struct Eng {
     else CK(cudaEventRecord(e, st));
   }
 
+  // K extent of the tensor maps' boxes: 64, or 32 for the digit kernel where no
+  // segment is longer than 64
+  int tc_box(const DevGemmBuf& g) const {
+    if (!r->exact) return 64;
+    for (const GSeg& sg : g.host.segs)
+      if (sg.K > 64) return 64;
+    return 32;
+  }
+
   // tcgen05 eligibility (K-major A and B, 16-byte aligned rows and offsets) and
   // the per-segment tensor maps for the current slot bases.
   bool prep_tc(DevGemmBuf& g, const Bases& b) {
@@ -682,6 +691,7 @@ struct Eng {
       g.tc_ok = false;
       return false;
     }
+    const int kbox = tc_box(g);
     const size_t nseg = g.host.segs.size();
     std::vector<CUtensorMap> maps(3 * nseg);
     std::vector<int> seg_group(nseg, 0);
@@ -698,11 +708,12 @@ struct Eng {
         if (!b.p[sl] || lo % 8 || sg.K < 1) { g.tc_ok = false; return false; }
         cuuint64_t dims[3] = {(cuuint64_t)sg.K, (cuuint64_t)std::max(1, w == 0 ? gg.M : gg.N), (cuuint64_t)r->nsplit};
         cuuint64_t strides[2] = {(cuuint64_t)(w == 0 ? sg.lda : sg.ldb) * 2, (cuuint64_t)lo * 2};
-        cuuint32_t box[3] = {64, (cuuint32_t)(w == 2 ? 64 : 128), 1};
+        cuuint32_t box[3] = {(cuuint32_t)kbox, (cuuint32_t)(w == 2 ? 64 : 128), 1};
         cuuint32_t estr[3] = {1, 1, 1};
         void* base = (char*)b.p[sl] + off * 2;
         CUresult cr = encode(&maps[3 * si + w], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, base, dims, strides, box, estr,
-                             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                             CU_TENSOR_MAP_INTERLEAVE_NONE,
+                             kbox == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
                              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (cr != CUDA_SUCCESS) {
           if (std::getenv("TT_DEBUG"))
@@ -810,6 +821,23 @@ struct Eng {
     return best;
   }
 
+  // CTAs that share a tile of the persistent digit kernel, with room for their
+  // partial sums (allocated in the uncaptured step, like every buffer)
+  int split_tiles(const DevGemmBuf& g) {
+    int ms = 0;
+    for (const GGroup& gg : g.host.groups) ms = std::max(ms, gg.seg1 - gg.seg0);
+    const int split = tcz_split(g.ntilesp, ms);
+    if (split == 1) return 1;
+    const size_t sb = tcz_scratch_bytes(g.ntilesp, split), tb = tcz_tickets(g.ntilesp) * sizeof(unsigned);
+    if (r->zscr.bytes < sb || r->ztick.bytes < tb) {
+      if (r->capturing) throw Err{TT_ERR_STATE, "split scratch missing during graph capture"};
+      ensure(c, r->zscr, sb);
+      ensure(c, r->ztick, tb);
+      CK(cudaMemsetAsync(r->ztick.p, 0, r->ztick.bytes, st));
+    }
+    return split;
+  }
+
   void gemm(DevGemmBuf& g, const Bases& b, bool use_mixed, int kind = 4) {
     if (use_mixed && r->exact) {
       if (!r->use_tc || !prep_tc(g, b))
@@ -826,8 +854,9 @@ struct Eng {
       for (const GGroup& gg : g.host.groups)
         if (((gg.flags & 2) != 0) != pair) throw Err{TT_ERR_STATE, "exact split: mixed output forms in one GEMM plan"};
       const long e = prof_begin(kind, g.d.flops);
-      CK(launch_gemm_tcz(g.d.groups, g.d.segs, (const GTile*)g.tilesp.p, g.ntilesp, g.maps.p, b, (int*)r->tcerr.p,
-                         c->wait_ns, pair, st));
+      const int split = split_tiles(g);
+      CK(launch_gemm_tcz(g.d.groups, g.d.segs, (const GTile*)g.tilesp.p, g.ntilesp, split, tc_box(g), g.maps.p, b, r->zscr.p,
+                         (unsigned*)r->ztick.p, (int*)r->tcerr.p, c->wait_ns, pair, st));
       prof_end(e);
       count();
       return;
@@ -2361,7 +2390,7 @@ void free_rho(tt_rho* r) {
   for (auto& g : r->absl) release(c, g);
   for (auto& g : r->absr) release(c, g);
   for (auto& m : r->meas) { release(c, m.t); release(c, m.el); dfree(c, m.items); }
-  for (DBuf* b : {&r->Qk, &r->W, &r->Xs, &r->Xn, &r->T1, &r->T2, &r->Sb, &r->ws, &r->partial, &r->ks, &r->rs, &r->tmp, &r->obs, &r->el0, &r->el1, &r->tcerr, &r->qrfb})
+  for (DBuf* b : {&r->Qk, &r->W, &r->Xs, &r->Xn, &r->T1, &r->T2, &r->Sb, &r->ws, &r->partial, &r->ks, &r->rs, &r->tmp, &r->obs, &r->el0, &r->el1, &r->tcerr, &r->qrfb, &r->zscr, &r->ztick})
     dfree(c, *b);
 }
 

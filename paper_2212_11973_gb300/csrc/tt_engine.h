@@ -170,7 +170,7 @@ struct tt_rho {
   std::vector<tt::DevGemmBuf> absl, absr;
   std::vector<char> absl_ok, absr_ok;
   std::vector<tt::MeasDev> meas;
-  tt::DBuf Qk, W, Xs, Xn, T1, T2, Sb, ws, partial, ks, rs, tmp, obs, el0, el1, tcerr, qrfb;
+  tt::DBuf Qk, W, Xs, Xn, T1, T2, Sb, ws, partial, ks, rs, tmp, obs, el0, el1, tcerr, qrfb, zscr, ztick;
   int64_t ldq = 0;
   tt_stats stats{};
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;

@@ -120,12 +120,20 @@ cudaError_t launch_gemm_tcp(const GGroup* groups, const GSeg* segs, const GTile*
                             const void* maps, const Bases& b, int nsplit, int* err, long long wait_ns, cudaStream_t s);
 // Exact-accumulation split GEMM on tcgen05 (tt_tcgen05z.cu): digit operands
 // (4 levels + int16 row exponents, GSeg.eA / eB), persistent 128 x 64 tiles,
-// the same maps; segments of K <= tcz_max_k(); output FP64 or two-float pairs
+// maps with boxes of kbox = 64 (128-byte swizzle) or 32 (64-byte) K;
+// segments of K <= tcz_max_k(); output FP64 or two-float pairs
 // (flags bit 1, the same in every group of a launch: pair).
 int tcz_max_k();
 size_t tcz_smem_bytes();
-cudaError_t launch_gemm_tcz(const GGroup* groups, const GSeg* segs, const GTile* tiles128x64, int ntiles,
-                            const void* maps, const Bases& b, int* err, long long wait_ns, bool pair, cudaStream_t s);
+// split CTAs share the segments of a tile (tcz_split: where the tiles leave SMs
+// idle); they need scratch of tcz_scratch_bytes and tcz_tickets zeroed counters
+// (left at zero).
+int tcz_split(int ntiles, int max_segs);
+size_t tcz_scratch_bytes(int ntiles, int split);
+size_t tcz_tickets(int ntiles);
+cudaError_t launch_gemm_tcz(const GGroup* groups, const GSeg* segs, const GTile* tiles128x64, int ntiles, int split,
+                            int kbox, const void* maps, const Bases& b, void* scratch, unsigned* tickets, int* err,
+                            long long wait_ns, bool pair, cudaStream_t s);
 // Digit producers (tt_digits.cu): FP64 rows -> digit rows; the W-gather of
 // the exact path (two-float S1 outputs -> digit rows of T2, rows up to
 // gather_digits_max_cols() long, at most gather_digits_max_contribs() MPO

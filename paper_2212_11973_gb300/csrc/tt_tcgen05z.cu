@@ -15,16 +15,29 @@
 // rounding that grows with K.
 //
 // Structure as gemm_tcp_kernel (tt_tcgen05p.cu): persistent, one CTA per SM,
-// 128 x 64 output tiles; warp 0 streams the digit tiles (A 4 x 16 KB, B 4 x
-// 8 KB per 64-wide K chunk) into two shared-memory stages, warp 1 issues the
-// MMAs of a segment into one of two TMEM buffers (4 accumulators x 64
-// columns each), warps 2-9 fold a finished buffer while the next segment's
-// MMAs run in the other (two warps per TMEM lane quarter, 32 columns each,
-// so that every SM sub-partition has two folding warps), and write each
-// finished tile as FP64 or as a two-float pair (flags bit 1) through a
-// per-warp, XOR-swizzled shared-memory staging buffer (coalesced 128-byte
-// row stores, no cross-warp barrier).  Waits are bounded as in the other
-// tcgen05 kernels.
+// 128 x 64 output tiles; warp 0 streams the digit tiles into a ring of two
+// shared-memory stages of 64 K (A 4 x 16 KB, B 4 x 8 KB) or four of 32, warp 1 issues the MMAs of
+// a segment into one of two TMEM buffers (4 accumulators x 64 columns each),
+// warps 2-9 fold a finished buffer while the next segment's MMAs run in the
+// other (two warps per TMEM lane quarter, 32 columns each, so that every SM
+// sub-partition has two folding warps), and write each finished tile as FP64
+// or as a two-float pair (flags bit 1) through a per-warp, XOR-swizzled
+// shared-memory staging buffer (coalesced 128-byte row stores, no cross-warp
+// barrier).  Waits are bounded as in the other tcgen05 kernels.
+//
+// What bounds it: the chain of 18 to 42 short segments (K = 3 to 180) behind
+// each output tile at small D, shared-memory and L2 bandwidth of the operands at
+// D = 1024; never the tensor pipe.  So (1) 16-wide K steps past a segment's end
+// are skipped, and plans whose segments are at most 64 long (D up to ~350) use
+// chunks of 32, four in flight (D = 300: 40 -> 24 us a launch; D = 1024, whose
+// longer segments feed fine from two stages of 64, was 15 % slower with them);
+// (2) a segment's tensor maps are
+// fenced and its K and exponent references read by the lanes of a warp, 32
+// segments at a time, and the row exponents of the next segment are loaded
+// before the wait for the current one; (3) where a plan has fewer tiles than
+// SMs, `split` CTAs share a tile's segments: each writes its two-float sums to
+// scratch and the last to arrive (a ticket per tile and folding warp, no CTA
+// waits for another) adds them in part order.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -40,16 +53,14 @@ namespace {
 
 using namespace tcx;
 
-constexpr int ZBM = 128, ZBN = 64, ZBK = 64, ZDIG = 4, ZPAIRS = 10;
-constexpr int ZA_BYTES = ZBM * ZBK * 2;  // 16 KB per digit level
-constexpr int ZB_BYTES = ZBN * ZBK * 2;  // 8 KB per digit level
-constexpr int ZSTAGE_BYTES = ZDIG * (ZA_BYTES + ZB_BYTES);
-constexpr int ZSTAGES = 2;
+constexpr int ZBM = 128, ZBN = 64, ZDIG = 4;
+constexpr int ZMAXSTAGES = 4;
+constexpr int ZRING_BYTES = 2 * ZDIG * (ZBM + ZBN) * 64 * 2;  // 192 KB of operand stages
 constexpr uint32_t ZTMEM_COLS = 512;
 constexpr int ZEPI = 8;  // epilogue warps
 constexpr int ZTHREADS = 64 + 32 * ZEPI;
 constexpr int ZMAXK = 256;  // longest segment whose digit sums stay exact
-// epilogue staging, after the two TMA stages: per epilogue warp 32 rows x 16
+// epilogue staging, after the TMA stages: per epilogue warp 32 rows x 16
 // columns of 8-byte outputs, column c of row r at word r * 16 + (c ^ (r & 15))
 constexpr int ZSTG_WARP = 32 * 16;
 constexpr int ZSTG_BYTES = ZEPI * ZSTG_WARP * 8;
@@ -107,23 +118,51 @@ __device__ __forceinline__ void two_sum_z(float& hi, float& lo, float x) {
   hi = s;
 }
 
-// digit pair p -> (s, t): d = s + t ascending, the first pair of each d at
-// p = 0, 1, 3, 6
-__device__ __forceinline__ void pair_of(int p, int& s, int& t) {
-  const int d = (p >= 1) + (p >= 3) + (p >= 6);
-  s = p - d * (d + 1) / 2;
-  t = d - s;
+// UMMA shared-memory descriptor, K-major, rows of BK elements in one swizzle
+// span (64: 128 bytes, 32: 64 bytes), 8-row groups contiguous
+template <int BK>
+__device__ __forceinline__ uint64_t desc_of(uint32_t saddr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr >> 4) & 0x3FFF);
+  d |= (uint64_t)1 << 16;                    // leading byte offset (unused for swizzled K-major)
+  d |= (uint64_t)((8 * BK * 2) >> 4) << 32;  // stride byte offset
+  d |= (uint64_t)1 << 46;                    // descriptor version
+  d |= (uint64_t)(BK == 64 ? 2 : 4) << 61;   // SWIZZLE_128B / SWIZZLE_64B
+  return d;
+}
+
+// one part of a tile: segments seg0 + part, + split, ... (n of them)
+struct ZItem {
+  GTile tl;
+  GGroup g;
+  int part, parts, n;
+};
+__device__ __forceinline__ ZItem item_of(const GGroup* groups, const GTile* tiles, int w, int split) {
+  ZItem it;
+  it.tl = tiles[w / split];
+  it.g = groups[it.tl.g];
+  const int nseg = it.g.seg1 - it.g.seg0;
+  it.part = w % split;
+  it.parts = max(1, min(split, nseg));
+  it.n = it.part < it.parts ? (nseg - it.part + it.parts - 1) / it.parts : 0;
+  return it;
 }
 
 // PAIR: every group of the launch writes two-float pairs (flags bit 1), else
 // FP64 (accumulating with flags bit 0); one kernel per output form keeps the
 // FP64 conversions out of the pair kernel entirely
-template <bool PAIR>
+template <bool PAIR, int ZBK>
 __global__ void __launch_bounds__(ZTHREADS, 1) gemm_tcz_kernel(const GGroup* __restrict__ groups,
                                                                const GSeg* __restrict__ segs,
-                                                               const GTile* __restrict__ tiles, int ntiles,
+                                                               const GTile* __restrict__ tiles, int nitems, int split,
                                                                const CUtensorMap* __restrict__ maps, Bases bs,
-                                                               int* __restrict__ err, long long wait_ns) {
+                                                               uint64_t* __restrict__ scratch,
+                                                               unsigned* __restrict__ tickets, int* __restrict__ err,
+                                                               long long wait_ns) {
+  constexpr int ZA_BYTES = ZBM * ZBK * 2, ZB_BYTES = ZBN * ZBK * 2;  // per digit level
+  constexpr int ZSTAGE_BYTES = ZDIG * (ZA_BYTES + ZB_BYTES);
+  constexpr int ZSTAGES = ZRING_BYTES / ZSTAGE_BYTES;
+  static_assert(ZSTAGES <= ZMAXSTAGES && ZSTAGES * ZSTAGE_BYTES == ZRING_BYTES, "operand ring");
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[ZSTAGES], empty_bar[ZSTAGES], accf[2], acce[2];
   __shared__ uint32_t tmem_base_s;
@@ -161,84 +200,94 @@ __global__ void __launch_bounds__(ZTHREADS, 1) gemm_tcz_kernel(const GGroup* __r
 
   if (warp == 0) {
     // ---------------- producer ----------------
-    if (lane == 0) {
-      int it = 0, fenced = -1;
-      for (int t = blockIdx.x; t < ntiles && !*abort_f; t += gridDim.x) {
-        const GTile tl = tiles[t];
-        const GGroup g = groups[tl.g];
-        for (int si = g.seg0; si < g.seg1 && !*abort_f; ++si) {
-          const int K = segs[si].K;
-          const CUtensorMap* ma = maps + 3 * si;
-          const CUtensorMap* mb = maps + 3 * si + 2;
-          if (fenced != si) {
-            asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(reinterpret_cast<uint64_t>(ma))
-                         : "memory");
-            asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(reinterpret_cast<uint64_t>(mb))
-                         : "memory");
-            fenced = si;
-          }
-          for (int k0 = 0; k0 < K; k0 += ZBK) {
-            const int s = it % ZSTAGES;
-            if (!wait_z(&empty_bar[s], ((it / ZSTAGES) & 1) ^ 1, wait_ns, abort_f, err)) break;
-            uint8_t* st = smem + s * ZSTAGE_BYTES;
-            mbar_expect_tx(&full_bar[s], ZSTAGE_BYTES);
-#pragma unroll
-            for (int l = 0; l < ZDIG; ++l) tma_load_3d(st + l * ZA_BYTES, ma, k0, tl.m0, l, &full_bar[s]);
-#pragma unroll
-            for (int l = 0; l < ZDIG; ++l)
-              tma_load_3d(st + ZDIG * ZA_BYTES + l * ZB_BYTES, mb, k0, tl.n0, l, &full_bar[s]);
-            ++it;
-            issued_s = it;
-          }
+    int it = 0, fenced = -1;  // group whose first 32 segments' maps this CTA has fenced
+    for (int w = blockIdx.x; w < nitems && !*abort_f; w += gridDim.x) {
+      const ZItem q = item_of(groups, tiles, w, split);
+      for (int s0 = 0; s0 < q.n; s0 += 32) {
+        const int sl = q.g.seg0 + q.part + min(s0 + lane, q.n - 1) * q.parts;
+        const int kl = segs[sl].K;
+        if (fenced != q.tl.g || q.n > 32) {
+          const uint64_t ma = reinterpret_cast<uint64_t>(maps + 3 * sl), mb = ma + 2 * sizeof(CUtensorMap);
+          asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(ma) : "memory");
+          asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(mb) : "memory");
+          asm volatile("prefetch.tensormap [%0];" ::"l"(ma) : "memory");
+          asm volatile("prefetch.tensormap [%0];" ::"l"(mb) : "memory");
+          fenced = q.parts == 1 ? q.tl.g : -1;
+          __syncwarp();
         }
+        for (int s = s0; s < min(q.n, s0 + 32); ++s) {
+          const int K = __shfl_sync(0xffffffffu, kl, s - s0);
+          if (lane == 0) {
+            const int si = q.g.seg0 + q.part + s * q.parts;
+            const CUtensorMap* ma = maps + 3 * si;
+            const CUtensorMap* mb = ma + 2;
+            for (int k0 = 0; k0 < K; k0 += ZBK) {
+              const int sg = it % ZSTAGES;
+              if (!wait_z(&empty_bar[sg], ((it / ZSTAGES) & 1) ^ 1, wait_ns, abort_f, err)) break;
+              uint8_t* st = smem + sg * ZSTAGE_BYTES;
+              mbar_expect_tx(&full_bar[sg], ZSTAGE_BYTES);
+#pragma unroll
+              for (int l = 0; l < ZDIG; ++l) tma_load_3d(st + l * ZA_BYTES, ma, k0, q.tl.m0, l, &full_bar[sg]);
+#pragma unroll
+              for (int l = 0; l < ZDIG; ++l)
+                tma_load_3d(st + ZDIG * ZA_BYTES + l * ZB_BYTES, mb, k0, q.tl.n0, l, &full_bar[sg]);
+              ++it;
+              issued_s = it;
+            }
+          }
+          __syncwarp();
+          if (*abort_f) break;
+        }
+        if (*abort_f) break;
       }
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer: one fold unit per segment ----------------
-    if (lane == 0) {
-      const uint32_t idesc =
-          (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(ZBN >> 3) << 17) | ((uint32_t)(ZBM >> 4) << 24);
-      int it = 0, fg = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-        const GTile tl = tiles[t];
-        const GGroup g = groups[tl.g];
-        for (int si = g.seg0; si < g.seg1 && ok; ++si) {
-          const int nch = (segs[si].K + ZBK - 1) / ZBK;
+    // A digit s times the B digits 0 .. 3 - s in one instruction: the B levels lie
+    // one after the other, 64 rows each, so they are an operand of N = 64 (4 - s)
+    // rows, and its products belong to D_s .. D_3, 64 TMEM columns each.  Four
+    // instructions per 16 K instead of ten, and A is read 4 times, not 10
+    // (operands from shared memory, 128 bytes per clock, bound the MMAs here)
+    constexpr uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(ZBM >> 4) << 24);
+    int it = 0, fg = 0;
+    bool ok = true;
+    for (int w = blockIdx.x; w < nitems && ok; w += gridDim.x) {
+      const ZItem q = item_of(groups, tiles, w, split);
+      int kl = 0;
+      for (int s = 0; s < q.n && ok; ++s) {
+        if ((s & 31) == 0) kl = segs[q.g.seg0 + q.part + min(s + lane, q.n - 1) * q.parts].K;
+        const int K = __shfl_sync(0xffffffffu, kl, s & 31);
+        if (lane == 0) {
           const int b = fg & 1;
           ok = wait_z(&acce[b], ((fg >> 1) & 1) ^ 1, wait_ns, abort_f, err);
-          if (!ok) break;
           fence_after();
           const uint32_t tb = tmem + 256 * b;
-          for (int c = 0; c < nch; ++c) {
-            const int s = it % ZSTAGES;
-            ok = wait_z(&full_bar[s], (it / ZSTAGES) & 1, wait_ns, abort_f, err);
+          for (int k0 = 0; k0 < K && ok; k0 += ZBK) {
+            const int sg = it % ZSTAGES;
+            ok = wait_z(&full_bar[sg], (it / ZSTAGES) & 1, wait_ns, abort_f, err);
             if (!ok) break;
             consumed_s = it + 1;
             fence_after();
-            const uint32_t sa = smem_u32(smem + s * ZSTAGE_BYTES);
+            const uint32_t sa = smem_u32(smem + sg * ZSTAGE_BYTES);
+            const int nk = (min(ZBK, K - k0) + 15) >> 4;  // 16-wide steps with data
+            for (int kk = 0; kk < nk; ++kk) {
+              const uint64_t bd = desc_of<ZBK>(sa + ZDIG * ZA_BYTES + kk * 32);
 #pragma unroll
-            for (int p = 0; p < ZPAIRS; ++p) {
-              int ls, lt;
-              pair_of(p, ls, lt);
-              const bool first = (p == 0 || p == 1 || p == 3 || p == 6);
-              const uint32_t aa = sa + ls * ZA_BYTES, ba = sa + ZDIG * ZA_BYTES + lt * ZB_BYTES;
-              const uint32_t dst = tb + 64 * (ls + lt);
-#pragma unroll
-              for (int kk = 0; kk < ZBK / 16; ++kk) {
-                const uint32_t acc = (c > 0 || kk > 0 || !first) ? 1u : 0u;
-                umma_f16(dst, make_desc(aa + kk * 32), make_desc(ba + kk * 32), idesc, acc);
-              }
+              for (int s = 0; s < ZDIG; ++s)
+                umma_f16(tb + 64 * s, desc_of<ZBK>(sa + s * ZA_BYTES + kk * 32), bd,
+                         idesc0 | ((uint32_t)((ZBN * (ZDIG - s)) >> 3) << 17), (k0 > 0 || kk > 0 || s > 0) ? 1u : 0u);
             }
-            umma_commit(&empty_bar[s]);
+            umma_commit(&empty_bar[sg]);
             last_commit_s = it;
             ++it;
           }
-          if (!ok) break;
-          umma_commit(&accf[b]);
-          last_accf_s = fg;
-          ++fg;
+          if (ok) {
+            umma_commit(&accf[b]);
+            last_accf_s = fg;
+            ++fg;
+          }
         }
+        ok = __shfl_sync(0xffffffffu, ok, 0);
       }
     }
   } else {
@@ -247,19 +296,50 @@ __global__ void __launch_bounds__(ZTHREADS, 1) gemm_tcz_kernel(const GGroup* __r
     // partition may access) and folds columns 32 h .. 32 h + 31 of them
     const int q = warp & 3, h = (warp - 2) >> 2;
     const uint32_t lane_off = (uint32_t)(32 * q) << 16;
-    uint64_t* stg = reinterpret_cast<uint64_t*>(smem + ZSTAGES * ZSTAGE_BYTES) + (warp - 2) * ZSTG_WARP;
+    uint64_t* stg = reinterpret_cast<uint64_t*>(smem + ZRING_BYTES) + (warp - 2) * ZSTG_WARP;
     int fg = 0;
     bool ok = true;
     float hi[32], lo[32];
-    for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-      const GTile tl = tiles[t];
-      const GGroup g = groups[tl.g];
+    for (int w = blockIdx.x; w < nitems && ok; w += gridDim.x) {
+      const ZItem z = item_of(groups, tiles, w, split);
+      const GTile tl = z.tl;
+      const GGroup& g = z.g;
+      if (z.part >= z.parts) continue;
       const int row = tl.m0 + 32 * q + lane;
       const int col_l = tl.n0 + 32 * h + lane;  // the column whose exponent this lane loads
 #pragma unroll
       for (int i = 0; i < 32; ++i) { hi[i] = 0.f; lo[i] = 0.f; }
-      for (int si = g.seg0; si < g.seg1; ++si) {
-        const GSeg sg = segs[si];
+      // exponent references of 32 segments, one per lane; the exponents of the
+      // segment after the current one are in flight while it is waited for
+      unsigned long long ral = 0, rbl = 0;
+      int sal = 0, sbl = 0;
+      auto refs = [&](int s) {
+        const GSeg* sp = segs + g.seg0 + z.part + min(s + lane, z.n - 1) * z.parts;
+        ral = sp->eA;
+        rbl = sp->eB;
+        sal = sp->eas;
+        sbl = sp->ebs;
+      };
+      auto exps = [&](int s, int& ea, int& eb) {
+        const int l = s & 31;
+        const Ref ra = __shfl_sync(0xffffffffu, ral, l), rb = __shfl_sync(0xffffffffu, rbl, l);
+        const int sa = __shfl_sync(0xffffffffu, sal, l), sb = __shfl_sync(0xffffffffu, sbl, l);
+        const short* pa = reinterpret_cast<const short*>(sel_base(bs, slot_of(ra))) + off_of(ra);
+        const short* pb = reinterpret_cast<const short*>(sel_base(bs, slot_of(rb))) + off_of(rb);
+        ea = row < g.M ? (int)pa[(long long)row * sa] : 0;
+        eb = col_l < g.N ? (int)pb[(long long)col_l * sb] : 0;
+      };
+      int ea = 0, eb = 0;
+      if (z.n > 0) {
+        refs(0);
+        exps(0, ea, eb);
+      }
+      for (int s = 0; s < z.n; ++s) {
+        int ean = 0, ebn = 0;
+        if (s + 1 < z.n) {
+          if (((s + 1) & 31) == 0) refs(s + 1);
+          exps(s + 1, ean, ebn);
+        }
         const int b = fg & 1;
         ok = __all_sync(0xffffffffu, wait_z(&accf[b], (fg >> 1) & 1, wait_ns, abort_f, err));
         if (!ok) break;
@@ -267,13 +347,9 @@ __global__ void __launch_bounds__(ZTHREADS, 1) gemm_tcz_kernel(const GGroup* __r
         // the scale of D_0 at (row, column) is 2^(eA + eB - 2060): as a biased
         // FP32 exponent xa + eB, clamped to [0, 254] (0: below the normal
         // range, dropped like the digits below it)
-        const short* eAp = reinterpret_cast<const short*>(sel_base(bs, slot_of(sg.eA))) + off_of(sg.eA);
-        const short* eBp = reinterpret_cast<const short*>(sel_base(bs, slot_of(sg.eB))) + off_of(sg.eB);
-        const int ea = row < g.M ? (int)eAp[(long long)row * sg.eas] : 0;
-        const int eb = col_l < g.N ? (int)eBp[(long long)col_l * sg.ebs] : 0;
         const int xa = ea - 2060 + 127;
         const uint32_t tb = tmem + 256 * b + lane_off + 32 * h;
-        const bool first = si == g.seg0;
+        const bool first = s == 0;
 #pragma unroll
         for (int cb = 0; cb < 32; cb += 16) {
           uint32_t dv[ZDIG][16];
@@ -309,8 +385,42 @@ __global__ void __launch_bounds__(ZTHREADS, 1) gemm_tcz_kernel(const GGroup* __r
         __syncwarp();
         if (lane == 0) mbar_arrive_z(&acce[b]);
         ++fg;
+        ea = ean;
+        eb = ebn;
       }
       if (!ok) break;
+      if (z.parts > 1) {
+        // this part's sums to scratch, 32 rows contiguous per column; the last
+        // part to arrive adds all of them in part order
+        const int t = w / split;
+        uint64_t* sc = scratch + ((size_t)t * split * ZEPI + (warp - 2)) * 1024 + lane;
+        uint64_t* mine = sc + (size_t)z.part * ZEPI * 1024;
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+          __stcg(mine + 32 * i, ((uint64_t)__float_as_uint(lo[i]) << 32) | (uint64_t)__float_as_uint(hi[i]));
+        __threadfence();
+        __syncwarp();
+        unsigned arrived = 0;
+        if (lane == 0) arrived = atomicInc(&tickets[t * ZEPI + warp - 2], z.parts - 1);
+        arrived = __shfl_sync(0xffffffffu, arrived, 0);
+        if (arrived != (unsigned)(z.parts - 1)) continue;
+        __threadfence();
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+          const uint64_t v = __ldcg(sc + 32 * i);
+          hi[i] = __uint_as_float((uint32_t)v);
+          lo[i] = __uint_as_float((uint32_t)(v >> 32));
+        }
+        for (int p = 1; p < z.parts; ++p) {
+          const uint64_t* o = sc + (size_t)p * ZEPI * 1024;
+#pragma unroll
+          for (int i = 0; i < 32; ++i) {
+            const uint64_t v = __ldcg(o + 32 * i);
+            two_sum_z(hi[i], lo[i], __uint_as_float((uint32_t)v));
+            lo[i] += __uint_as_float((uint32_t)(v >> 32));
+          }
+        }
+      }
       // the finished 32 x 32 block, 16 columns at a time through this warp's
       // staging buffer: one row per lane on the way in, 16 lanes per row (128
       // contiguous bytes) on the way out
@@ -380,26 +490,32 @@ int sm_count_z() {
 }  // namespace
 
 int tcz_max_k() { return ZMAXK; }
-size_t tcz_smem_bytes() { return (size_t)ZSTAGES * ZSTAGE_BYTES + ZSTG_BYTES + 1024; }
+size_t tcz_smem_bytes() { return (size_t)ZRING_BYTES + ZSTG_BYTES + 1024; }
 
-cudaError_t launch_gemm_tcz(const GGroup* groups, const GSeg* segs, const GTile* tiles, int ntiles, const void* maps,
-                            const Bases& b, int* err, long long wait_ns, bool pair, cudaStream_t s) {
+int tcz_split(int ntiles, int max_segs) {
+  if (ntiles <= 0) return 1;
+  const int room = sm_count_z() / ntiles;
+  return room < 2 || max_segs < 4 ? 1 : (room < max_segs / 2 ? room : max_segs / 2);
+}
+size_t tcz_scratch_bytes(int ntiles, int split) { return split > 1 ? (size_t)ntiles * split * ZBM * ZBN * 8 : 0; }
+size_t tcz_tickets(int ntiles) { return (size_t)ntiles * ZEPI; }
+
+cudaError_t launch_gemm_tcz(const GGroup* groups, const GSeg* segs, const GTile* tiles, int ntiles, int split,
+                            int kbox, const void* maps, const Bases& b, void* scratch, unsigned* tickets, int* err,
+                            long long wait_ns, bool pair, cudaStream_t s) {
   if (ntiles == 0) return cudaSuccess;
+  if ((kbox != 32 && kbox != 64) || split < 1 || (split > 1 && (!scratch || !tickets))) return cudaErrorInvalidValue;
   const size_t smem = tcz_smem_bytes();
-  static const cudaError_t e1 =
-      cudaFuncSetAttribute(gemm_tcz_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  static const cudaError_t e2 =
-      cudaFuncSetAttribute(gemm_tcz_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e1 != cudaSuccess) return e1;
-  if (e2 != cudaSuccess) return e2;
-  const int grid = ntiles < sm_count_z() ? ntiles : sm_count_z();
-  if (pair)
-    gemm_tcz_kernel<true><<<grid, ZTHREADS, smem, s>>>(groups, segs, tiles, ntiles, (const CUtensorMap*)maps, b, err,
-                                                       wait_ns);
-  else
-    gemm_tcz_kernel<false><<<grid, ZTHREADS, smem, s>>>(groups, segs, tiles, ntiles, (const CUtensorMap*)maps, b, err,
-                                                        wait_ns);
-  return cudaGetLastError();
+  const int nitems = ntiles * split, grid = nitems < sm_count_z() ? nitems : sm_count_z();
+  auto run = [&](auto kernel) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kernel<<<grid, ZTHREADS, smem, s>>>(groups, segs, tiles, nitems, split, (const CUtensorMap*)maps, b,
+                                        (uint64_t*)scratch, tickets, err, wait_ns);
+    return cudaGetLastError();
+  };
+  if (pair) return kbox == 64 ? run(gemm_tcz_kernel<true, 64>) : run(gemm_tcz_kernel<true, 32>);
+  return kbox == 64 ? run(gemm_tcz_kernel<false, 64>) : run(gemm_tcz_kernel<false, 32>);
 }
 
 }  // namespace tt
