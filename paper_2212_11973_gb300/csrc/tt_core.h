@@ -200,6 +200,8 @@ struct GItem {
   // digit output: the int16 exponent of item row i at e + i * e_rs
   Ref e = 0;
   int64_t e_rs = 0;
+  // rows r0 .. rows - 1 are this record's (device plans: an item cut by rows)
+  int r0 = 0;
 };
 struct GContrib {
   Ref src;

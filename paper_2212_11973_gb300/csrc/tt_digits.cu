@@ -155,13 +155,24 @@ __device__ __forceinline__ void digits_of_pair(float S, float Sl, uint32_t* d) {
   d[3] = __float_as_uint(a3);
 }
 
-// One CTA per item.  Each row is taken by a group of G lanes (G the smallest
-// power of two with 2 G >= cols, at most 32), two adjacent columns per lane,
-// so that 32 / G rows share a warp when the item is narrow; the row exponent
-// is a max-reduction inside the group.
-__global__ void __launch_bounds__(DT) gather_digits_kernel(const GItem* __restrict__ items,
-                                                           const GContrib* __restrict__ cs, Bases bs) {
-  const GItem it = items[blockIdx.x];
+// One CTA per item (or share of its rows).  Each row is taken by a group of G
+// lanes (G the smallest power of two with 2 G >= cols, at most 32), two adjacent
+// columns per lane and PP such pairs, so that 32 / G rows share a warp when the
+// item is narrow; the row exponent is a max-reduction inside the group.
+//
+// What bounds it: memory latency (see gather_kernel), then HBM: 8 bytes read per
+// term and 8 written per element.  The term records are in shared memory, a
+// warp has JR rows of PP pairs and two terms in flight (JR PP = 4), and items
+// are cut by rows according to their terms, longest first.
+struct GTerms {
+  const float2* p[GMAXK];
+  int rs[GMAXK];
+  float2 f[GMAXK];  // coefficients as float pairs
+};
+
+template <int PP>
+__device__ __forceinline__ void gather_rows(const GItem& it, const GTerms& t, int nk, const Bases& bs) {
+  constexpr int JR = 4 / PP;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int lg = 0;
   while ((1 << lg) < 32 && 2 * (1 << lg) < it.cols) ++lg;
@@ -171,86 +182,123 @@ __global__ void __launch_bounds__(DT) gather_digits_kernel(const GItem* __restri
                                               off_of(it.dst));
   short* ex = reinterpret_cast<short*>(sel_base(bs, slot_of(it.e))) + off_of(it.e);
   const long long lo2 = sel_lo(bs, slot_of(it.dst)) / 2;  // level stride in BF16 pairs
-  constexpr int PP = GMAXC / 64;                          // column pairs per lane at G = 32
-  // the item's MPO coefficients as float pairs, split once per CTA (FP64
-  // arithmetic runs at ~1/64 of FP32 on GB300)
-  __shared__ float2 cf[GMAXK];
+  const int step = (DT / 32) * rpw;
+  for (int rb = it.r0 + warp * rpw; rb < it.rows; rb += step * JR) {
+    float h[JR][2 * PP], l[JR][2 * PP];
+#pragma unroll
+    for (int j = 0; j < JR; ++j)
+#pragma unroll
+      for (int i = 0; i < 2 * PP; ++i) { h[j][i] = 0.f; l[j][i] = 0.f; }
+    auto load = [&](int k, float4 (*v)[PP]) {
+#pragma unroll
+      for (int j = 0; j < JR; ++j) {
+        const int r = rb + sub + j * step;
+        const float2* s = t.p[k] + (long long)r * t.rs[k];
+        const bool al16 = (reinterpret_cast<uintptr_t>(s) & 15) == 0;
+#pragma unroll
+        for (int i = 0; i < PP; ++i) {
+          const int c = 2 * (gl + G * i);
+          float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (r < it.rows && c < it.cols) {
+            if (al16 && c + 1 < it.cols) {
+              x = *reinterpret_cast<const float4*>(s + c);
+            } else {
+              const float2 v0 = s[c];
+              const float2 v1 = c + 1 < it.cols ? s[c + 1] : make_float2(0.f, 0.f);
+              x = make_float4(v0.x, v0.y, v1.x, v1.y);
+            }
+          }
+          v[j][i] = x;
+        }
+      }
+    };
+    auto add = [&](int k, const float4 (*v)[PP]) {
+      const float2 f = t.f[k];
+#pragma unroll
+      for (int j = 0; j < JR; ++j)
+#pragma unroll
+        for (int i = 0; i < PP; ++i) {
+          df_fma(h[j][2 * i], l[j][2 * i], f.x, f.y, v[j][i].x, v[j][i].y);
+          df_fma(h[j][2 * i + 1], l[j][2 * i + 1], f.x, f.y, v[j][i].z, v[j][i].w);
+        }
+    };
+    int k = 0;
+    for (; k + 1 < nk; k += 2) {
+      float4 v0[JR][PP], v1[JR][PP];
+      load(k, v0);
+      load(k + 1, v1);
+      add(k, v0);
+      add(k + 1, v1);
+    }
+    if (k < nk) {
+      float4 v0[JR][PP];
+      load(k, v0);
+      add(k, v0);
+    }
+#pragma unroll
+    for (int j = 0; j < JR; ++j) {
+      const int r = rb + sub + j * step;
+      // renormalise every pair (TwoSum of h and l): after cancellation l may be
+      // as large as h, and the digits below are taken from h and l separately
+#pragma unroll
+      for (int i = 0; i < 2 * PP; ++i) {
+        const float sv = h[j][i] + l[j][i];
+        const float bp = sv - h[j][i];
+        l[j][i] = (h[j][i] - (sv - bp)) + (l[j][i] - bp);
+        h[j][i] = sv;
+      }
+      int m = 0;
+#pragma unroll
+      for (int i = 0; i < PP; ++i) {
+        const int c = 2 * (gl + G * i);
+        if (c < it.cols) m = max(m, fexp(h[j][2 * i]));
+        if (c + 1 < it.cols) m = max(m, fexp(h[j][2 * i + 1]));
+      }
+      for (int o = G >> 1; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+      // one exponent above the largest: |h + l| < 2^(m - 1023), so the scaled
+      // values stay below 2^31 also after rounding
+      if (m) m = m + 1;
+      // scale 2^(1054 - m) as two exact power-of-two factors in the FP32 range
+      const int sh = m ? 1054 - m : 0, sa = sh / 2, sb = sh - sa;
+      const float fa = p2f(sa), fb = p2f(sb);
+      if (r < it.rows) {
+        uint32_t* drow = dst + ((long long)r * it.dst_rs >> 1);
+#pragma unroll
+        for (int i = 0; i < PP; ++i) {
+          const int c = 2 * (gl + G * i);
+          if (c < it.cols) {
+            uint32_t d0[4], d1[4] = {0u, 0u, 0u, 0u};
+            digits_of_pair((h[j][2 * i] * fa) * fb, (l[j][2 * i] * fa) * fb, d0);
+            if (c + 1 < it.cols) digits_of_pair((h[j][2 * i + 1] * fa) * fb, (l[j][2 * i + 1] * fa) * fb, d1);
+#pragma unroll
+            for (int lv = 0; lv < 4; ++lv) drow[lv * lo2 + (c >> 1)] = __byte_perm(d0[lv], d1[lv], 0x7632);
+          }
+        }
+        if (gl == 0) ex[(long long)r * it.e_rs] = (short)m;
+      }
+    }
+  }
+}
+
+__global__ void __launch_bounds__(DT) gather_digits_kernel(const GItem* __restrict__ items,
+                                                           const GContrib* __restrict__ cs, Bases bs) {
+  const GItem it = items[blockIdx.x];
+  // the item's terms, the MPO coefficients split into float pairs once per CTA
+  // (FP64 arithmetic runs at ~1/64 of FP32 on GB300)
+  __shared__ GTerms t;
   // the host rejects items with more terms; the clamp keeps the table in bounds
   const int nk = min(it.c1 - it.c0, GMAXK);
   for (int k = threadIdx.x; k < nk; k += DT) {
-    const double v = cs[it.c0 + k].coef;
-    const float ch = (float)v;
-    cf[k] = make_float2(ch, (float)(v - (double)ch));
+    const GContrib cb = cs[it.c0 + k];
+    const float ch = (float)cb.coef;
+    t.p[k] = reinterpret_cast<const float2*>(sel_base(bs, slot_of(cb.src))) + off_of(cb.src);
+    t.rs[k] = (int)cb.src_rs;
+    t.f[k] = make_float2(ch, (float)(cb.coef - (double)ch));
   }
   __syncthreads();
-  for (int r0 = warp * rpw; r0 < it.rows; r0 += (DT / 32) * rpw) {
-    const int r = r0 + sub;
-    const bool rin = r < it.rows;
-    float h[2 * PP], l[2 * PP];
-#pragma unroll
-    for (int i = 0; i < 2 * PP; ++i) { h[i] = 0.f; l[i] = 0.f; }
-    for (int k = it.c0; k < it.c0 + nk; ++k) {
-      const GContrib cb = cs[k];
-      const float ch = cf[k - it.c0].x, cl = cf[k - it.c0].y;
-      const float2* s = reinterpret_cast<const float2*>(sel_base(bs, slot_of(cb.src))) + off_of(cb.src) +
-                        (long long)r * cb.src_rs;
-      const bool al16 = (reinterpret_cast<uintptr_t>(s) & 15) == 0;
-#pragma unroll
-      for (int i = 0; i < PP; ++i) {
-        const int c = 2 * (gl + G * i);
-        if (rin && c < it.cols) {
-          float4 v;
-          if (al16 && c + 1 < it.cols) {
-            v = *reinterpret_cast<const float4*>(s + c);
-          } else {
-            const float2 v0 = s[c];
-            const float2 v1 = c + 1 < it.cols ? s[c + 1] : make_float2(0.f, 0.f);
-            v = make_float4(v0.x, v0.y, v1.x, v1.y);
-          }
-          df_fma(h[2 * i], l[2 * i], ch, cl, v.x, v.y);
-          df_fma(h[2 * i + 1], l[2 * i + 1], ch, cl, v.z, v.w);
-        }
-      }
-    }
-    // renormalise every pair (TwoSum of h and l): after cancellation l may be
-    // as large as h, and the digits below are taken from h and l separately
-#pragma unroll
-    for (int i = 0; i < 2 * PP; ++i) {
-      const float sv = h[i] + l[i];
-      const float bp = sv - h[i];
-      l[i] = (h[i] - (sv - bp)) + (l[i] - bp);
-      h[i] = sv;
-    }
-    int m = 0;
-#pragma unroll
-    for (int i = 0; i < PP; ++i) {
-      const int c = 2 * (gl + G * i);
-      if (c < it.cols) m = max(m, fexp(h[2 * i]));
-      if (c + 1 < it.cols) m = max(m, fexp(h[2 * i + 1]));
-    }
-    for (int o = G >> 1; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-    // one exponent above the largest: |h + l| < 2^(m - 1023), so the scaled
-    // values stay below 2^31 also after rounding
-    if (m) m = m + 1;
-    // scale 2^(1054 - m) as two exact power-of-two factors in the FP32 range
-    const int sh = m ? 1054 - m : 0, sa = sh / 2, sb = sh - sa;
-    const float fa = p2f(sa), fb = p2f(sb);
-    if (rin) {
-      uint32_t* drow = dst + ((long long)r * it.dst_rs >> 1);
-#pragma unroll
-      for (int i = 0; i < PP; ++i) {
-        const int c = 2 * (gl + G * i);
-        if (c < it.cols) {
-          uint32_t d0[4], d1[4] = {0u, 0u, 0u, 0u};
-          digits_of_pair((h[2 * i] * fa) * fb, (l[2 * i] * fa) * fb, d0);
-          if (c + 1 < it.cols) digits_of_pair((h[2 * i + 1] * fa) * fb, (l[2 * i + 1] * fa) * fb, d1);
-#pragma unroll
-          for (int lv = 0; lv < 4; ++lv) drow[lv * lo2 + (c >> 1)] = __byte_perm(d0[lv], d1[lv], 0x7632);
-        }
-      }
-      if (gl == 0) ex[(long long)r * it.e_rs] = (short)m;
-    }
-  }
+  if (it.cols <= 64) gather_rows<1>(it, t, nk, bs);
+  else if (it.cols <= 128) gather_rows<2>(it, t, nk, bs);
+  else gather_rows<GMAXC / 64>(it, t, nk, bs);
 }
 
 }  // namespace

@@ -118,16 +118,36 @@ void upload(tt_ctx* c, const GemmPlan& p, DevGemmBuf& o) {
 }
 
 void upload(tt_ctx* c, const GatherPlan& p, DevGatherBuf& o) {
-  size_t bi = align_up<GItem>(p.items.size() * sizeof(GItem));
+  // items cut by rows into shares of one or more passes (the rows a CTA has in
+  // flight: 32, or fewer of a wide item), the fewer the more terms: an item that
+  // closes 50 hops over 180 rows would outlast all others by itself.  Those
+  // with the most terms first.
+  std::vector<std::vector<GItem>> by_terms(64);
+  size_t count = 0;
+  for (const GItem& it : p.items) {
+    const int nk = it.c1 - it.c0;
+    const int pass = it.cols <= 64 ? 32 : (it.cols <= 128 ? 16 : 8);
+    const int per = pass * std::max(1, 24 / (nk + 2));
+    std::vector<GItem>& to = by_terms[std::min(nk, 63)];
+    for (int r0 = 0; r0 < it.rows; r0 += per, ++count) {
+      to.push_back(it);
+      to.back().r0 = r0;
+      to.back().rows = std::min(it.rows, r0 + per);
+    }
+  }
+  std::vector<GItem> items;
+  items.reserve(count);
+  for (int k = 63; k >= 0; --k) items.insert(items.end(), by_terms[k].begin(), by_terms[k].end());
+  size_t bi = align_up<GItem>(items.size() * sizeof(GItem));
   size_t bc = align_up<GContrib>(p.contribs.size() * sizeof(GContrib));
   ensure(c, o.buf, bi + bc);
   char* base = (char*)o.buf.p;
-  if (!p.items.empty()) CK(cudaMemcpyAsync(base, p.items.data(), p.items.size() * sizeof(GItem), cudaMemcpyHostToDevice, c->st));
+  if (!items.empty()) CK(cudaMemcpyAsync(base, items.data(), items.size() * sizeof(GItem), cudaMemcpyHostToDevice, c->st));
   if (!p.contribs.empty()) CK(cudaMemcpyAsync(base + bi, p.contribs.data(), p.contribs.size() * sizeof(GContrib), cudaMemcpyHostToDevice, c->st));
   CK(cudaStreamSynchronize(c->st));
   o.d.items = (GItem*)base;
   o.d.contribs = (GContrib*)(base + bi);
-  o.d.nitems = (int)p.items.size();
+  o.d.nitems = (int)items.size();
   o.d.elems = p.elems;
   o.host = p;
   o.checked = false;

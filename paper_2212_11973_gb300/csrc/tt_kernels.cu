@@ -13,6 +13,7 @@
 
 #include <cmath>
 #include <cstdint>
+#include <type_traits>
 
 #include "tt_df.h"
 #include "tt_kernels.h"
@@ -268,12 +269,20 @@ __global__ void __launch_bounds__(128) gemm_bf16_split_kernel(const GGroup* __re
 }
 
 // ---------------------------------------------------------------------------
-// W gather: dst[r, c] = sum_k coef_k src_k[r, c]  (one CTA per item, rows
-// strided over the 8 warps, columns over the lanes).  FP64 in, FP64 out for
-// the FP64 path.  Mixed path: the sources are the FP32 outputs of S1, so the
-// sum and the split into bf16 levels run in FP32 (GB300 has about 1/64 of
+// W gather: dst[r, c] = sum_k coef_k src_k[r, c].  One CTA per item (or share of
+// its rows), rows over the 8 warps, columns over the lanes.  FP64 in, FP64 out
+// for the FP64 path.  Mixed path: the sources are the FP32 outputs of S1, so
+// the sum and the split into bf16 levels run in FP32 (GB300 has about 1/64 of
 // its FP32 rate in FP64); each level's remainder is exact in FP32.
+//
+// What bounds it: memory latency.  Most items have one or two terms, the ones
+// that close a hop several dozen, and with one row and one load at a time per
+// warp such an item alone took longer than all others.  The term records sit in
+// shared memory, four rows and two terms are in flight per lane, and items are
+// cut by rows according to their terms (upload), longest first.
 // ---------------------------------------------------------------------------
+constexpr int GT_TAB = 64;  // terms kept in shared memory (more: read as they come)
+
 template <int NS>
 __device__ __forceinline__ void store_split_f32(__nv_bfloat16* p, long long lo, float v) {
 #pragma unroll
@@ -296,29 +305,61 @@ __device__ __forceinline__ void store_split_f64(__nv_bfloat16* p, long long lo, 
 template <int IN, int OUT>
 __global__ void __launch_bounds__(256) gather_kernel(const GItem* __restrict__ items,
                                                      const GContrib* __restrict__ cs, Bases bs) {
+  using T = typename std::conditional<IN == 0, double, float>::type;
+  constexpr int JR = 4;
+  __shared__ const T* tp[GT_TAB];
+  __shared__ long long trs[GT_TAB];
+  __shared__ T tc[GT_TAB];
   const GItem it = items[blockIdx.x];
+  const int nk = it.c1 - it.c0;
+  for (int k = threadIdx.x; k < min(nk, GT_TAB); k += 256) {
+    const GContrib cb = cs[it.c0 + k];
+    tp[k] = rptr<const T>(bs, cb.src);
+    trs[k] = cb.src_rs;
+    tc[k] = (T)cb.coef;
+  }
+  __syncthreads();
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  for (int r = ty; r < it.rows; r += 8)
+  for (int r = it.r0 + ty; r < it.rows; r += 8 * JR)
     for (int c = tx; c < it.cols; c += 32) {
-      const long long d = (long long)r * it.dst_rs + c;
-      if constexpr (IN == 0) {
-        double acc = 0.0;
-        for (int k = it.c0; k < it.c1; ++k) {
-          const GContrib cb = cs[k];
-          acc = fma(cb.coef, rptr<const double>(bs, cb.src)[(long long)r * cb.src_rs + c], acc);
+      T acc[JR];
+#pragma unroll
+      for (int j = 0; j < JR; ++j) acc[j] = (T)0;
+      auto load = [&](const T* p, long long rs, T* v) {
+#pragma unroll
+        for (int j = 0; j < JR; ++j) v[j] = r + 8 * j < it.rows ? p[(long long)(r + 8 * j) * rs + c] : (T)0;
+      };
+      auto add = [&](T f, const T* v) {
+#pragma unroll
+        for (int j = 0; j < JR; ++j) acc[j] = fma(f, v[j], acc[j]);
+      };
+      int k = 0;
+      for (; k + 1 < min(nk, GT_TAB); k += 2) {
+        T v0[JR], v1[JR];
+        load(tp[k], trs[k], v0);
+        load(tp[k + 1], trs[k + 1], v1);
+        add(tc[k], v0);
+        add(tc[k + 1], v1);
+      }
+      for (; k < nk; ++k) {
+        T v0[JR];
+        if (k < GT_TAB) {
+          load(tp[k], trs[k], v0);
+          add(tc[k], v0);
+        } else {
+          const GContrib cb = cs[it.c0 + k];
+          load(rptr<const T>(bs, cb.src), cb.src_rs, v0);
+          add((T)cb.coef, v0);
         }
-        if constexpr (OUT == 0) rptr<double>(bs, it.dst)[d] = acc;
-        else if constexpr (OUT == 1) rptr<float>(bs, it.dst)[d] = (float)acc;
-        else store_split_f64<OUT>(rptr<__nv_bfloat16>(bs, it.dst) + d, sel_lo(bs, slot_of(it.dst)), acc);
-      } else {
-        float acc = 0.f;
-        for (int k = it.c0; k < it.c1; ++k) {
-          const GContrib cb = cs[k];
-          acc = fmaf((float)cb.coef, rptr<const float>(bs, cb.src)[(long long)r * cb.src_rs + c], acc);
-        }
-        if constexpr (OUT == 0) rptr<double>(bs, it.dst)[d] = (double)acc;
-        else if constexpr (OUT == 1) rptr<float>(bs, it.dst)[d] = acc;
-        else store_split_f32<OUT>(rptr<__nv_bfloat16>(bs, it.dst) + d, sel_lo(bs, slot_of(it.dst)), acc);
+      }
+#pragma unroll
+      for (int j = 0; j < JR; ++j) {
+        if (r + 8 * j >= it.rows) continue;
+        const long long d = (long long)(r + 8 * j) * it.dst_rs + c;
+        if constexpr (OUT == 0) rptr<double>(bs, it.dst)[d] = (double)acc[j];
+        else if constexpr (OUT == 1) rptr<float>(bs, it.dst)[d] = (float)acc[j];
+        else if constexpr (IN == 0) store_split_f64<OUT>(rptr<__nv_bfloat16>(bs, it.dst) + d, sel_lo(bs, slot_of(it.dst)), acc[j]);
+        else store_split_f32<OUT>(rptr<__nv_bfloat16>(bs, it.dst) + d, sel_lo(bs, slot_of(it.dst)), acc[j]);
       }
     }
 }
