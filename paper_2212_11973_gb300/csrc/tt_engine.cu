@@ -78,7 +78,31 @@ static size_t align_up(size_t x) {
   return (x + 255) / 256 * 256 + 0 * sizeof(T);
 }
 
-void upload(tt_ctx* c, const GemmPlan& p, DevGemmBuf& o) {
+// Arrays of one or more plans gathered on the host and sent to the device in one
+// allocation and one copy: a site has ten plans of several arrays each, and an
+// allocation, a pageable copy and a synchronisation apiece took longer than
+// the contractions of a small system.
+struct Stager {
+  std::vector<char> h;
+  std::vector<std::pair<void**, size_t>> fix;
+  template <class T>
+  void add(const std::vector<T>& v, T** dst) {
+    const size_t off = (h.size() + 255) / 256 * 256, bytes = v.size() * sizeof(T);
+    h.resize(off + bytes);
+    if (bytes) std::memcpy(h.data() + off, v.data(), bytes);
+    fix.push_back({(void**)dst, off});
+  }
+  void commit(tt_ctx* c, DBuf& buf) {
+    ensure(c, buf, h.size() + 16);
+    if (!h.empty()) {
+      CK(cudaMemcpyAsync(buf.p, h.data(), h.size(), cudaMemcpyHostToDevice, c->st));
+      CK(cudaStreamSynchronize(c->st));
+    }
+    for (auto& f : fix) *f.first = (char*)buf.p + f.second;
+  }
+};
+
+static std::vector<GTile> tiles64_of(const GemmPlan& p) {
   std::vector<GTile> tiles;
   std::vector<std::pair<double, int>> order;
   for (size_t g = 0; g < p.groups.size(); ++g) {
@@ -92,32 +116,36 @@ void upload(tt_ctx* c, const GemmPlan& p, DevGemmBuf& o) {
     for (int m0 = 0; m0 < g.M; m0 += 64)
       for (int n0 = 0; n0 < g.N; n0 += 64) tiles.push_back(GTile{og.second, m0, n0, 0});
   }
-  size_t bg = align_up<GGroup>(p.groups.size() * sizeof(GGroup));
-  size_t bsg = align_up<GSeg>(p.segs.size() * sizeof(GSeg));
-  size_t bt = align_up<GTile>(tiles.size() * sizeof(GTile));
-  ensure(c, o.buf, bg + bsg + bt);
-  char* base = (char*)o.buf.p;
-  if (!p.groups.empty()) CK(cudaMemcpyAsync(base, p.groups.data(), p.groups.size() * sizeof(GGroup), cudaMemcpyHostToDevice, c->st));
-  if (!p.segs.empty()) CK(cudaMemcpyAsync(base + bg, p.segs.data(), p.segs.size() * sizeof(GSeg), cudaMemcpyHostToDevice, c->st));
-  if (!tiles.empty()) CK(cudaMemcpyAsync(base + bg + bsg, tiles.data(), tiles.size() * sizeof(GTile), cudaMemcpyHostToDevice, c->st));
-  CK(cudaStreamSynchronize(c->st));
-  o.d.groups = (GGroup*)base;
-  o.d.segs = (GSeg*)(base + bg);
-  o.d.tiles64 = (GTile*)(base + bg + bsg);
+  return tiles;
+}
+
+// The plan's arrays into a stager; the tile lists of the 64 x 64 kernels and, by
+// default, of the FP64 kernel follow when a launch first needs them.
+static void upload(Stager& s, GemmPlan p, DevGemmBuf& o, bool f64list = false) {
+  s.add(p.groups, &o.d.groups);
+  s.add(p.segs, &o.d.segs);
   o.d.ngroups = (int)p.groups.size();
   o.d.nsegs = (int)p.segs.size();
-  o.d.ntiles64 = (int)tiles.size();
+  o.d.ntiles64 = -1;
   o.d.flops = p.flops;
-  o.host = p;
   o.checked = false;
   o.tc_checked = o.tc_ok = false;
   o.ntiles128 = o.ntilesp = 0;
   o.d.ntilesf = o.d.tf = 0;
+  if (f64list) {
+    const F64Shape sh = f64_shape(p);
+    o.d.tf = sh.T;
+    o.d.wkf = sh.wk;
+    const std::vector<FTile> t = f64_tiles(p, sh.T);
+    s.add(t, &o.d.tilesf);
+    o.d.ntilesf = (int)t.size();
+  }
   o.choice = -1;
   for (int i = 0; i < 8; ++i) { o.key_p[i] = nullptr; o.key_lo[i] = 0; }
+  o.host = std::move(p);
 }
 
-void upload(tt_ctx* c, const GatherPlan& p, DevGatherBuf& o) {
+static void upload(Stager& s, const GatherPlan& p, DevGatherBuf& o) {
   // items cut by rows into shares of one or more passes (the rows a CTA has in
   // flight: 32, or fewer of a wide item), the fewer the more terms: an item that
   // closes 50 hops over 180 rows would outlast all others by itself.  Those
@@ -138,40 +166,40 @@ void upload(tt_ctx* c, const GatherPlan& p, DevGatherBuf& o) {
   std::vector<GItem> items;
   items.reserve(count);
   for (int k = 63; k >= 0; --k) items.insert(items.end(), by_terms[k].begin(), by_terms[k].end());
-  size_t bi = align_up<GItem>(items.size() * sizeof(GItem));
-  size_t bc = align_up<GContrib>(p.contribs.size() * sizeof(GContrib));
-  ensure(c, o.buf, bi + bc);
-  char* base = (char*)o.buf.p;
-  if (!items.empty()) CK(cudaMemcpyAsync(base, items.data(), items.size() * sizeof(GItem), cudaMemcpyHostToDevice, c->st));
-  if (!p.contribs.empty()) CK(cudaMemcpyAsync(base + bi, p.contribs.data(), p.contribs.size() * sizeof(GContrib), cudaMemcpyHostToDevice, c->st));
-  CK(cudaStreamSynchronize(c->st));
-  o.d.items = (GItem*)base;
-  o.d.contribs = (GContrib*)(base + bi);
+  s.add(items, &o.d.items);
+  s.add(p.contribs, &o.d.contribs);
   o.d.nitems = (int)items.size();
   o.d.elems = p.elems;
-  o.host = p;
-  o.checked = false;
 }
 
-void upload(tt_ctx* c, const CopyPlan& p, DevCopyBuf& o) {
-  ensure(c, o.buf, p.items.size() * sizeof(CItem));
-  if (!p.items.empty()) CK(cudaMemcpyAsync(o.buf.p, p.items.data(), p.items.size() * sizeof(CItem), cudaMemcpyHostToDevice, c->st));
-  CK(cudaStreamSynchronize(c->st));
-  o.d.items = (CItem*)o.buf.p;
+static void upload(Stager& s, const CopyPlan& p, DevCopyBuf& o) {
+  s.add(p.items, &o.d.items);
   o.d.nitems = (int)p.items.size();
   o.d.maxtiles = 0;
   for (const CItem& it : p.items)
     o.d.maxtiles = std::max<int64_t>(o.d.maxtiles, (int64_t)((it.rows + 31) / 32) * ((it.cols + 31) / 32));
-  o.host = p;
-  o.checked = false;
+}
+
+static void upload(Stager& s, const DigitPlan& p, DevDigitBuf& o) {
+  s.add(p.items, &o.d.items);
+  o.d.nitems = (int)p.items.size();
+  o.d.maxgroups = 0;
+  for (const DItem& it : p.items) o.d.maxgroups = std::max(o.d.maxgroups, (it.rows + 31) / 32);
+}
+
+// one plan by itself
+template <class Plan, class Dev>
+static void upload(tt_ctx* c, Plan&& p, Dev& o) {
+  Stager s;
+  upload(s, std::forward<Plan>(p), o);
+  s.commit(c, o.buf);
 }
 
 void release(tt_ctx* c, DevGemmBuf& o) {
   dfree(c, o.buf);
-  dfree(c, o.maps);
-  dfree(c, o.tiles128);
-  dfree(c, o.tilesp);
+  dfree(c, o.tcbuf);
   dfree(c, o.tilesf);
+  dfree(c, o.tiles64);
   o.d = DevGemm();
   o.host = GemmPlan();
   o.checked = o.tc_checked = o.tc_ok = false;
@@ -179,21 +207,9 @@ void release(tt_ctx* c, DevGemmBuf& o) {
   o.choice = -1;
   for (int i = 0; i < 8; ++i) { o.key_p[i] = nullptr; o.key_lo[i] = 0; }
 }
-void release(tt_ctx* c, DevGatherBuf& o) { dfree(c, o.buf); o.d = DevGather(); o.host = GatherPlan(); o.checked = false; }
-void release(tt_ctx* c, DevCopyBuf& o) { dfree(c, o.buf); o.d = DevCopy(); o.host = CopyPlan(); o.checked = false; }
-
-void upload(tt_ctx* c, const DigitPlan& p, DevDigitBuf& o) {
-  ensure(c, o.buf, p.items.size() * sizeof(DItem) + 16);
-  if (!p.items.empty())
-    CK(cudaMemcpyAsync(o.buf.p, p.items.data(), p.items.size() * sizeof(DItem), cudaMemcpyHostToDevice, c->st));
-  CK(cudaStreamSynchronize(c->st));
-  o.d.items = (DItem*)o.buf.p;
-  o.d.nitems = (int)p.items.size();
-  o.d.maxgroups = 0;
-  for (const DItem& it : p.items) o.d.maxgroups = std::max(o.d.maxgroups, (it.rows + 31) / 32);
-  o.host = p;
-}
-void release(tt_ctx* c, DevDigitBuf& o) { dfree(c, o.buf); o.d = DevDigit(); o.host = DigitPlan(); }
+void release(tt_ctx* c, DevGatherBuf& o) { dfree(c, o.buf); o.d = DevGather(); }
+void release(tt_ctx* c, DevCopyBuf& o) { dfree(c, o.buf); o.d = DevCopy(); }
+void release(tt_ctx* c, DevDigitBuf& o) { dfree(c, o.buf); o.d = DevDigit(); }
 
 static void check_ref(Ref r, int64_t last, const Caps& c, const char* what, const char* op) {
   int slot = (int)(r >> 56);
@@ -362,6 +378,11 @@ struct Eng {
     for (int j = 0; j < r->N; ++j) nmax = std::max(nmax, r->lay[j].size);
     for (int k = 0; k <= r->N; ++k) nmax = std::max(nmax, make_bondmat_layout(r->bond[k]).size);
     if (nmax > r->ldq) {
+      if (r->apply_only) {  // one apply: the output vector is all it needs
+        r->ldq = nmax;
+        ensure(c, r->W, (size_t)nmax * sizeof(double));
+        return;
+      }
       int64_t cap = nmax + nmax / 4 + 64;
       r->ldq = cap;
       ensure(c, r->Qk, (size_t)cap * r->opts.krylov_dim * sizeof(double));
@@ -375,6 +396,24 @@ struct Eng {
 
   // ---- plans --------------------------------------------------------------
   // FP64 plans of site j whatever the precision (the measurement's energy)
+  // a site's plans to the device, all in one buffer
+  void stage_site(SiteDev& s, bool f64list) {
+    Stager g;
+    upload(g, s.h.xsplit, s.xs);
+    upload(g, s.h.xdig, s.xd);
+    upload(g, std::move(s.h.s1), s.s1, f64list);
+    upload(g, s.h.s2, s.s2);
+    upload(g, std::move(s.h.s3), s.s3, f64list);
+    upload(g, std::move(s.h.s3l), s.s3l, f64list);
+    upload(g, std::move(s.h.r1), s.r1, f64list);
+    upload(g, s.h.r2, s.r2);
+    upload(g, std::move(s.h.r3), s.r3, f64list);
+    g.commit(c, s.arena);
+    s.h.s2 = GatherPlan();
+    s.h.r2 = GatherPlan();
+    s.h.xsplit = CopyPlan();
+    s.h.xdig = DigitPlan();
+  }
   SiteDev& site_plan_fp64(int j) {
     if (!mixed()) return site_plan(j);
     SiteDev& s = r->sp64[j];
@@ -382,13 +421,7 @@ struct Eng {
     const Mpo& m = M();
     s.h = build_site_plan(r->bond[j], r->bond[j + 1], m.ls, m.site[j].terms, m.chan[j], m.chan[j + 1], false);
     validate_site(s.h, r->bond[j], r->bond[j + 1], m.chan[j], m.chan[j + 1], false);
-    upload(c, s.h.s1, s.s1);
-    upload(c, s.h.s2, s.s2);
-    upload(c, s.h.s3, s.s3);
-    upload(c, s.h.s3l, s.s3l);
-    upload(c, s.h.r1, s.r1);
-    upload(c, s.h.r2, s.r2);
-    upload(c, s.h.r3, s.r3);
+    stage_site(s, false);
     ensure(c, r->T1, (size_t)std::max(s.h.t1_size, s.h.u1_size) * 8);
     ensure(c, r->T2, (size_t)std::max(s.h.t2_size, s.h.u2_size) * 8);
     s.valid = true;
@@ -410,19 +443,13 @@ struct Eng {
     SiteDev& s = r->sp[j];
     if (s.valid) return s;
     const Mpo& m = M();
+    // the environment updates run on these plans in FP64 and env_precision -1
+    const unsigned parts = r->apply_only || (mixed() && !env_mixed()) ? SP_APPLY : SP_ALL;
     s.h = build_site_plan(r->bond[j], r->bond[j + 1], m.ls, m.site[j].terms, m.chan[j], m.chan[j + 1], mixed(),
-                          r->exact);
+                          r->exact, parts);
     validate_site(s.h, r->bond[j], r->bond[j + 1], m.chan[j], m.chan[j + 1], mixed(), r->exact);
-    upload(c, s.h.xsplit, s.xs);
-    upload(c, s.h.xdig, s.xd);
     if (mixed()) ensure(c, r->Xs, (size_t)std::max<int64_t>(s.h.xt_size, 1) * split_bytes());
-    upload(c, s.h.s1, s.s1);
-    upload(c, s.h.s2, s.s2);
-    upload(c, s.h.s3, s.s3);
-    upload(c, s.h.s3l, s.s3l);
-    upload(c, s.h.r1, s.r1);
-    upload(c, s.h.r2, s.r2);
-    upload(c, s.h.r3, s.r3);
+    stage_site(s, !mixed());
     ensure(c, r->T1, (size_t)std::max(s.h.t1_size, s.h.u1_size) * 8);
     // FP64, split levels or digit levels plus exponents
     ensure(c, r->T2, (size_t)std::max(s.h.t2_size, s.h.u2_size) * std::max<size_t>(8, split_bytes()));
@@ -499,16 +526,18 @@ struct Eng {
                    "B T digits");
       }
     }
-    upload(c, b.h.b1, b.b1);
-    upload(c, b.h.b2, b.b2);
+    Stager g;
+    upload(g, std::move(b.h.b1), b.b1, !mixed());
+    upload(g, std::move(b.h.b2), b.b2, !mixed());
     if (mixed()) {
-      upload(c, b.h.xsplit, b.xs);
-      upload(c, b.h.tsplit, b.ts);
-      upload(c, b.h.xdig, b.xd);
-      upload(c, b.h.tdig, b.td);
+      upload(g, b.h.xsplit, b.xs);
+      upload(g, b.h.tsplit, b.ts);
+      upload(g, b.h.xdig, b.xd);
+      upload(g, b.h.tdig, b.td);
       ensure(c, r->Xs, (size_t)std::max<int64_t>(b.h.xt_size, 1) * split_bytes());
       ensure(c, r->T2, (size_t)std::max<int64_t>(b.h.tp_size, 1) * split_bytes());
     }
+    g.commit(c, b.arena);
     ensure(c, r->T1, (size_t)b.h.t_size * 8);
     ensure(c, r->T2, (size_t)b.h.t_size * 8);
     b.valid = true;
@@ -544,12 +573,11 @@ struct Eng {
             J.r + (int64_t)J.n * J.n > q.h.ws_size || J.n > 2048)
           throw Err{TT_ERR_STATE, "QR job outside the workspace or wider than 2048"};
     }
-    ensure(c, q.jobs, q.h.jobs.size() * sizeof(QrJob));
-    if (!q.h.jobs.empty())
-      CK(cudaMemcpyAsync(q.jobs.p, q.h.jobs.data(), q.h.jobs.size() * sizeof(QrJob), cudaMemcpyHostToDevice, st));
-    upload(c, q.h.gather, q.gather);
-    upload(c, q.h.scatter, q.scatter);
-    upload(c, q.h.rout, q.rout);
+    Stager g;
+    g.add(q.h.jobs, &q.jobs);
+    upload(g, q.h.gather, q.gather);
+    upload(g, q.h.scatter, q.scatter);
+    upload(g, q.h.rout, q.rout);
     int64_t wsz = q.h.ws_size;
     if (r->use_cholqr) {
       CholQrPlan cp = build_cholqr(q.h.jobs, q.h.ws_size);
@@ -558,8 +586,8 @@ struct Eng {
       for (int p = 0; p < 3; ++p) {
         check_plan(cp.gram[p], cw, "CholQR gram");
         check_plan(cp.app[p], cw, "CholQR apply");
-        upload(c, cp.gram[p], q.gram[p]);
-        upload(c, cp.app[p], q.app[p]);
+        upload(g, std::move(cp.gram[p]), q.gram[p], true);
+        upload(g, std::move(cp.app[p]), q.app[p], true);
         for (const CholJob& J : cp.cj[p])
           if (J.g + (int64_t)J.parts * J.n * J.n > wsz || J.parts < 1 || J.r + (int64_t)J.n * J.n > wsz ||
               J.ri + (int64_t)J.n * J.n > wsz || J.pk < 0 || J.pk + (int64_t)J.n * (J.n + 1) / 2 > wsz)
@@ -567,23 +595,26 @@ struct Eng {
         q.ncj[p] = (int)cp.cj[p].size();
         q.maxn[p] = 0;
         for (const CholJob& cj : cp.cj[p]) q.maxn[p] = std::max(q.maxn[p], cj.n);
-        ensure(c, q.cjobs[p], cp.cj[p].size() * sizeof(CholJob) + 16);
-        if (!cp.cj[p].empty())
-          CK(cudaMemcpyAsync(q.cjobs[p].p, cp.cj[p].data(), cp.cj[p].size() * sizeof(CholJob), cudaMemcpyHostToDevice,
-                             st));
+        g.add(cp.cj[p], &q.cjobs[p]);
       }
       check_plan(cp.tt, cw, "CholQR T");
       check_plan(cp.rf, cw, "CholQR R");
-      upload(c, cp.tt, q.tt);
-      upload(c, cp.rf, q.rf);
+      upload(g, std::move(cp.tt), q.tt, true);
+      upload(g, std::move(cp.rf), q.rf, true);
       ensure(c, q.fail, q.h.jobs.size() * sizeof(int) + 16);
     }
+    g.commit(c, q.arena);
     ensure(c, r->ws, (size_t)wsz * 8);
     ensure(c, r->Sb, (size_t)q.h.s_size * 8);
     q.valid = true;
     return q;
   }
 
+  void upload_f64(GemmPlan p, DevGemmBuf& o) {
+    Stager s;
+    upload(s, std::move(p), o, true);
+    s.commit(c, o.buf);
+  }
   DevGemmBuf& absorb_left_plan(int j) {  // into site j from the bond on its left
     if (!r->absl_ok[j]) {
       std::vector<int> ident(r->bond[j].nsec());
@@ -591,7 +622,7 @@ struct Eng {
       BondMatLayout bm = make_bondmat_layout(r->bond[j]);
       GemmPlan g = build_absorb_left(r->lay[j], r->lay[j], r->bond[j], r->bond[j], bm.off, ident);
       check_plan(g, caps({{S_X, r->lay[j].size}, {S_AUX, bm.size}, {S_Y, r->lay[j].size}}), "absorb L");
-      upload(c, g, r->absl[j]);
+      upload_f64(std::move(g), r->absl[j]);
       r->absl_ok[j] = 1;
     }
     return r->absl[j];
@@ -603,7 +634,7 @@ struct Eng {
       BondMatLayout bm = make_bondmat_layout(r->bond[j + 1]);
       GemmPlan g = build_absorb_right(r->lay[j], r->lay[j], r->bond[j + 1], r->bond[j + 1], bm.off, ident);
       check_plan(g, caps({{S_X, r->lay[j].size}, {S_AUX, bm.size}, {S_Y, r->lay[j].size}}), "absorb R");
-      upload(c, g, r->absr[j]);
+      upload_f64(std::move(g), r->absr[j]);
       r->absr_ok[j] = 1;
     }
     return r->absr[j];
@@ -665,27 +696,6 @@ struct Eng {
         if (sg.tA != 0 || sg.tB != 1 || sg.lda % 8 || sg.ldb % 8 || oa % 8 || ob % 8) g.tc_ok = false;
       }
       if (!g.tc_ok) return false;
-      // tile lists of both tcgen05 kernels: 128 x 128 and 128 x 64; the
-      // persistent kernel's list is ordered longest group first (more K
-      // chunks), so the long tiles start in the first wave
-      std::vector<GTile> tiles, tp;
-      std::vector<int> chunks(g.host.groups.size(), 0);
-      for (size_t gi = 0; gi < g.host.groups.size(); ++gi) {
-        const GGroup& gg = g.host.groups[gi];
-        for (int si = gg.seg0; si < gg.seg1; ++si) chunks[gi] += (g.host.segs[si].K + 63) / 64;
-        for (int m0 = 0; m0 < gg.M; m0 += 128) {
-          for (int n0 = 0; n0 < gg.N; n0 += 128) tiles.push_back(GTile{(int)gi, m0, n0, 0});
-          for (int n0 = 0; n0 < gg.N; n0 += 64) tp.push_back(GTile{(int)gi, m0, n0, 0});
-        }
-      }
-      std::stable_sort(tp.begin(), tp.end(), [&](const GTile& a, const GTile& b2) { return chunks[a.g] > chunks[b2.g]; });
-      ensure(c, g.tiles128, tiles.size() * sizeof(GTile) + 16);
-      ensure(c, g.tilesp, tp.size() * sizeof(GTile) + 16);
-      if (!tiles.empty())
-        CK(cudaMemcpyAsync(g.tiles128.p, tiles.data(), tiles.size() * sizeof(GTile), cudaMemcpyHostToDevice, st));
-      if (!tp.empty()) CK(cudaMemcpyAsync(g.tilesp.p, tp.data(), tp.size() * sizeof(GTile), cudaMemcpyHostToDevice, st));
-      g.ntiles128 = (int)tiles.size();
-      g.ntilesp = (int)tp.size();
     }
     if (!g.tc_ok) return false;
     // the maps depend only on the slots the A and B operands live in
@@ -694,7 +704,7 @@ struct Eng {
     bool same = true;
     for (int i = 0; i < 8; ++i)
       if (used & (1u << i)) same = same && g.key_p[i] == b.p[i] && g.key_lo[i] == b.lo[i];
-    if (same && g.maps.p) return true;
+    if (same && g.tcbuf.p) return true;
     // a captured step must replay the uploads of the uncaptured one
     if (r->capturing) throw Err{TT_ERR_STATE, "tensor-map operands moved during graph capture"};
     // looked up once per process (thread-safe static initialisation)
@@ -721,6 +731,7 @@ struct Eng {
       const GSeg& sg = g.host.segs[si];
       const GGroup& gg = g.host.groups[seg_group[si]];
       for (int w = 0; w < 3; ++w) {  // A (box 64 x 128), B (64 x 128), B (64 x 64)
+        if (w == 1 && r->exact) continue;  // (the digit kernel takes B by 64 rows)
         const Ref ref = w == 0 ? sg.A : sg.B;
         const int sl = (int)(ref >> 56);
         const int64_t off = (int64_t)(ref & 0x00FFFFFFFFFFFFFFull);
@@ -744,15 +755,39 @@ struct Eng {
         }
       }
     }
-    ensure(c, g.maps, maps.size() * sizeof(CUtensorMap) + 128);
-    CK(cudaMemcpyAsync(g.maps.p, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice, st));
-    CK(cudaStreamSynchronize(st));
+    // tile lists of the tcgen05 kernels, 128 x 128 and 128 x 64 (the digit kernel
+    // runs on the second only); the persistent kernels' list is ordered longest
+    // group first (more K chunks), so the long tiles start in the first wave
+    std::vector<GTile> tiles, tp;
+    std::vector<std::pair<int, int>> order;
+    for (size_t gi = 0; gi < g.host.groups.size(); ++gi) {
+      const GGroup& gg = g.host.groups[gi];
+      int chunks = 0;
+      for (int si = gg.seg0; si < gg.seg1; ++si) chunks += (g.host.segs[si].K + 63) / 64;
+      order.push_back({-chunks, (int)gi});
+      if (!r->exact)
+        for (int m0 = 0; m0 < gg.M; m0 += 128)
+          for (int n0 = 0; n0 < gg.N; n0 += 128) tiles.push_back(GTile{(int)gi, m0, n0, 0});
+    }
+    std::stable_sort(order.begin(), order.end());
+    for (auto& og : order) {
+      const GGroup& gg = g.host.groups[og.second];
+      for (int m0 = 0; m0 < gg.M; m0 += 128)
+        for (int n0 = 0; n0 < gg.N; n0 += 64) tp.push_back(GTile{og.second, m0, n0, 0});
+    }
+    Stager s;
+    s.add(maps, (CUtensorMap**)&g.maps);
+    s.add(tiles, &g.tiles128);
+    s.add(tp, &g.tilesp);
+    s.commit(c, g.tcbuf);
+    g.ntiles128 = (int)tiles.size();
+    g.ntilesp = (int)tp.size();
     for (int i = 0; i < 8; ++i) { g.key_p[i] = b.p[i]; g.key_lo[i] = b.lo[i]; }
     return true;
   }
 
-  // FP64 launch of a plan; its tile list is built and uploaded the first time
-  // (in the uncaptured step, as for the tensor maps)
+  // FP64 launch of a plan; the tile lists are built and uploaded when first
+  // needed (in the uncaptured step, as for the tensor maps)
   void f64(DevGemmBuf& g, const Bases& b) {
     if (g.d.tf == 0) {
       if (r->capturing) throw Err{TT_ERR_STATE, "FP64 tile list missing during graph capture"};
@@ -760,13 +795,24 @@ struct Eng {
       g.d.tf = sh.T;
       g.d.wkf = sh.wk;
       const std::vector<FTile> t = f64_tiles(g.host, g.d.tf);
-      ensure(c, g.tilesf, t.size() * sizeof(FTile) + 16);
-      if (!t.empty()) CK(cudaMemcpyAsync(g.tilesf.p, t.data(), t.size() * sizeof(FTile), cudaMemcpyHostToDevice, st));
-      CK(cudaStreamSynchronize(st));
-      g.d.tilesf = (FTile*)g.tilesf.p;
+      Stager s;
+      s.add(t, &g.d.tilesf);
+      s.commit(c, g.tilesf);
       g.d.ntilesf = (int)t.size();
     }
     CK(launch_gemm_f64(g.d, b, st));
+  }
+  // the plan with its list of 64 x 64 tiles (the mma.sync and double-float kernels)
+  const DevGemm& with64(DevGemmBuf& g) {
+    if (g.d.ntiles64 < 0) {
+      if (r->capturing) throw Err{TT_ERR_STATE, "64 x 64 tile list missing during graph capture"};
+      const std::vector<GTile> t = tiles64_of(g.host);
+      Stager s;
+      s.add(t, &g.d.tiles64);
+      s.commit(c, g.tiles64);
+      g.d.ntiles64 = (int)t.size();
+    }
+    return g.d;
   }
 
   // one launch of a split-BF16 plan on kernel k (tcgen05 kernels need prep_tc)
@@ -776,13 +822,13 @@ struct Eng {
       CK(cudaMemsetAsync(r->tcerr.p, 0, 16, st));
     }
     if (k == TK_TC128)
-      CK(launch_gemm_tc(g.d.groups, g.d.segs, (const GTile*)g.tiles128.p, g.ntiles128, g.maps.p, b, r->nsplit,
+      CK(launch_gemm_tc(g.d.groups, g.d.segs, g.tiles128, g.ntiles128, g.maps, b, r->nsplit,
                         (int*)r->tcerr.p, c->wait_ns, st));
     else if (k == TK_TCP128X64)
-      CK(launch_gemm_tcp(g.d.groups, g.d.segs, (const GTile*)g.tilesp.p, g.ntilesp, g.maps.p, b, r->nsplit,
+      CK(launch_gemm_tcp(g.d.groups, g.d.segs, g.tilesp, g.ntilesp, g.maps, b, r->nsplit,
                          (int*)r->tcerr.p, c->wait_ns, st));
     else
-      CK(launch_gemm_bf16(g.d, b, r->nsplit, st));
+      CK(launch_gemm_bf16(with64(g), b, r->nsplit, st));
   }
 
   // Tile-shape autotuner: the first uncaptured launch of a split-BF16 plan
@@ -875,7 +921,7 @@ struct Eng {
         if (((gg.flags & 2) != 0) != pair) throw Err{TT_ERR_STATE, "exact split: mixed output forms in one GEMM plan"};
       const long e = prof_begin(kind, g.d.flops);
       const int split = split_tiles(g);
-      CK(launch_gemm_tcz(g.d.groups, g.d.segs, (const GTile*)g.tilesp.p, g.ntilesp, split, tc_box(g), g.maps.p, b, r->zscr.p,
+      CK(launch_gemm_tcz(g.d.groups, g.d.segs, g.tilesp, g.ntilesp, split, tc_box(g), g.maps, b, r->zscr.p,
                          (unsigned*)r->ztick.p, (int*)r->tcerr.p, c->wait_ns, pair, st));
       prof_end(e);
       count();
@@ -892,9 +938,9 @@ struct Eng {
     if (use_mixed) {
       launch_split(g, b, g.choice);
     } else if (f64_kernel == 1) {
-      CK(launch_gemm_oz(g.d, b, st));
+      CK(launch_gemm_oz(with64(g), b, st));
     } else if (f64_kernel == 2) {
-      CK(launch_gemm_df(g.d, b, st));
+      CK(launch_gemm_df(with64(g), b, st));
     } else {
       f64(g, b);
     }
@@ -980,7 +1026,7 @@ struct Eng {
     need(r->T1, std::max(s.h.t1_size, s.h.u1_size) * 8, "T1");
     need(r->T2, std::max(s.h.t2_size, s.h.u2_size) * 8, "T2");
     need(r->W, s.h.lay.size * 8, "W");
-    need(r->Xn, s.h.lay.size * 2 * std::max(r->nsplit, 1), "Xn");
+    if (!r->apply_only) need(r->Xn, s.h.lay.size * 2 * std::max(r->nsplit, 1), "Xn");
     if (r->ldq < s.h.lay.size) throw Err{TT_ERR_STATE, "Krylov capacity"};
   }
 
@@ -1172,7 +1218,7 @@ struct Eng {
   }
   void run_qr_inner(QrDev& q, const Bases& b) {
     if (!r->use_cholqr) {
-      CK(launch_qr((const QrJob*)q.jobs.p, (int)q.h.jobs.size(), dptr(r->ws), st));
+      CK(launch_qr(q.jobs, (int)q.h.jobs.size(), dptr(r->ws), st));
       count();
       return;
     }
@@ -1184,7 +1230,7 @@ struct Eng {
       e = prof_begin(12, 0);
       // the mixed modes factorise in double-float (their error budget is far
       // above ~2^-46), FP64 mode in FP64
-      CK(launch_chol_inv((const CholJob*)q.cjobs[p].p, q.ncj[p], dptr(r->ws), (int*)q.fail.p, st, q.maxn[p], mixed()));
+      CK(launch_chol_inv(q.cjobs[p], q.ncj[p], dptr(r->ws), (int*)q.fail.p, st, q.maxn[p], mixed()));
       prof_end(e);
       e = prof_begin(11, q.app[p].d.flops);
       f64(q.app[p], b);
@@ -1201,7 +1247,7 @@ struct Eng {
       CK(cudaMemsetAsync(r->qrfb.p, 0, 16, st));
     }
     r->qr_sectors_acc += (long long)q.h.jobs.size();
-    CK(launch_qr_masked((const QrJob*)q.jobs.p, (int)q.h.jobs.size(), dptr(r->ws), (const int*)q.fail.p,
+    CK(launch_qr_masked(q.jobs, (int)q.h.jobs.size(), dptr(r->ws), (const int*)q.fail.p,
                         (int*)r->qrfb.p, st));
     count();
   }
@@ -1844,8 +1890,8 @@ struct Eng {
     }
     check_plan(t, caps({{S_AUX, el.size}, {S_X, S.size}, {S_T1, S.size}}), "measure T");
     check_plan(e, caps({{S_X, S.size}, {S_T1, S.size}, {S_AUX2, md.next.size}}), "measure EL");
-    upload(c, t, md.t);
-    upload(c, e, md.el);
+    upload_f64(std::move(t), md.t);
+    upload_f64(std::move(e), md.el);
     std::vector<ObsItem> items;
     for (const SiteBlock& b : S.blk) {
       ObsItem it{};
@@ -2210,15 +2256,21 @@ struct Eng {
   void two_site_exp(int j, const SiteLayout& C2, DBuf& Cbuf, double t) {
     const Mpo& m = M();
     MpoSite w12 = combine_two_sites(m, j, r->mpo->ls2);
-    SitePlanHost h = build_site_plan(r->bond[j], r->bond[j + 2], r->mpo->ls2, w12.terms, m.chan[j], m.chan[j + 2], mixed());
+    SitePlanHost h = build_site_plan(r->bond[j], r->bond[j + 2], r->mpo->ls2, w12.terms, m.chan[j], m.chan[j + 2], mixed(),
+                                     false, SP_APPLY);
     validate_site(h, r->bond[j], r->bond[j + 2], m.chan[j], m.chan[j + 2], mixed());
     DevGemmBuf s1, s3;
     DevGatherBuf s2;
     DevCopyBuf xs;
-    upload(c, h.s1, s1);
-    upload(c, h.s2, s2);
-    upload(c, h.s3, s3);
-    upload(c, h.xsplit, xs);
+    DBuf arena;
+    {
+      Stager g;
+      upload(g, std::move(h.s1), s1, !mixed());
+      upload(g, h.s2, s2);
+      upload(g, std::move(h.s3), s3, !mixed());
+      upload(g, h.xsplit, xs);
+      g.commit(c, arena);
+    }
     if (mixed()) ensure(c, r->Xs, (size_t)std::max<int64_t>(h.xt_size, 1) * 2 * r->nsplit);
     ensure(c, r->T1, (size_t)std::max<int64_t>(h.t1_size, 1) * 8);
     ensure(c, r->T2, (size_t)std::max<int64_t>(h.t2_size, 1) * 8);
@@ -2245,9 +2297,9 @@ struct Eng {
         b.p[S_L] = r->Lsp[j].p; b.lo[S_L] = r->Lpsize[j];
         b.p[S_R] = r->Rsp[j + 2].p; b.lo[S_R] = r->Rpsize[j + 2];
         b.lo[S_T2] = h.t2_size;
-        CK(launch_gemm_bf16(s1.d, b, r->nsplit, st));
+        CK(launch_gemm_bf16(with64(s1), b, r->nsplit, st));
         CK(launch_gather(s2.d, b, 1, r->nsplit, st));
-        CK(launch_gemm_bf16(s3.d, b, r->nsplit, st));
+        CK(launch_gemm_bf16(with64(s3), b, r->nsplit, st));
       } else {
         b.p[S_X] = (void*)x;
         b.p[S_L] = r->L[j].p;
@@ -2263,6 +2315,7 @@ struct Eng {
     release(c, s2);
     release(c, s3);
     release(c, xs);
+    dfree(c, arena);
   }
 
   void grow_sweep_lr(double tau) {
@@ -2378,6 +2431,7 @@ void alloc_rho_arrays(tt_rho* r) {
   r->absl_ok.assign(N, 0);
   r->absr_ok.assign(N, 0);
   r->meas.assign(N, MeasDev());
+  if (r->apply_only) return;
   tt_ctx* c = r->ctx;
   ensure(c, r->partial, (size_t)lanczos_nblk() * 17 * 8);
   ensure(c, r->ks, sizeof(KrylovState));
@@ -2394,17 +2448,17 @@ void free_rho(tt_rho* r) {
   for (auto* v : {&r->sp, &r->sp64})
     for (auto& s : *v) {
       release(c, s.s1); release(c, s.s2); release(c, s.s3); release(c, s.s3l); release(c, s.r1); release(c, s.r2);
-      release(c, s.r3); release(c, s.xs); release(c, s.xd);
+      release(c, s.r3); release(c, s.xs); release(c, s.xd); dfree(c, s.arena);
     }
   for (auto& e : r->esplit) release(c, e);
   for (auto& e : r->edig) release(c, e);
   for (auto& s : r->bp) {
-    release(c, s.b1); release(c, s.b2); release(c, s.xs); release(c, s.ts); release(c, s.xd); release(c, s.td);
+    release(c, s.b1); release(c, s.b2); release(c, s.xs); release(c, s.ts); release(c, s.xd); release(c, s.td); dfree(c, s.arena);
   }
   for (auto* v : {&r->qrl, &r->lqr})
     for (auto& q : *v) {
-      dfree(c, q.jobs); release(c, q.gather); release(c, q.scatter); release(c, q.rout);
-      for (int p = 0; p < 3; ++p) { release(c, q.gram[p]); release(c, q.app[p]); dfree(c, q.cjobs[p]); }
+      dfree(c, q.arena); release(c, q.gather); release(c, q.scatter); release(c, q.rout);
+      for (int p = 0; p < 3; ++p) { release(c, q.gram[p]); release(c, q.app[p]); }
       release(c, q.tt); release(c, q.rf); dfree(c, q.fail);
     }
   for (auto& g : r->absl) release(c, g);
@@ -2890,6 +2944,7 @@ static tt_status heff_apply_impl(tt_ctx* ctx, const tt_mpo* mpo, int site, int p
   r->N = mpo->mpo.N;
   r->nsplit = (precision == 1) ? 2 : (precision == 2 ? 3 : (precision == 3 ? 4 : 0));
   r->exact = precision == 3;
+  r->apply_only = true;
   tt_status s = guarded(ctx, nullptr, [&] {
     alloc_rho_arrays(r);
     r->bond.assign(r->N + 1, Bond());

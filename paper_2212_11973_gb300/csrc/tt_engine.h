@@ -55,8 +55,10 @@ struct DevGemmBuf {
   bool checked = false;
   // tcgen05 path: eligibility, 128 x 128 tile list, per-segment tensor maps
   bool tc_checked = false, tc_ok = false;
-  DBuf maps, tiles128, tilesp;
-  DBuf tilesf;  // FP64 kernel's tiles (built for its first launch)
+  DBuf tcbuf;  // tensor maps and both tile lists
+  void* maps = nullptr;
+  GTile *tiles128 = nullptr, *tilesp = nullptr;
+  DBuf tilesf, tiles64;  // tile lists of the FP64 and the 64 x 64 kernels, where not uploaded with the plan
   int ntiles128 = 0, ntilesp = 0;  // 128 x 128 tiles (tc), 128 x 64 tiles (persistent tc)
   // autotuned kernel of a split-BF16 plan: -1 not chosen yet, else a TcKernel
   int choice = -1;
@@ -68,15 +70,11 @@ enum TcKernel { TK_TC128 = 0, TK_TCP128X64 = 1, TK_MMA64 = 2, TK_N = 3 };
 
 struct DevGatherBuf {
   DevGather d;
-  DBuf buf;
-  GatherPlan host;
-  bool checked = false;
+  DBuf buf;  // a plan uploaded by itself
 };
 struct DevCopyBuf {
   DevCopy d;
   DBuf buf;
-  CopyPlan host;
-  bool checked = false;
 };
 
 // Element capacity of every slot (per split level for split-BF16 slots);
@@ -91,9 +89,6 @@ void check_plan(const CopyPlan& p, const Caps& c, const char* what);
 void check_exps(const GemmPlan& p, const Caps& ex, const char* what);
 void check_plan(const DigitPlan& p, const Caps& c, const Caps& ex, const char* what);
 
-void upload(tt_ctx* c, const GemmPlan& p, DevGemmBuf& o);
-void upload(tt_ctx* c, const GatherPlan& p, DevGatherBuf& o);
-void upload(tt_ctx* c, const CopyPlan& p, DevCopyBuf& o);
 void release(tt_ctx* c, DevGemmBuf& o);
 void release(tt_ctx* c, DevGatherBuf& o);
 void release(tt_ctx* c, DevCopyBuf& o);
@@ -101,9 +96,7 @@ void release(tt_ctx* c, DevCopyBuf& o);
 struct DevDigitBuf {
   DevDigit d;
   DBuf buf;
-  DigitPlan host;
 };
-void upload(tt_ctx* c, const DigitPlan& p, DevDigitBuf& o);
 void release(tt_ctx* c, DevDigitBuf& o);
 
 struct SiteDev {
@@ -113,6 +106,7 @@ struct SiteDev {
   DevGatherBuf s2, r2;
   DevCopyBuf xs;  // split-bf16 mode: x -> transposed padded copy (S1's B operand)
   DevDigitBuf xd; // exact mode: the same as digits
+  DBuf arena;     // the plans' arrays
 };
 struct BondDev {
   bool valid = false;
@@ -120,15 +114,18 @@ struct BondDev {
   DevGemmBuf b1, b2;
   DevCopyBuf xs, ts;  // mixed precision: padded split copies of x and T
   DevDigitBuf xd, td; // exact mode: digit copies of x and T
+  DBuf arena;
 };
 struct QrDev {
   bool valid = false;
   QrPlanHost h;
-  DBuf jobs;
+  DBuf arena;
+  QrJob* jobs = nullptr;
   DevCopyBuf gather, scatter, rout;
   // shifted CholeskyQR3 (FP64 GEMMs on all SMs) with Householder fallback
   DevGemmBuf gram[3], app[3], tt, rf;
-  DBuf cjobs[3], fail;
+  CholJob* cjobs[3] = {nullptr, nullptr, nullptr};
+  DBuf fail;
   int ncj[3] = {0, 0, 0};
   int maxn[3] = {0, 0, 0};  // largest sector (columns) of each pass's Cholesky jobs
 };
@@ -160,6 +157,7 @@ struct tt_rho {
   std::vector<tt::DevCopyBuf> esplit;     // per bond: FP64 environment -> padded split copy
   std::vector<tt::DevDigitBuf> edig;      // per bond: FP64 environment -> digits (exact mode)
   std::vector<char> esplit_ok;
+  bool apply_only = false;                // a single H_eff apply: no sweep buffers or plans
   bool use_tc = true;                     // tcgen05 kernel for eligible split-bf16 GEMMs
   bool use_cholqr = true;                 // CholeskyQR3 gauge (else Householder only)
   std::vector<tt::SiteDev> sp;

@@ -22,13 +22,14 @@
 namespace tt {
 
 namespace {
-// (wr, sig) -> terms ; (wl, sig) -> terms
+// terms by (wr, sig) and by (wl, sig): index w * d + sig
 struct TermIndex {
-  std::map<std::pair<int, int>, std::vector<const MpoTerm*>> by_r, by_l;
-  explicit TermIndex(const std::vector<MpoTerm>& t) {
+  std::vector<std::vector<const MpoTerm*>> by_r, by_l;
+  TermIndex(const std::vector<MpoTerm>& t, int nwl, int nwr, int d)
+      : by_r((size_t)nwr * d), by_l((size_t)nwl * d) {
     for (const auto& x : t) {
-      by_r[{x.wr, x.sig}].push_back(&x);
-      by_l[{x.wl, x.sig}].push_back(&x);
+      by_r[(size_t)x.wr * d + x.sig].push_back(&x);
+      by_l[(size_t)x.wl * d + x.sig].push_back(&x);
     }
   }
 };
@@ -45,7 +46,8 @@ std::vector<int64_t> env_row_starts(const EnvLayout& E) {
 }
 
 SitePlanHost build_site_plan(const Bond& BL, const Bond& BR, const LocalSpace& ls, const std::vector<MpoTerm>& terms,
-                             const std::vector<Q>& chl, const std::vector<Q>& chr, bool mixed, bool exact) {
+                             const std::vector<Q>& chl, const std::vector<Q>& chr, bool mixed, bool exact,
+                             unsigned parts) {
   exact = exact && mixed;
   SitePlanHost P;
   P.lay = make_site_layout(BL, BR, ls);
@@ -59,8 +61,8 @@ SitePlanHost build_site_plan(const Bond& BL, const Bond& BR, const LocalSpace& l
   auto wpad = [&](int x) { return mixed ? pad8i(x) : x; };
   const int nwl = (int)chl.size(), nwr = (int)chr.size();
   const int t1flag = mixed ? 2 : 0;
-  TermIndex ti(terms);
   const int d = ls.d;
+  const TermIndex ti(terms, nwl, nwr, d);
 
   // ---- S1 (mixed: B = transposed x block [(s, a_r)][a_l], rows padded: K-major)
   std::vector<int64_t> t1off(S.blk.size(), -1), t1ld(S.blk.size(), 0), xtoff(S.blk.size(), 0), xtrow(S.blk.size(), 0);
@@ -146,9 +148,8 @@ SitePlanHost build_site_plan(const Bond& BL, const Bond& BR, const LocalSpace& l
         it.rows = ob.dl;
         it.cols = BR.dim[br];
         it.c0 = (int)P.s2.contribs.size();
-        auto f = ti.by_r.find({w2, sig});
-        if (f != ti.by_r.end())
-          for (const MpoTerm* t : f->second) {
+        {
+          for (const MpoTerm* t : ti.by_r[(size_t)w2 * d + sig]) {
             const int w = t->wl, tau = t->tau;
             int lb = BL.find(BL.q[ob.l] - chl[w]);
             if (lb < 0) continue;
@@ -165,6 +166,7 @@ SitePlanHost build_site_plan(const Bond& BL, const Bond& BR, const LocalSpace& l
             c.coef = t->v;
             P.s2.contribs.push_back(c);
           }
+        }
         it.c1 = (int)P.s2.contribs.size();
         if (exact) {
           it.e = mkref(S_T2, t2x + t2e[r] + (ob.grp_row + so) * nseg[r] + t2seg[(size_t)r * nwr + w2]);
@@ -178,7 +180,7 @@ SitePlanHost build_site_plan(const Bond& BL, const Bond& BR, const LocalSpace& l
 
   // ---- S3 (H_eff output) and S3L (left environment update)
   for (int r = 0; r < nr; ++r) {
-    if (S.grp_rows[r] > 0) {
+    if (S.grp_rows[r] > 0 && (parts & SP_APPLY)) {
       P.s3.add_group((int)S.grp_rows[r], BR.dim[r], mkref(S_Y, S.grp_off[r]), BR.dim[r], 0);
       for (int w2 = 0; w2 < nwr; ++w2) {
         int64_t col = t2col[(size_t)r * nwr + w2];
@@ -192,7 +194,7 @@ SitePlanHost build_site_plan(const Bond& BL, const Bond& BR, const LocalSpace& l
                         mkref(S_R, ere + errow[b] + rrow), 1);
       }
     }
-    for (int w2 = 0; w2 < nwr; ++w2) {
+    for (int w2 = 0; w2 < nwr && (parts & SP_ENVL); ++w2) {
       int64_t col = t2col[(size_t)r * nwr + w2];
       if (col < 0) continue;
       const int b = t2ket[(size_t)r * nwr + w2];
@@ -204,6 +206,8 @@ SitePlanHost build_site_plan(const Bond& BL, const Bond& BR, const LocalSpace& l
     }
   }
   P.lenv_size = ER.size;
+  P.renv_size = EL.size;
+  if (!(parts & SP_ENVR)) return P;
 
   // ---- R1
   std::vector<int64_t> u1off(S.blk.size(), -1), u1ld(S.blk.size(), 0);
@@ -268,9 +272,8 @@ SitePlanHost build_site_plan(const Bond& BL, const Bond& BR, const LocalSpace& l
           it.rows = BL.dim[lb];
           it.cols = ob.dr;
           it.c0 = (int)P.r2.contribs.size();
-          auto f = ti.by_l.find({w, sig});
-          if (f != ti.by_l.end())
-            for (const MpoTerm* t : f->second) {
+          {
+            for (const MpoTerm* t : ti.by_l[(size_t)w * d + sig]) {
               const int w2 = t->wr, tau = t->tau;
               const int pidx = tau * d + sgp;
               const int pin = ls.sec_of[pidx], si = ls.pos_of[pidx];
@@ -286,6 +289,7 @@ SitePlanHost build_site_plan(const Bond& BL, const Bond& BR, const LocalSpace& l
               c.coef = t->v;
               P.r2.contribs.push_back(c);
             }
+          }
           it.c1 = (int)P.r2.contribs.size();
           P.r2.items.push_back(it);
           P.r2.elems += (double)it.rows * it.cols * (1 + it.c1 - it.c0);
@@ -310,7 +314,6 @@ SitePlanHost build_site_plan(const Bond& BL, const Bond& BR, const LocalSpace& l
                      mkref(S_T2, u2off[a] + row0 * u2cols[a] + colseg[(size_t)a * S.npq + p]), (int)u2cols[a], 1, K);
       }
     }
-  P.renv_size = EL.size;
   return P;
 }
 

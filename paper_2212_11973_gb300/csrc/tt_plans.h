@@ -60,8 +60,12 @@ CholQrPlan build_cholqr(const std::vector<QrJob>& jobs, int64_t ws0);
 // exact (with mixed): the split-BF16 layouts carry fixed-point digits; the
 // GEMM segments get the operands' row exponents, the gather items the output
 // exponents, S1 writes two-float pairs.
+// parts: the H_eff apply (S1, S2, S3), the left environment update (S1, S2, S3L)
+// and the right one (R1, R2, R3).
+enum : unsigned { SP_APPLY = 1, SP_ENVL = 2, SP_ENVR = 4, SP_ALL = 7 };
 SitePlanHost build_site_plan(const Bond& BL, const Bond& BR, const LocalSpace& ls, const std::vector<MpoTerm>& terms,
-                             const std::vector<Q>& chl, const std::vector<Q>& chr, bool mixed, bool exact = false);
+                             const std::vector<Q>& chl, const std::vector<Q>& chr, bool mixed, bool exact = false,
+                             unsigned parts = SP_ALL);
 BondPlanHost build_bond_plan(const Bond& B, const std::vector<Q>& ch, bool mixed, bool exact = false);
 GemmPlan build_absorb_left(const SiteLayout& oldl, const SiteLayout& newl, const Bond& Bold, const Bond& Bnew,
                            const std::vector<int64_t>& soff, const std::vector<int>& new_of_old);
