@@ -173,18 +173,23 @@ static void upload(Stager& s, const GatherPlan& p, DevGatherBuf& o) {
 }
 
 static void upload(Stager& s, const CopyPlan& p, DevCopyBuf& o) {
+  std::vector<CPart> parts;
+  for (size_t i = 0; i < p.items.size(); ++i) {
+    const int64_t n = (int64_t)((p.items[i].rows + 31) / 32) * ((p.items[i].cols + 31) / 32);
+    for (int64_t t = 0; t < n; t += COPY_TILES) parts.push_back(CPart{(int)i, (int)t});
+  }
   s.add(p.items, &o.d.items);
-  o.d.nitems = (int)p.items.size();
-  o.d.maxtiles = 0;
-  for (const CItem& it : p.items)
-    o.d.maxtiles = std::max<int64_t>(o.d.maxtiles, (int64_t)((it.rows + 31) / 32) * ((it.cols + 31) / 32));
+  s.add(parts, &o.d.parts);
+  o.d.nparts = (int)parts.size();
 }
 
 static void upload(Stager& s, const DigitPlan& p, DevDigitBuf& o) {
+  std::vector<CPart> parts;
+  for (size_t i = 0; i < p.items.size(); ++i)
+    for (int r0 = 0; r0 < p.items[i].rows; r0 += 32) parts.push_back(CPart{(int)i, r0});
   s.add(p.items, &o.d.items);
-  o.d.nitems = (int)p.items.size();
-  o.d.maxgroups = 0;
-  for (const DItem& it : p.items) o.d.maxgroups = std::max(o.d.maxgroups, (it.rows + 31) / 32);
+  s.add(parts, &o.d.parts);
+  o.d.nparts = (int)parts.size();
 }
 
 // one plan by itself

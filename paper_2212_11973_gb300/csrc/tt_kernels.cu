@@ -365,23 +365,25 @@ __global__ void __launch_bounds__(256) gather_kernel(const GItem* __restrict__ i
 }
 
 // Strided 2-D copies, one item = rows x cols elements with arbitrary row and
-// column strides on both sides.  The item is cut into 32 x 32 tiles; the
-// CTAs of grid row blockIdx.x share item blockIdx.x's tiles (stride
-// gridDim.y).  A tile goes through shared memory so that both the load and
-// the store run along whichever side has unit stride (a transposing copy is
-// coalesced on both ends).  NS = 0: FP64 -> FP64; NS = 2, 3: FP64 -> split
+// column strides on both sides.  The items are cut into 32 x 32 tiles, a CTA
+// takes COPY_TILES of them (a list made with the plan: sized by the largest item,
+// most CTAs of a grid had nothing to do, 12 us for 1 MB).  A tile goes through
+// shared memory so that both the load and the store run along whichever side
+// has unit stride (a transposing copy is coalesced on both ends).  NS = 0: FP64 -> FP64; NS = 2, 3: FP64 -> split
 // bf16 levels at dst + l * lo[slot(dst)].
 template <int NS>
-__global__ void __launch_bounds__(256) tile_copy_kernel(const CItem* __restrict__ items, Bases bs) {
+__global__ void __launch_bounds__(256) tile_copy_kernel(const CItem* __restrict__ items, const CPart* __restrict__ parts,
+                                                        Bases bs) {
   __shared__ double tile[32][33];
-  const CItem it = items[blockIdx.x];
+  const CPart part = parts[blockIdx.x];
+  const CItem it = items[part.item];
   const double* src = rptr<const double>(bs, it.src);
   const int tcr = (it.rows + 31) >> 5, tcc = (it.cols + 31) >> 5;
   const int ntiles = tcr * tcc;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 8
   const bool src_rmaj = it.src_cs == 1 || it.src_rs != 1;   // src contiguous along c
   const bool dst_rmaj = it.dst_cs == 1 || it.dst_rs != 1;
-  for (int t = blockIdx.y; t < ntiles; t += gridDim.y) {
+  for (int t = part.first; t < min(ntiles, part.first + COPY_TILES); ++t) {
     const int r0 = (t / tcc) << 5, c0 = (t % tcc) << 5;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -408,12 +410,6 @@ __global__ void __launch_bounds__(256) tile_copy_kernel(const CItem* __restrict_
     }
     __syncthreads();
   }
-}
-
-static dim3 copy_grid(const DevCopy& c) {
-  // enough CTAs per item for about four tiles each, at most 256 per item
-  const int y = std::max(1, std::min(256, (c.maxtiles + 3) / 4));
-  return dim3((unsigned)c.nitems, (unsigned)y);
 }
 
 // x (FP64, n) -> ns bf16 levels out[l * n + i], x ~ sum_l out[l].
@@ -674,8 +670,8 @@ cudaError_t launch_gather(const DevGather& g, const Bases& b, int in_type, int o
 }
 
 cudaError_t launch_copy(const DevCopy& c, const Bases& b, cudaStream_t s) {
-  if (c.nitems == 0) return cudaSuccess;
-  tile_copy_kernel<0><<<copy_grid(c), 256, 0, s>>>(c.items, b);
+  if (c.nparts == 0) return cudaSuccess;
+  tile_copy_kernel<0><<<c.nparts, 256, 0, s>>>(c.items, c.parts, b);
   return cudaGetLastError();
 }
 
@@ -688,9 +684,9 @@ cudaError_t launch_split_bf16(const double* x, int64_t n, int nsplit, void* out,
 cudaError_t launch_zero(void* p, size_t bytes, cudaStream_t s) { return cudaMemsetAsync(p, 0, bytes, s); }
 
 cudaError_t launch_split_copy(const DevCopy& c, const Bases& b, int nsplit, cudaStream_t s) {
-  if (c.nitems == 0) return cudaSuccess;
-  if (nsplit == 2) tile_copy_kernel<2><<<copy_grid(c), 256, 0, s>>>(c.items, b);
-  else if (nsplit == 3) tile_copy_kernel<3><<<copy_grid(c), 256, 0, s>>>(c.items, b);
+  if (c.nparts == 0) return cudaSuccess;
+  if (nsplit == 2) tile_copy_kernel<2><<<c.nparts, 256, 0, s>>>(c.items, c.parts, b);
+  else if (nsplit == 3) tile_copy_kernel<3><<<c.nparts, 256, 0, s>>>(c.items, c.parts, b);
   else return cudaErrorInvalidValue;
   return cudaGetLastError();
 }

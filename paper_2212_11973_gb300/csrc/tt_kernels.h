@@ -50,15 +50,21 @@ struct DevGather {
   int nitems = 0;
   double elems = 0;
 };
+// copies and digit copies: one CTA per part, an item and its first 32 x 32 tile
+// (of COPY_TILES) or digit row (of 32)
+struct CPart {
+  int item, first;
+};
+constexpr int COPY_TILES = 2;
 struct DevCopy {
   CItem* items = nullptr;
-  int nitems = 0;
-  int maxtiles = 0;  // largest item, in 32 x 32 tiles
+  CPart* parts = nullptr;
+  int nparts = 0;
 };
 struct DevDigit {
   DItem* items = nullptr;
-  int nitems = 0;
-  int maxgroups = 0;  // largest item, in groups of 32 digit rows
+  CPart* parts = nullptr;
+  int nparts = 0;
 };
 
 // Device-side Krylov bookkeeping of one Lanczos exponential.

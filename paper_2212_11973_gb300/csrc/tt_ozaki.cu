@@ -32,6 +32,7 @@
 
 #include <cstdint>
 
+#include "tt_fixed.h"
 #include "tt_kernels.h"
 
 namespace tt {
@@ -47,33 +48,6 @@ __device__ __forceinline__ long long off_of(Ref r) { return (long long)(r & 0x00
 
 __device__ __forceinline__ int biased_exp(double v) {
   return (int)((static_cast<unsigned long long>(__double_as_longlong(v)) >> 52) & 0x7FF);
-}
-
-// Balanced base-256 digits of F = round(v 2^(1054 - emax)) (emax: the largest
-// biased exponent of the row, so |v| < 2^(emax - 1022) and |F| <= 2^32).
-// Zero and subnormal v give F = 0.
-__device__ __forceinline__ void fixed_digits(double v, int emax, __nv_bfloat16* d0, long long stride) {
-  const unsigned long long bits = static_cast<unsigned long long>(__double_as_longlong(v));
-  const int E = (int)((bits >> 52) & 0x7FF);
-  long long F = 0;
-  if (E != 0) {
-    const unsigned long long M = (bits & 0xFFFFFFFFFFFFFull) | (1ull << 52);
-    const int sh = 21 + emax - E;  // >= 21
-    if (sh < 64) {
-      F = (long long)((M + (1ull << (sh - 1))) >> sh);
-      if (bits >> 63) F = -F;
-    }
-  }
-  const long long a0 = (F + (1ll << 23)) >> 24;  // floor division (arithmetic shift)
-  const long long r0 = F - a0 * (1ll << 24);     // [-2^23, 2^23)
-  const long long a1 = (r0 + (1ll << 15)) >> 16;
-  const long long r1 = r0 - a1 * (1ll << 16);    // [-2^15, 2^15)
-  const long long a2 = (r1 + (1ll << 7)) >> 8;
-  const long long a3 = r1 - a2 * (1ll << 8);     // [-128, 128)
-  d0[0] = __float2bfloat16_rn((float)a0);
-  d0[stride] = __float2bfloat16_rn((float)a1);
-  d0[2 * stride] = __float2bfloat16_rn((float)a2);
-  d0[3 * stride] = __float2bfloat16_rn((float)a3);
 }
 
 __device__ __forceinline__ void mma16816(float* c, const uint32_t* a, const uint32_t* b) {
@@ -172,8 +146,15 @@ __global__ void __launch_bounds__(OT) gemm_oz_kernel(const GGroup* __restrict__ 
 #pragma unroll
       for (int i = 0; i < OEL; ++i) {
         const int ra = tile_row(ka, tid, i), rb = tile_row(kb, tid, i);
-        fixed_digits(va[i], eA[ra], &As[0][ra][tile_k(ka, tid, i)], DS);
-        fixed_digits(vb[i], eB[rb], &Bs[0][rb][tile_k(kb, tid, i)], DS);
+        uint32_t d[ODIG];
+        fixed_digit_bits(va[i], eA[ra], d);
+#pragma unroll
+        for (int s = 0; s < ODIG; ++s)
+          (&As[0][ra][tile_k(ka, tid, i)])[s * DS] = __ushort_as_bfloat16((unsigned short)(d[s] >> 16));
+        fixed_digit_bits(vb[i], eB[rb], d);
+#pragma unroll
+        for (int s = 0; s < ODIG; ++s)
+          (&Bs[0][rb][tile_k(kb, tid, i)])[s * DS] = __ushort_as_bfloat16((unsigned short)(d[s] >> 16));
       }
       __syncthreads();
 #pragma unroll
