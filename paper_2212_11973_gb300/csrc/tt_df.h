@@ -38,4 +38,32 @@ __device__ __forceinline__ double dbl_of_float(float f) {
   return __longlong_as_double((long long)b);
 }
 
+// hi + lo as FP64 by integer operations (two conversions and an addition on the
+// FP64 pipe cost 192 clocks of an SM sub-partition per warp): renormalised by
+// TwoSum to |t| <= ulp(s) / 2, then the mantissas added, t's truncated at 2^-53 of
+// s.  Infinities and NaN pass through; FP32 subnormals give zero.
+__device__ __forceinline__ double dbl_of_pair(float hi, float lo) {
+  const float s = hi + lo;
+  const float bp = s - hi;
+  const float t = (hi - (s - bp)) + (lo - bp);
+  const unsigned us = __float_as_uint(s), ut = __float_as_uint(t);
+  int es = (us >> 23) & 0xFF;
+  const int et = (ut >> 23) & 0xFF;
+  const unsigned sign = us & 0x80000000u;
+  if (es == 0) return 0.0;
+  if (es == 255)
+    return __hiloint2double((int)(sign | 0x7FF00000u | ((us & 0x7FFFFFu) >> 3)), (int)(us << 29));
+  const unsigned mt = et ? (ut & 0x7FFFFFu) | 0x800000u : 0u;
+  const int sh = es - et - 29;  // >= -5
+  const unsigned T = sh >= 0 ? (sh < 32 ? mt >> sh : 0u) : mt << -sh;
+  unsigned long long m = (unsigned long long)((us & 0x7FFFFFu) | 0x800000u) << 29;
+  m = ((us ^ ut) >> 31) ? m - T : m + T;
+  if (!(m >> 52)) {  // s a power of two, t of the other sign
+    m <<= 1;
+    --es;
+  }
+  return __longlong_as_double((long long)(((unsigned long long)sign << 32) | ((unsigned long long)(es + 896) << 52) |
+                                          (m & 0xFFFFFFFFFFFFFull)));
+}
+
 }  // namespace tt

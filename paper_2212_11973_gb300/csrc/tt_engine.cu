@@ -681,12 +681,11 @@ struct Eng {
     else CK(cudaEventRecord(e, st));
   }
 
-  // K extent of the tensor maps' boxes: 64, or 32 for the digit kernel where no
-  // segment is longer than 64
+  // K extent of the persistent kernels' boxes: 32 where no segment is longer
+  // than 64 (digits) or 128 (split-BF16), else 64
   int tc_box(const DevGemmBuf& g) const {
-    if (!r->exact) return 64;
     for (const GSeg& sg : g.host.segs)
-      if (sg.K > 64) return 64;
+      if (sg.K > (r->exact ? 64 : 128)) return 64;
     return 32;
   }
 
@@ -728,33 +727,36 @@ struct Eng {
     }
     const int kbox = tc_box(g);
     const size_t nseg = g.host.segs.size();
-    std::vector<CUtensorMap> maps(3 * nseg);
+    std::vector<CUtensorMap> maps(4 * nseg);
     std::vector<int> seg_group(nseg, 0);
     for (size_t gi = 0; gi < g.host.groups.size(); ++gi)
       for (int si = g.host.groups[gi].seg0; si < g.host.groups[gi].seg1; ++si) seg_group[si] = (int)gi;
     for (size_t si = 0; si < nseg; ++si) {
       const GSeg& sg = g.host.segs[si];
       const GGroup& gg = g.host.groups[seg_group[si]];
-      for (int w = 0; w < 3; ++w) {  // A (box 64 x 128), B (64 x 128), B (64 x 64)
-        if (w == 1 && r->exact) continue;  // (the digit kernel takes B by 64 rows)
-        const Ref ref = w == 0 ? sg.A : sg.B;
+      // 0, 1: A and B boxes of 64 K x 128 rows (128 x 128 kernel); 2, 3: B box of
+      // kbox x 64 and A box of kbox x 128 (persistent kernels)
+      for (int w = r->exact ? 2 : 0; w < 4; ++w) {
+        const bool isA = w == 0 || w == 3;
+        const int bk = w < 2 ? 64 : kbox;
+        const Ref ref = isA ? sg.A : sg.B;
         const int sl = (int)(ref >> 56);
         const int64_t off = (int64_t)(ref & 0x00FFFFFFFFFFFFFFull);
         const long long lo = b.lo[sl];
         if (!b.p[sl] || lo % 8 || sg.K < 1) { g.tc_ok = false; return false; }
-        cuuint64_t dims[3] = {(cuuint64_t)sg.K, (cuuint64_t)std::max(1, w == 0 ? gg.M : gg.N), (cuuint64_t)r->nsplit};
-        cuuint64_t strides[2] = {(cuuint64_t)(w == 0 ? sg.lda : sg.ldb) * 2, (cuuint64_t)lo * 2};
-        cuuint32_t box[3] = {(cuuint32_t)kbox, (cuuint32_t)(w == 2 ? 64 : 128), 1};
+        cuuint64_t dims[3] = {(cuuint64_t)sg.K, (cuuint64_t)std::max(1, isA ? gg.M : gg.N), (cuuint64_t)r->nsplit};
+        cuuint64_t strides[2] = {(cuuint64_t)(isA ? sg.lda : sg.ldb) * 2, (cuuint64_t)lo * 2};
+        cuuint32_t box[3] = {(cuuint32_t)bk, (cuuint32_t)(w == 2 ? 64 : 128), 1};
         cuuint32_t estr[3] = {1, 1, 1};
         void* base = (char*)b.p[sl] + off * 2;
-        CUresult cr = encode(&maps[3 * si + w], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, base, dims, strides, box, estr,
+        CUresult cr = encode(&maps[4 * si + w], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, base, dims, strides, box, estr,
                              CU_TENSOR_MAP_INTERLEAVE_NONE,
-                             kbox == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+                             bk == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
                              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (cr != CUDA_SUCCESS) {
           if (std::getenv("TT_DEBUG"))
             std::fprintf(stderr, "[tc] tensor map encode failed (%d) seg %zu K %d ld %d lo %lld\n", (int)cr, si, sg.K,
-                         w == 0 ? sg.lda : sg.ldb, lo);
+                         isA ? sg.lda : sg.ldb, lo);
           g.tc_ok = false;
           return false;
         }
@@ -830,7 +832,8 @@ struct Eng {
       CK(launch_gemm_tc(g.d.groups, g.d.segs, g.tiles128, g.ntiles128, g.maps, b, r->nsplit,
                         (int*)r->tcerr.p, c->wait_ns, st));
     else if (k == TK_TCP128X64)
-      CK(launch_gemm_tcp(g.d.groups, g.d.segs, g.tilesp, g.ntilesp, g.maps, b, r->nsplit,
+      CK(launch_gemm_tcp(g.d.groups, g.d.segs, g.tilesp, g.ntilesp, split_tiles(g), tc_box(g), g.maps, b, r->nsplit,
+                         !g.host.groups.empty() && (g.host.groups[0].flags & 2), r->zscr.p, (unsigned*)r->ztick.p,
                          (int*)r->tcerr.p, c->wait_ns, st));
     else
       CK(launch_gemm_bf16(with64(g), b, r->nsplit, st));
@@ -892,7 +895,7 @@ struct Eng {
     return best;
   }
 
-  // CTAs that share a tile of the persistent digit kernel, with room for their
+  // CTAs that share a tile of a persistent tcgen05 kernel, with room for their
   // partial sums (allocated in the uncaptured step, like every buffer)
   int split_tiles(const DevGemmBuf& g) {
     int ms = 0;

@@ -114,16 +114,18 @@ cudaError_t launch_split_bf16(const double* x, int64_t n, int nsplit, void* out 
 cudaError_t launch_zero(void* p, size_t bytes, cudaStream_t s);
 // strided FP64 -> split-bf16 copy (levels at dst + l * lo[slot(dst)])
 cudaError_t launch_split_copy(const DevCopy& c, const Bases& b, int nsplit, cudaStream_t s);
-// tcgen05 grouped GEMM (tt_tcgen05.cu): K-major A and B, 128 x 128 tiles,
-// maps = 3 CUtensorMap per segment in global memory: A (box 64 K x 128 rows),
-// B (64 x 128), B (64 x 64).
+// tcgen05 grouped GEMM (tt_tcgen05.cu): K-major A and B, 128 x 128 tiles, maps =
+// 4 CUtensorMap per segment in global memory: A (box 64 K x 128 rows), B (64 x
+// 128), B (kbox x 64), A (kbox x 128).
 size_t tc_smem_bytes(int nsplit);
 // Persistent warp-specialised variant (tt_tcgen05p.cu): 128 x 64 tiles, one
 // CTA per SM, TMA ring / MMA warp / fold-and-epilogue warps, the same
 // arithmetic and maps.
-size_t tcp_smem_bytes(int nsplit);
-cudaError_t launch_gemm_tcp(const GGroup* groups, const GSeg* segs, const GTile* tiles128x64, int ntiles,
-                            const void* maps, const Bases& b, int nsplit, int* err, long long wait_ns, cudaStream_t s);
+// out32: every group writes FP32 (flags bit 1), else FP64; split, kbox, scratch
+// and tickets as for launch_gemm_tcz below.
+cudaError_t launch_gemm_tcp(const GGroup* groups, const GSeg* segs, const GTile* tiles128x64, int ntiles, int split,
+                            int kbox, const void* maps, const Bases& b, int nsplit, bool out32, void* scratch,
+                            unsigned* tickets, int* err, long long wait_ns, cudaStream_t s);
 // Exact-accumulation split GEMM on tcgen05 (tt_tcgen05z.cu): digit operands
 // (4 levels + int16 row exponents, GSeg.eA / eB), persistent 128 x 64 tiles,
 // maps with boxes of kbox = 64 (128-byte swizzle) or 32 (64-byte) K;

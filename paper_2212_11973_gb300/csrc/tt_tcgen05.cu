@@ -102,8 +102,8 @@ __global__ void __launch_bounds__(128, 1) gemm_tc_kernel(const GGroup* __restric
     while (cur_seg < g.seg1 && cur_k >= segs[cur_seg].K) { ++cur_seg; cur_k = 0; }
     const int s = c & 1;
     uint8_t* st = smem + s * STAGE_BYTES;
-    const CUtensorMap* ma = maps + 3 * cur_seg;
-    const CUtensorMap* mb = maps + 3 * cur_seg + 1;
+    const CUtensorMap* ma = maps + 4 * cur_seg;
+    const CUtensorMap* mb = maps + 4 * cur_seg + 1;
     if (fenced_seg != cur_seg) {  // tensor maps written by a host copy: acquire before first use
       asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(reinterpret_cast<uint64_t>(ma)) : "memory");
       asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(reinterpret_cast<uint64_t>(mb)) : "memory");

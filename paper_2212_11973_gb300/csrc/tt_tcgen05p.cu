@@ -1,33 +1,36 @@
 // Persistent, warp-specialised split-BF16 grouped GEMM on the 5th-generation
-// tensor cores (sm_103a): the same arithmetic as gemm_tc_kernel
-// (tt_tcgen05.cu: NS bf16 levels per operand, the level products l_A + l_B <
-// NS, the leading product in one TMEM accumulator and the smaller ones in a
-// second, folded every two 64-wide K chunks into a two-float TwoSum sum), laid
-// out for throughput:
+// tensor cores (sm_103a): operands as NS bf16 levels, the level products l_A +
+// l_B < NS, folded every 128 of K at most into a two-float TwoSum sum.
 //
-//  * one CTA per SM walks the 128 x 64 output tiles blockIdx.x, blockIdx.x +
-//    gridDim.x, ... so TMEM allocation and barrier set-up happen once;
-//  * warp 0 (one lane) streams the A (128 x 64 K) and B (64 x 64 K) level
-//    tiles by TMA into a ring of STAGES shared-memory stages, running ahead
-//    across fold groups and tiles;
-//  * warp 1 (one lane) issues tcgen05.mma (M = 128, N = 64, K = 16) into one
-//    of two TMEM accumulator buffers per fold group and commits each stage
-//    back to the producer and each buffer to the epilogue;
-//  * warps 2-5 fold a finished buffer into the two-float sum (TMEM, hi and lo)
-//    while the MMAs of the next fold group run in the other buffer, and write
-//    every finished tile's hi + lo (FP32 or FP64, optionally accumulated).
+// Laid out as the digit kernel (tt_tcgen05z.cu): one CTA per SM walks 128 x 64
+// output tiles; warp 0 streams the level tiles by TMA into a ring of
+// shared-memory stages (K chunks of 64, or of 32 where no segment is longer than
+// 128), warp 1 issues the MMAs, warps 2-9 fold a finished accumulator while the
+// next fold group's MMAs run in the other buffer, and write the tile's hi + lo
+// as FP32 or FP64 through a per-warp staging buffer.  The products of one order
+// d = l_A + l_B share an accumulator (D_0 .. D_{NS-1}, 64 TMEM columns each), so
+// level l of A meets the B levels 0 .. NS-1-l, which lie one after the other, in
+// one MMA of N = 64 (NS - l).  D_0 goes through TwoSum, the smaller orders into
+// lo.  Where a plan has fewer tiles than SMs, `split` CTAs share a tile's
+// segments and the last to arrive adds their sums in part order.
 //
-// TMEM (512 columns): buffer b at [128 b, 128 b + 128) (leading product,
-// smaller products), hi [256, 320), lo [320, 384).  Every wait is bounded by
-// wait_ns; a role whose wait runs out raises a shared abort flag that the
-// other roles' waits observe, the CTA records the error, drains its own TMA
-// copies and MMAs (fixed budget), frees its TMEM and returns.
+// What bounds it: the chain of segments (18 to 42 of K = 3 to 180) behind each
+// tile; see the digit kernel.  D = 512, all four launches of an H_eff and a bond
+// apply, average: 29 -> 24 us from one lane fencing and loading each segment's
+// maps, K chunks of 64 throughout, six MMAs per 16 K and rows stored as they came
+// (S1, whose tiles have one segment each and are bound by their output, 23 us; with
+// the shared-memory reads of the output one by one it took 40).
+//
+// Every wait is bounded by wait_ns; a role whose wait runs out raises a shared
+// abort flag that the other roles' waits observe, the CTA records the error,
+// drains its own TMA copies and MMAs (fixed budget), frees its TMEM and returns.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 #include <cstdint>
 
+#include "tt_df.h"
 #include "tt_kernels.h"
 #include "tt_tc_ptx.h"
 
@@ -37,62 +40,63 @@ namespace {
 
 using namespace tcx;
 
-constexpr int PBM = 128, PBN = 64, PBK = 64;
-constexpr int PA_BYTES = PBM * PBK * 2;  // 16 KB per level
-constexpr int PB_BYTES = PBN * PBK * 2;  // 8 KB per level
-constexpr int PFOLD = 2;
+constexpr int PBM = 128, PBN = 64, PFOLD_K = 128;
 constexpr uint32_t PTMEM_COLS = 512;
-constexpr int PTHREADS = 192;
+constexpr int PEPI = 8;  // epilogue warps
+constexpr int PTHREADS = 64 + 32 * PEPI;
+constexpr int PSTG_WARP = 16 * 16;  // staging per epilogue warp: 16 rows x 16 columns of 8 bytes
+constexpr int PSTG_BYTES = PEPI * PSTG_WARP * 8;
+constexpr size_t PSMEM = 222 * 1024;  // dynamic shared memory (the item table is static)
 
-template <int NS>
+template <int NS, int BK>
 struct PCfg {
-  static constexpr int STAGES = NS == 3 ? 3 : 4;
-  static constexpr int STAGE_BYTES = NS * (PA_BYTES + PB_BYTES);
-  static constexpr int NPROD = NS == 2 ? 3 : 6;
+  static constexpr int A_BYTES = PBM * BK * 2, B_BYTES = PBN * BK * 2;  // per level
+  static constexpr int STAGE_BYTES = NS * (A_BYTES + B_BYTES);
+  static constexpr int STAGES = (int)((PSMEM - PSTG_BYTES - 1024) / STAGE_BYTES);
 };
 
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
-// bounded wait that also gives up when another role raised the abort flag
-__device__ __forceinline__ bool wait_ab(uint64_t* bar, uint32_t parity, long long budget, volatile int* abort_f,
-                                        int* err) {
-  if (mbar_test_wait(bar, parity)) return true;
-  const unsigned long long t0 = globaltimer();
-  while (true) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if (*abort_f) return false;
-    if (budget <= 0 || (long long)(globaltimer() - t0) > budget) {
-      *abort_f = 1;
-      if (err) atomicExch(err, 1);
-      return false;
-    }
-  }
-}
-
-__device__ __forceinline__ int tile_chunks(const GGroup& g, const GSeg* segs) {
+// K chunks of the tile part: the sum over its segments, by the whole warp
+template <int BK>
+__device__ __forceinline__ int part_chunks(const TileItem& q, const GSeg* segs) {
+  if (q.n <= 1) return (q.K0 + BK - 1) / BK;
   int t = 0;
-  for (int si = g.seg0; si < g.seg1; ++si) t += (segs[si].K + PBK - 1) / PBK;
-  return t;
+  for (int s = threadIdx.x & 31; s < q.n; s += 32) t += (segs[q.seg0 + s * q.parts].K + BK - 1) / BK;
+  return __reduce_add_sync(0xffffffffu, t);
 }
 
-template <int NS>
+// OUT32: every group of the launch writes FP32 (flags bit 1), else FP64
+template <int NS, int BK, bool OUT32>
 __global__ void __launch_bounds__(PTHREADS, 1) gemm_tcp_kernel(const GGroup* __restrict__ groups,
                                                                const GSeg* __restrict__ segs,
-                                                               const GTile* __restrict__ tiles, int ntiles,
+                                                               const GTile* __restrict__ tiles, int nitems, int split,
                                                                const CUtensorMap* __restrict__ maps, Bases bs,
-                                                               int* __restrict__ err, long long wait_ns) {
-  using C = PCfg<NS>;
-  constexpr int S = C::STAGES;
+                                                               uint64_t* __restrict__ scratch,
+                                                               unsigned* __restrict__ tickets, int* __restrict__ err,
+                                                               long long wait_ns) {
+  using C = PCfg<NS, BK>;
+  constexpr int S = C::STAGES, FOLD = PFOLD_K / BK;  // chunks per fold group
+  constexpr int BUF = 64 * NS;                       // TMEM columns of one accumulator buffer
+  static_assert(S >= 2 && 2 * BUF <= (int)PTMEM_COLS, "stages and accumulators");
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[S], empty_bar[S], accf[2], acce[2];
   __shared__ uint32_t tmem_base_s;
   __shared__ int abort_s, issued_s, consumed_s, last_commit_s, last_accf_s;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   volatile int* abort_f = &abort_s;
+  __shared__ TileItem table[TITEMS];
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // the CTA's i-th item, in shared memory (beyond the table in a slot of the warp;
+  // an item and its successor may be in use together)
+  __shared__ TileItem own[(PTHREADS / 32)][2];
+  auto item = [&](int i) -> const TileItem& {
+    if (i < TITEMS) return table[i];
+    TileItem& o = own[warp][i & 1];
+    __syncwarp();
+    if (lane == 0) o = load_item(groups, segs, tiles, bs, (OUT32 ? 4 : 8), blockIdx.x + i * gridDim.x, split);
+    __syncwarp();
+    return o;
+  };
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)),
                  "r"(PTMEM_COLS)
@@ -106,7 +110,7 @@ __global__ void __launch_bounds__(PTHREADS, 1) gemm_tcp_kernel(const GGroup* __r
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&accf[b], 1);
-      mbar_init(&acce[b], 4);  // one arrive per epilogue warp
+      mbar_init(&acce[b], PEPI);
     }
     abort_s = 0;
     issued_s = 0;
@@ -115,171 +119,160 @@ __global__ void __launch_bounds__(PTHREADS, 1) gemm_tcp_kernel(const GGroup* __r
     last_accf_s = -1;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  int kl0 = 0;
+  if (warp == 0) kl0 = first_segments(groups, segs, tiles, maps, split);
+  else load_items(table, groups, segs, tiles, maps, bs, (OUT32 ? 4 : 8), nitems, split);
   fence_before();
   __syncthreads();
   fence_after();
   const uint32_t tmem = tmem_base_s;
 
   if (warp == 0) {
-    // ---------------- producer: TMA ring ----------------
-    if (lane == 0) {
-      int it = 0, fenced = -1;
-      for (int t = blockIdx.x; t < ntiles && !*abort_f; t += gridDim.x) {
-        const GTile tl = tiles[t];
-        const GGroup g = groups[tl.g];
-        for (int si = g.seg0; si < g.seg1 && !*abort_f; ++si) {
-          const int K = segs[si].K;
-          const CUtensorMap* ma = maps + 3 * si;
-          const CUtensorMap* mb = maps + 3 * si + 2;
-          if (fenced != si) {  // tensor maps written by a host copy: acquire before first use
-            asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(reinterpret_cast<uint64_t>(ma))
-                         : "memory");
-            asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(reinterpret_cast<uint64_t>(mb))
-                         : "memory");
-            fenced = si;
-          }
-          for (int k0 = 0; k0 < K; k0 += PBK) {
-            const int s = it % S;
-            if (!wait_ab(&empty_bar[s], ((it / S) & 1) ^ 1, wait_ns, abort_f, err)) break;
-            uint8_t* st = smem + s * C::STAGE_BYTES;
-            mbar_expect_tx(&full_bar[s], C::STAGE_BYTES);
-#pragma unroll
-            for (int l = 0; l < NS; ++l) tma_load_3d(st + l * PA_BYTES, ma, k0, tl.m0, l, &full_bar[s]);
-#pragma unroll
-            for (int l = 0; l < NS; ++l) tma_load_3d(st + NS * PA_BYTES + l * PB_BYTES, mb, k0, tl.n0, l, &full_bar[s]);
-            ++it;
-            issued_s = it;
-          }
+    // ---------------- producer ----------------
+    int it = 0;
+    for (int i = 0; blockIdx.x + i * gridDim.x < nitems && !*abort_f; ++i) {
+      const TileItem& q = item(i);
+      for (int s0 = 0; s0 < q.n; s0 += 32) {
+        int kl = q.K0;
+        if (i == 0 && s0 == 0) {
+          kl = kl0;
+        } else if (q.n > 1 || i >= TITEMS) {
+          const int sl = q.seg0 + min(s0 + lane, q.n - 1) * q.parts;
+          kl = segs[sl].K;
+          fence_maps(maps, sl);
+          __syncwarp();
         }
+        for (int s = s0; s < min(q.n, s0 + 32); ++s) {
+          const int K = __shfl_sync(0xffffffffu, kl, s - s0);
+          if (lane == 0) {
+            const CUtensorMap* ma = maps + 4 * (q.seg0 + s * q.parts) + 3;
+            const CUtensorMap* mb = ma - 1;
+            for (int k0 = 0; k0 < K; k0 += BK) {
+              const int sg = it % S;
+              if (!wait_ab(&empty_bar[sg], ((it / S) & 1) ^ 1, wait_ns, abort_f, err)) break;
+              uint8_t* st = smem + sg * C::STAGE_BYTES;
+              mbar_expect_tx(&full_bar[sg], C::STAGE_BYTES);
+#pragma unroll
+              for (int l = 0; l < NS; ++l) tma_load_3d(st + l * C::A_BYTES, ma, k0, q.m0, l, &full_bar[sg]);
+#pragma unroll
+              for (int l = 0; l < NS; ++l)
+                tma_load_3d(st + NS * C::A_BYTES + l * C::B_BYTES, mb, k0, q.n0, l, &full_bar[sg]);
+              ++it;
+              issued_s = it;
+            }
+          }
+          __syncwarp();
+          if (*abort_f) break;
+        }
+        if (*abort_f) break;
       }
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
-      const uint32_t idesc =
-          (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(PBN >> 3) << 17) | ((uint32_t)(PBM >> 4) << 24);
-      int it = 0, fg = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-        const GTile tl = tiles[t];
-        const GGroup g = groups[tl.g];
-        const int T = tile_chunks(g, segs);
-        for (int b0 = 0; b0 < T && ok; b0 += PFOLD) {
-          const int b = fg & 1;
-          ok = wait_ab(&acce[b], ((fg >> 1) & 1) ^ 1, wait_ns, abort_f, err);
-          if (!ok) break;
-          fence_after();
-          const uint32_t t_acc = tmem + 128 * b, t_acc2 = t_acc + 64;
-          const int b1 = min(T, b0 + PFOLD);
-          for (int c = b0; c < b1; ++c) {
-            const int s = it % S;
-            ok = wait_ab(&full_bar[s], (it / S) & 1, wait_ns, abort_f, err);
+    constexpr uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(PBM >> 4) << 24);
+    int it = 0, fg = 0;
+    bool ok = true;
+    for (int i = 0; blockIdx.x + i * gridDim.x < nitems && ok; ++i) {
+      const TileItem& q = item(i);
+      int kl = q.K0, c = 0;  // c: chunk within the part; a fold group is FOLD chunks
+      const int T = part_chunks<BK>(q, segs);
+      for (int s = 0; s < q.n && ok; ++s) {
+        if ((s & 31) == 0 && q.n > 1) kl = segs[q.seg0 + min(s + lane, q.n - 1) * q.parts].K;
+        const int K = __shfl_sync(0xffffffffu, kl, s & 31);
+        if (lane == 0) {
+          for (int k0 = 0; k0 < K && ok; k0 += BK, ++c) {
+            const int b = fg & 1;
+            const bool first = c % FOLD == 0;
+            if (first) {
+              ok = wait_ab(&acce[b], ((fg >> 1) & 1) ^ 1, wait_ns, abort_f, err);
+              if (!ok) break;
+            }
+            const int sg = it % S;
+            ok = wait_ab(&full_bar[sg], (it / S) & 1, wait_ns, abort_f, err);
             if (!ok) break;
             consumed_s = it + 1;
             fence_after();
-            const uint32_t sa = smem_u32(smem + s * C::STAGE_BYTES);
+            const uint32_t tb = tmem + BUF * b;
+            const uint32_t sa = smem_u32(smem + sg * C::STAGE_BYTES);
+            const int nk = (min(BK, K - k0) + 15) >> 4;  // 16-wide steps with data
+            for (int kk = 0; kk < nk; ++kk) {
+              const uint64_t bd = desc_of<BK>(sa + NS * C::A_BYTES + kk * 32);
 #pragma unroll
-            for (int p = 0; p < C::NPROD; ++p) {
-              const int la = (p == 2 || p == 4) ? 1 : (p == 5 ? 2 : 0);
-              const int lb = (p == 1 || p == 4) ? 1 : (p == 3 ? 2 : 0);
-              const uint32_t aa = sa + la * PA_BYTES, ba = sa + NS * PA_BYTES + lb * PB_BYTES;
-#pragma unroll
-              for (int kk = 0; kk < PBK / 16; ++kk) {
-                const uint32_t acc = (c > b0 || p > 1 || kk > 0) ? 1u : 0u;
-                umma_f16(p == 0 ? t_acc : t_acc2, make_desc(aa + kk * 32), make_desc(ba + kk * 32), idesc, acc);
-              }
+              for (int l = 0; l < NS; ++l)
+                umma_f16(tb + 64 * l, desc_of<BK>(sa + l * C::A_BYTES + kk * 32), bd,
+                         idesc0 | ((uint32_t)((PBN * (NS - l)) >> 3) << 17), (!first || kk > 0 || l > 0) ? 1u : 0u);
             }
-            umma_commit(&empty_bar[s]);
+            umma_commit(&empty_bar[sg]);
             last_commit_s = it;
             ++it;
+            if (c % FOLD == FOLD - 1 || c == T - 1) {
+              umma_commit(&accf[b]);
+              last_accf_s = fg;
+              ++fg;
+            }
           }
-          if (!ok) break;
-          umma_commit(&accf[b]);
-          last_accf_s = fg;
-          ++fg;
         }
+        ok = __shfl_sync(0xffffffffu, ok, 0);
       }
     }
   } else {
-    // ---------------- epilogue: warps 2..5 ----------------
-    const int q = warp & 3;  // TMEM lane quarter this warp may access
+    // ---------------- epilogue: fold, write per tile ----------------
+    // warp w reads TMEM lanes 32 (w % 4) .. + 31 and folds columns 32 h .. + 31
+    const int q = warp & 3, h = (warp - 2) >> 2;
     const uint32_t lane_off = (uint32_t)(32 * q) << 16;
-    const uint32_t t_hi = tmem + 256, t_lo = tmem + 320;
+    uint64_t* stg = reinterpret_cast<uint64_t*>(smem + S * C::STAGE_BYTES) + (warp - 2) * PSTG_WARP;
     int fg = 0;
     bool ok = true;
-    float v[32], u[32], h[32], w[32];
-    for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-      const GTile tl = tiles[t];
-      const GGroup g = groups[tl.g];
-      const int T = tile_chunks(g, segs);
-      int folds = 0;
-      for (int b0 = 0; b0 < T; b0 += PFOLD) {
+    float hi[32], lo[32];
+    for (int i = 0; blockIdx.x + i * gridDim.x < nitems && ok; ++i) {
+      const TileItem& z = item(i);
+      if (z.part >= z.parts) continue;
+#pragma unroll
+      for (int i = 0; i < 32; ++i) { hi[i] = 0.f; lo[i] = 0.f; }
+      const int units = (part_chunks<BK>(z, segs) + FOLD - 1) / FOLD;
+      for (int f = 0; f < units; ++f) {
         const int b = fg & 1;
         ok = __all_sync(0xffffffffu, wait_ab(&accf[b], (fg >> 1) & 1, wait_ns, abort_f, err));
-        if (!ok) break;  // warp-uniform: the TMEM loads below are warp-collective
+        if (!ok) break;
         fence_after();
-        const uint32_t t_acc = tmem + 128 * b, t_acc2 = t_acc + 64;
-#pragma unroll 1
-        for (int cb = 0; cb < PBN; cb += 32) {
-          tmem_ld32(t_acc + lane_off + cb, v);
-          tmem_ld32(t_acc2 + lane_off + cb, u);
-          if (folds == 0) {
-            tmem_st32(t_hi + lane_off + cb, v);
-            tmem_st32(t_lo + lane_off + cb, u);
-          } else {
-            tmem_ld32(t_hi + lane_off + cb, h);
-            tmem_ld32(t_lo + lane_off + cb, w);
+        const uint32_t tb = tmem + BUF * b + lane_off + 32 * h;
 #pragma unroll
-            for (int i = 0; i < 32; ++i) {
-              const float s = h[i] + v[i];
-              const float bp = s - h[i];
-              const float ap = s - bp;
-              w[i] += ((h[i] - ap) + (v[i] - bp)) + u[i];
-              h[i] = s;
-            }
-            tmem_st32(t_hi + lane_off + cb, h);
-            tmem_st32(t_lo + lane_off + cb, w);
+        for (int cb = 0; cb < 32; cb += 16) {
+          uint32_t dv[NS][16];
+#pragma unroll
+          for (int d = 0; d < NS; ++d) tmem_ld16_nw(tb + 64 * d + cb, dv[d]);
+          tmem_wait_ld16(dv[0]);
+#pragma unroll
+          for (int d = 1; d < NS; ++d) tmem_dep16(dv[d]);
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            float u = __uint_as_float(dv[NS - 1][i]);
+#pragma unroll
+            for (int d = NS - 2; d >= 1; --d) u += __uint_as_float(dv[d][i]);
+            two_sum_into(hi[cb + i], lo[cb + i], __uint_as_float(dv[0][i]));
+            lo[cb + i] += u;
           }
         }
         fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&acce[b]);
-        ++folds;
         ++fg;
       }
       if (!ok) break;
-      // the finished tile: row = TMEM lane, 32 consecutive columns per load
-      const bool accum = g.flags & 1, out_f32 = g.flags & 2;
-      const int row = tl.m0 + 32 * q + lane;
-#pragma unroll 1
-      for (int cb = 0; cb < PBN; cb += 32) {
-        if (folds > 0) {
-          tmem_ld32(t_hi + lane_off + cb, h);
-          tmem_ld32(t_lo + lane_off + cb, w);
+      if (z.parts > 1 && !gather_parts(z, (blockIdx.x + i * gridDim.x) / split, split, PEPI, warp - 2, scratch, tickets, hi, lo)) continue;
+#pragma unroll
+      for (int cb = 0; cb < 32; cb += 16) {
+        if (OUT32) {
+          store_block16(stg, [&](int k) { return (uint64_t)__float_as_uint(hi[cb + k] + lo[cb + k]); },
+                        reinterpret_cast<float*>(z.C), z.ldc, z.m0 + 32 * q, z.n0 + 32 * h + cb, z.M, z.N, z.flags & 1);
         } else {
+          double v[16];
 #pragma unroll
-          for (int i = 0; i < 32; ++i) { h[i] = 0.f; w[i] = 0.f; }
-        }
-        if (row < g.M) {
-          const long long o = (long long)row * g.ldc + tl.n0 + cb;
-          const int ncol = min(32, g.N - tl.n0 - cb);
-          if (out_f32) {
-            float* Cp = reinterpret_cast<float*>(sel_base(bs, slot_of(g.C))) + off_of(g.C) + o;
-#pragma unroll
-            for (int i = 0; i < 32; ++i)
-              if (i < ncol) Cp[i] = accum ? Cp[i] + (h[i] + w[i]) : (h[i] + w[i]);
-          } else {
-            double* Cp = reinterpret_cast<double*>(sel_base(bs, slot_of(g.C))) + off_of(g.C) + o;
-#pragma unroll
-            for (int i = 0; i < 32; ++i)
-              if (i < ncol) {
-                const double val = (double)h[i] + (double)w[i];
-                Cp[i] = accum ? Cp[i] + val : val;
-              }
-          }
+          for (int k = 0; k < 16; ++k) v[k] = dbl_of_pair(hi[cb + k], lo[cb + k]);
+          store_block16(stg, [&](int k) { return (uint64_t)__double_as_longlong(v[k]); },
+                        reinterpret_cast<double*>(z.C), z.ldc, z.m0 + 32 * q, z.n0 + 32 * h + cb, z.M, z.N, z.flags & 1);
         }
       }
-      fence_before();  // the next tile's first fold overwrites hi / lo after these loads
     }
   }
 
@@ -315,32 +308,27 @@ int sm_count() {
 
 }  // namespace
 
-size_t tcp_smem_bytes(int nsplit) {
-  return nsplit == 3 ? (size_t)PCfg<3>::STAGES * PCfg<3>::STAGE_BYTES + 1024
-                     : (size_t)PCfg<2>::STAGES * PCfg<2>::STAGE_BYTES + 1024;
-}
-
-cudaError_t launch_gemm_tcp(const GGroup* groups, const GSeg* segs, const GTile* tiles, int ntiles, const void* maps,
-                            const Bases& b, int nsplit, int* err, long long wait_ns, cudaStream_t s) {
+cudaError_t launch_gemm_tcp(const GGroup* groups, const GSeg* segs, const GTile* tiles, int ntiles, int split,
+                            int kbox, const void* maps, const Bases& b, int nsplit, bool out32, void* scratch,
+                            unsigned* tickets, int* err, long long wait_ns, cudaStream_t s) {
   if (ntiles == 0) return cudaSuccess;
-  const size_t smem = tcp_smem_bytes(nsplit);
-  const int grid = ntiles < sm_count() ? ntiles : sm_count();
-  if (nsplit == 2) {
-    static const cudaError_t e =
-        cudaFuncSetAttribute(gemm_tcp_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if ((kbox != 32 && kbox != 64) || split < 1 || (split > 1 && (!scratch || !tickets))) return cudaErrorInvalidValue;
+  const int nitems = ntiles * split, grid = nitems < sm_count() ? nitems : sm_count();
+  auto run = [&](auto kernel) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PSMEM);
     if (e != cudaSuccess) return e;
-    gemm_tcp_kernel<2><<<grid, PTHREADS, smem, s>>>(groups, segs, tiles, ntiles, (const CUtensorMap*)maps, b, err,
-                                                    wait_ns);
-  } else if (nsplit == 3) {
-    static const cudaError_t e =
-        cudaFuncSetAttribute(gemm_tcp_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    gemm_tcp_kernel<3><<<grid, PTHREADS, smem, s>>>(groups, segs, tiles, ntiles, (const CUtensorMap*)maps, b, err,
-                                                    wait_ns);
-  } else {
-    return cudaErrorInvalidValue;
-  }
-  return cudaGetLastError();
+    kernel<<<grid, PTHREADS, PSMEM, s>>>(groups, segs, tiles, nitems, split, (const CUtensorMap*)maps, b,
+                                         (uint64_t*)scratch, tickets, err, wait_ns);
+    return cudaGetLastError();
+  };
+  auto pick = [&](auto ns) {
+    constexpr int NS = decltype(ns)::value;
+    if (kbox == 64) return out32 ? run(gemm_tcp_kernel<NS, 64, true>) : run(gemm_tcp_kernel<NS, 64, false>);
+    return out32 ? run(gemm_tcp_kernel<NS, 32, true>) : run(gemm_tcp_kernel<NS, 32, false>);
+  };
+  if (nsplit == 2) return pick(std::integral_constant<int, 2>{});
+  if (nsplit == 3) return pick(std::integral_constant<int, 3>{});
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace tt

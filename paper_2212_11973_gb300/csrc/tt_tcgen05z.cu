@@ -26,24 +26,32 @@
 // barrier).  Waits are bounded as in the other tcgen05 kernels.
 //
 // What bounds it: the chain of 18 to 42 short segments (K = 3 to 180) behind
-// each output tile at small D, shared-memory and L2 bandwidth of the operands at
-// D = 1024; never the tensor pipe.  So (1) 16-wide K steps past a segment's end
-// are skipped, and plans whose segments are at most 64 long (D up to ~350) use
-// chunks of 32, four in flight (D = 300: 40 -> 24 us a launch; D = 1024, whose
-// longer segments feed fine from two stages of 64, was 15 % slower with them);
-// (2) a segment's tensor maps are
-// fenced and its K and exponent references read by the lanes of a warp, 32
-// segments at a time, and the row exponents of the next segment are loaded
-// before the wait for the current one; (3) where a plan has fewer tiles than
-// SMs, `split` CTAs share a tile's segments: each writes its two-float sums to
-// scratch and the last to arrive (a ticket per tile and folding warp, no CTA
-// waits for another) adds them in part order.
+// each output tile at small D, shared-memory and L2 bandwidth of the operands and
+// the output stores at D = 1024; never the tensor pipe.  So
+//   (1) 16-wide K steps past a segment's end are skipped, and plans whose segments
+//       are at most 64 long (D up to ~350) use chunks of 32, four in flight (D =
+//       1024, whose longer segments feed fine from two stages of 64, was 15 %
+//       slower with them);
+//   (2) the items of a CTA are read side by side into shared memory before the
+//       roles start; a segment's tensor maps are fenced and its K and exponent
+//       references read by the lanes of a warp, 32 segments at a time; exponents
+//       are loaded one segment ahead of the wait;
+//   (3) where a plan has fewer tiles than SMs, `split` CTAs share a tile's
+//       segments: each writes its two-float sums to scratch and the last to
+//       arrive (a ticket per tile and folding warp, no CTA waits for another)
+//       adds them in part order;
+//   (4) FP64 outputs are put together by integer operations, and all stores of
+//       16 rows are in flight together.
+// Measured, a launch: S3, B1 and B2 at D = 300 40 -> 19 us on average; S3 at D =
+// 1024 205 -> 150 us, S1 133 -> 121 us (25 tiles a CTA, each a single segment:
+// its stores are half of the time).
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 #include <cstdint>
 
+#include "tt_df.h"
 #include "tt_kernels.h"
 #include "tt_tc_ptx.h"
 
@@ -60,93 +68,10 @@ constexpr uint32_t ZTMEM_COLS = 512;
 constexpr int ZEPI = 8;  // epilogue warps
 constexpr int ZTHREADS = 64 + 32 * ZEPI;
 constexpr int ZMAXK = 256;  // longest segment whose digit sums stay exact
-// epilogue staging, after the TMA stages: per epilogue warp 32 rows x 16
-// columns of 8-byte outputs, column c of row r at word r * 16 + (c ^ (r & 15))
-constexpr int ZSTG_WARP = 32 * 16;
+// epilogue staging, after the TMA stages: per epilogue warp 16 rows x 16
+// columns of 8-byte outputs
+constexpr int ZSTG_WARP = 16 * 16;
 constexpr int ZSTG_BYTES = ZEPI * ZSTG_WARP * 8;
-
-__device__ __forceinline__ void mbar_arrive_z(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
-__device__ __forceinline__ bool wait_z(uint64_t* bar, uint32_t parity, long long budget, volatile int* abort_f,
-                                       int* err) {
-  if (mbar_test_wait(bar, parity)) return true;
-  const unsigned long long t0 = globaltimer();
-  while (true) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if (*abort_f) return false;
-    if (budget <= 0 || (long long)(globaltimer() - t0) > budget) {
-      *abort_f = 1;
-      if (err) atomicExch(err, 1);
-      return false;
-    }
-  }
-}
-
-// 16 TMEM columns of this warp's lane quarter, not yet waited for: the caller
-// issues tmem_wait_ld16() with one set of registers and tmem_dep16() with
-// every other set before reading them (the registers pass through those asm
-// statements, so no use is scheduled before the wait)
-__device__ __forceinline__ void tmem_ld16_nw(uint32_t taddr, uint32_t* r) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-}
-__device__ __forceinline__ void tmem_wait_ld16(uint32_t* r) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
-               :
-               : "memory");
-}
-__device__ __forceinline__ void tmem_dep16(uint32_t* r) {
-  asm volatile(""
-               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
-               :
-               : "memory");
-}
-
-__device__ __forceinline__ void two_sum_z(float& hi, float& lo, float x) {
-  const float s = hi + x;
-  const float bp = s - hi;
-  const float ap = s - bp;
-  lo += (hi - ap) + (x - bp);
-  hi = s;
-}
-
-// UMMA shared-memory descriptor, K-major, rows of BK elements in one swizzle
-// span (64: 128 bytes, 32: 64 bytes), 8-row groups contiguous
-template <int BK>
-__device__ __forceinline__ uint64_t desc_of(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr >> 4) & 0x3FFF);
-  d |= (uint64_t)1 << 16;                    // leading byte offset (unused for swizzled K-major)
-  d |= (uint64_t)((8 * BK * 2) >> 4) << 32;  // stride byte offset
-  d |= (uint64_t)1 << 46;                    // descriptor version
-  d |= (uint64_t)(BK == 64 ? 2 : 4) << 61;   // SWIZZLE_128B / SWIZZLE_64B
-  return d;
-}
-
-// one part of a tile: segments seg0 + part, + split, ... (n of them)
-struct ZItem {
-  GTile tl;
-  GGroup g;
-  int part, parts, n;
-};
-__device__ __forceinline__ ZItem item_of(const GGroup* groups, const GTile* tiles, int w, int split) {
-  ZItem it;
-  it.tl = tiles[w / split];
-  it.g = groups[it.tl.g];
-  const int nseg = it.g.seg1 - it.g.seg0;
-  it.part = w % split;
-  it.parts = max(1, min(split, nseg));
-  it.n = it.part < it.parts ? (nseg - it.part + it.parts - 1) / it.parts : 0;
-  return it;
-}
 
 // PAIR: every group of the launch writes two-float pairs (flags bit 1), else
 // FP64 (accumulating with flags bit 0); one kernel per output form keeps the
@@ -169,8 +94,20 @@ __global__ void __launch_bounds__(ZTHREADS, 1) gemm_tcz_kernel(const GGroup* __r
   __shared__ int abort_s, issued_s, consumed_s, last_commit_s, last_accf_s;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   volatile int* abort_f = &abort_s;
+  __shared__ TileItem table[TITEMS];
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // the CTA's i-th item, in shared memory (beyond the table in a slot of the warp;
+  // an item and its successor may be in use together)
+  __shared__ TileItem own[(ZTHREADS / 32)][2];
+  auto item = [&](int i) -> const TileItem& {
+    if (i < TITEMS) return table[i];
+    TileItem& o = own[warp][i & 1];
+    __syncwarp();
+    if (lane == 0) o = load_item(groups, segs, tiles, bs, 8, blockIdx.x + i * gridDim.x, split);
+    __syncwarp();
+    return o;
+  };
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)),
                  "r"(ZTMEM_COLS)
@@ -193,6 +130,9 @@ __global__ void __launch_bounds__(ZTHREADS, 1) gemm_tcz_kernel(const GGroup* __r
     last_accf_s = -1;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  int kl0 = 0;
+  if (warp == 0) kl0 = first_segments(groups, segs, tiles, maps, split);
+  else load_items(table, groups, segs, tiles, maps, bs, 8, nitems, split);
   fence_before();
   __syncthreads();
   fence_after();
@@ -200,37 +140,34 @@ __global__ void __launch_bounds__(ZTHREADS, 1) gemm_tcz_kernel(const GGroup* __r
 
   if (warp == 0) {
     // ---------------- producer ----------------
-    int it = 0, fenced = -1;  // group whose first 32 segments' maps this CTA has fenced
-    for (int w = blockIdx.x; w < nitems && !*abort_f; w += gridDim.x) {
-      const ZItem q = item_of(groups, tiles, w, split);
+    int it = 0;
+    for (int i = 0; blockIdx.x + i * gridDim.x < nitems && !*abort_f; ++i) {
+      const TileItem& q = item(i);
       for (int s0 = 0; s0 < q.n; s0 += 32) {
-        const int sl = q.g.seg0 + q.part + min(s0 + lane, q.n - 1) * q.parts;
-        const int kl = segs[sl].K;
-        if (fenced != q.tl.g || q.n > 32) {
-          const uint64_t ma = reinterpret_cast<uint64_t>(maps + 3 * sl), mb = ma + 2 * sizeof(CUtensorMap);
-          asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(ma) : "memory");
-          asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(mb) : "memory");
-          asm volatile("prefetch.tensormap [%0];" ::"l"(ma) : "memory");
-          asm volatile("prefetch.tensormap [%0];" ::"l"(mb) : "memory");
-          fenced = q.parts == 1 ? q.tl.g : -1;
+        int kl = q.K0;
+        if (i == 0 && s0 == 0) {
+          kl = kl0;
+        } else if (q.n > 1 || i >= TITEMS) {
+          const int sl = q.seg0 + min(s0 + lane, q.n - 1) * q.parts;
+          kl = segs[sl].K;
+          fence_maps(maps, sl);
           __syncwarp();
         }
         for (int s = s0; s < min(q.n, s0 + 32); ++s) {
           const int K = __shfl_sync(0xffffffffu, kl, s - s0);
           if (lane == 0) {
-            const int si = q.g.seg0 + q.part + s * q.parts;
-            const CUtensorMap* ma = maps + 3 * si;
-            const CUtensorMap* mb = ma + 2;
+            const CUtensorMap* ma = maps + 4 * (q.seg0 + s * q.parts) + 3;
+            const CUtensorMap* mb = ma - 1;
             for (int k0 = 0; k0 < K; k0 += ZBK) {
               const int sg = it % ZSTAGES;
-              if (!wait_z(&empty_bar[sg], ((it / ZSTAGES) & 1) ^ 1, wait_ns, abort_f, err)) break;
+              if (!wait_ab(&empty_bar[sg], ((it / ZSTAGES) & 1) ^ 1, wait_ns, abort_f, err)) break;
               uint8_t* st = smem + sg * ZSTAGE_BYTES;
               mbar_expect_tx(&full_bar[sg], ZSTAGE_BYTES);
 #pragma unroll
-              for (int l = 0; l < ZDIG; ++l) tma_load_3d(st + l * ZA_BYTES, ma, k0, q.tl.m0, l, &full_bar[sg]);
+              for (int l = 0; l < ZDIG; ++l) tma_load_3d(st + l * ZA_BYTES, ma, k0, q.m0, l, &full_bar[sg]);
 #pragma unroll
               for (int l = 0; l < ZDIG; ++l)
-                tma_load_3d(st + ZDIG * ZA_BYTES + l * ZB_BYTES, mb, k0, q.tl.n0, l, &full_bar[sg]);
+                tma_load_3d(st + ZDIG * ZA_BYTES + l * ZB_BYTES, mb, k0, q.n0, l, &full_bar[sg]);
               ++it;
               issued_s = it;
             }
@@ -251,20 +188,20 @@ __global__ void __launch_bounds__(ZTHREADS, 1) gemm_tcz_kernel(const GGroup* __r
     constexpr uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(ZBM >> 4) << 24);
     int it = 0, fg = 0;
     bool ok = true;
-    for (int w = blockIdx.x; w < nitems && ok; w += gridDim.x) {
-      const ZItem q = item_of(groups, tiles, w, split);
-      int kl = 0;
+    for (int i = 0; blockIdx.x + i * gridDim.x < nitems && ok; ++i) {
+      const TileItem& q = item(i);
+      int kl = q.K0;
       for (int s = 0; s < q.n && ok; ++s) {
-        if ((s & 31) == 0) kl = segs[q.g.seg0 + q.part + min(s + lane, q.n - 1) * q.parts].K;
+        if ((s & 31) == 0 && q.n > 1) kl = segs[q.seg0 + min(s + lane, q.n - 1) * q.parts].K;
         const int K = __shfl_sync(0xffffffffu, kl, s & 31);
         if (lane == 0) {
           const int b = fg & 1;
-          ok = wait_z(&acce[b], ((fg >> 1) & 1) ^ 1, wait_ns, abort_f, err);
+          ok = wait_ab(&acce[b], ((fg >> 1) & 1) ^ 1, wait_ns, abort_f, err);
           fence_after();
           const uint32_t tb = tmem + 256 * b;
           for (int k0 = 0; k0 < K && ok; k0 += ZBK) {
             const int sg = it % ZSTAGES;
-            ok = wait_z(&full_bar[sg], (it / ZSTAGES) & 1, wait_ns, abort_f, err);
+            ok = wait_ab(&full_bar[sg], (it / ZSTAGES) & 1, wait_ns, abort_f, err);
             if (!ok) break;
             consumed_s = it + 1;
             fence_after();
@@ -300,48 +237,52 @@ __global__ void __launch_bounds__(ZTHREADS, 1) gemm_tcz_kernel(const GGroup* __r
     int fg = 0;
     bool ok = true;
     float hi[32], lo[32];
-    for (int w = blockIdx.x; w < nitems && ok; w += gridDim.x) {
-      const ZItem z = item_of(groups, tiles, w, split);
-      const GTile tl = z.tl;
-      const GGroup& g = z.g;
-      if (z.part >= z.parts) continue;
-      const int row = tl.m0 + 32 * q + lane;
-      const int col_l = tl.n0 + 32 * h + lane;  // the column whose exponent this lane loads
-#pragma unroll
-      for (int i = 0; i < 32; ++i) { hi[i] = 0.f; lo[i] = 0.f; }
+    // row exponents of the segment at hand: this lane's row, and the column of
+    // which it holds the exponent for the others
+    int ea = 0, eb = 0;
+    auto exps = [&](const TileItem& t, const short* pa, int sa, const short* pb, int sb, int& xa, int& xb) {
+      const int row = t.m0 + 32 * q + lane, col = t.n0 + 32 * h + lane;
+      xa = t.n > 0 && row < t.M ? (int)pa[(long long)row * sa] : 0;
+      xb = t.n > 0 && col < t.N ? (int)pb[(long long)col * sb] : 0;
+    };
+    for (int i = 0; blockIdx.x + i * gridDim.x < nitems && ok; ++i) {
+      const TileItem& z = item(i);
       // exponent references of 32 segments, one per lane; the exponents of the
-      // segment after the current one are in flight while it is waited for
+      // segment (or the next item's first segment) after the current one are in
+      // flight while it is waited for
       unsigned long long ral = 0, rbl = 0;
       int sal = 0, sbl = 0;
       auto refs = [&](int s) {
-        const GSeg* sp = segs + g.seg0 + z.part + min(s + lane, z.n - 1) * z.parts;
-        ral = sp->eA;
-        rbl = sp->eB;
+        const GSeg* sp = segs + z.seg0 + min(s + lane, z.n - 1) * z.parts;
+        ral = reinterpret_cast<unsigned long long>(exps_ptr(bs, sp->eA));
+        rbl = reinterpret_cast<unsigned long long>(exps_ptr(bs, sp->eB));
         sal = sp->eas;
         sbl = sp->ebs;
       };
-      auto exps = [&](int s, int& ea, int& eb) {
-        const int l = s & 31;
-        const Ref ra = __shfl_sync(0xffffffffu, ral, l), rb = __shfl_sync(0xffffffffu, rbl, l);
-        const int sa = __shfl_sync(0xffffffffu, sal, l), sb = __shfl_sync(0xffffffffu, sbl, l);
-        const short* pa = reinterpret_cast<const short*>(sel_base(bs, slot_of(ra))) + off_of(ra);
-        const short* pb = reinterpret_cast<const short*>(sel_base(bs, slot_of(rb))) + off_of(rb);
-        ea = row < g.M ? (int)pa[(long long)row * sa] : 0;
-        eb = col_l < g.N ? (int)pb[(long long)col_l * sb] : 0;
-      };
-      int ea = 0, eb = 0;
-      if (z.n > 0) {
-        refs(0);
-        exps(0, ea, eb);
+      if (z.n > 1) refs(0);
+      if (i == 0) exps(z, z.pa, z.eas, z.pb, z.ebs, ea, eb);
+#pragma unroll
+      for (int i = 0; i < 32; ++i) { hi[i] = 0.f; lo[i] = 0.f; }
+      if (z.n == 0) {
+        if (blockIdx.x + (i + 1) * gridDim.x < nitems) {
+          const TileItem& nx = item(i + 1);
+          exps(nx, nx.pa, nx.eas, nx.pb, nx.ebs, ea, eb);
+        }
+        if (z.part >= z.parts) continue;  // (no segment left for this part)
       }
       for (int s = 0; s < z.n; ++s) {
         int ean = 0, ebn = 0;
         if (s + 1 < z.n) {
           if (((s + 1) & 31) == 0) refs(s + 1);
-          exps(s + 1, ean, ebn);
+          const int l = (s + 1) & 31;
+          exps(z, reinterpret_cast<const short*>(__shfl_sync(0xffffffffu, ral, l)), __shfl_sync(0xffffffffu, sal, l),
+               reinterpret_cast<const short*>(__shfl_sync(0xffffffffu, rbl, l)), __shfl_sync(0xffffffffu, sbl, l), ean, ebn);
+        } else if (blockIdx.x + (i + 1) * gridDim.x < nitems) {
+          const TileItem& nx = item(i + 1);
+          exps(nx, nx.pa, nx.eas, nx.pb, nx.ebs, ean, ebn);
         }
         const int b = fg & 1;
-        ok = __all_sync(0xffffffffu, wait_z(&accf[b], (fg >> 1) & 1, wait_ns, abort_f, err));
+        ok = __all_sync(0xffffffffu, wait_ab(&accf[b], (fg >> 1) & 1, wait_ns, abort_f, err));
         if (!ok) break;
         fence_after();
         // the scale of D_0 at (row, column) is 2^(eA + eB - 2060): as a biased
@@ -376,86 +317,37 @@ __global__ void __launch_bounds__(ZTHREADS, 1) gemm_tcz_kernel(const GGroup* __r
               hi[cb + i] = s2;
               lo[cb + i] = e2;
             } else {
-              two_sum_z(hi[cb + i], lo[cb + i], s2);
+              two_sum_into(hi[cb + i], lo[cb + i], s2);
               lo[cb + i] += e2;
             }
           }
         }
         fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive_z(&acce[b]);
+        if (lane == 0) mbar_arrive(&acce[b]);
         ++fg;
         ea = ean;
         eb = ebn;
       }
       if (!ok) break;
-      if (z.parts > 1) {
-        // this part's sums to scratch, 32 rows contiguous per column; the last
-        // part to arrive adds all of them in part order
-        const int t = w / split;
-        uint64_t* sc = scratch + ((size_t)t * split * ZEPI + (warp - 2)) * 1024 + lane;
-        uint64_t* mine = sc + (size_t)z.part * ZEPI * 1024;
-#pragma unroll
-        for (int i = 0; i < 32; ++i)
-          __stcg(mine + 32 * i, ((uint64_t)__float_as_uint(lo[i]) << 32) | (uint64_t)__float_as_uint(hi[i]));
-        __threadfence();
-        __syncwarp();
-        unsigned arrived = 0;
-        if (lane == 0) arrived = atomicInc(&tickets[t * ZEPI + warp - 2], z.parts - 1);
-        arrived = __shfl_sync(0xffffffffu, arrived, 0);
-        if (arrived != (unsigned)(z.parts - 1)) continue;
-        __threadfence();
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const uint64_t v = __ldcg(sc + 32 * i);
-          hi[i] = __uint_as_float((uint32_t)v);
-          lo[i] = __uint_as_float((uint32_t)(v >> 32));
-        }
-        for (int p = 1; p < z.parts; ++p) {
-          const uint64_t* o = sc + (size_t)p * ZEPI * 1024;
-#pragma unroll
-          for (int i = 0; i < 32; ++i) {
-            const uint64_t v = __ldcg(o + 32 * i);
-            two_sum_z(hi[i], lo[i], __uint_as_float((uint32_t)v));
-            lo[i] += __uint_as_float((uint32_t)(v >> 32));
-          }
-        }
-      }
-      // the finished 32 x 32 block, 16 columns at a time through this warp's
-      // staging buffer: one row per lane on the way in, 16 lanes per row (128
-      // contiguous bytes) on the way out
-      const bool accum = g.flags & 1;
-      const int c_l = lane & 15;
-      uint64_t* const Cb = reinterpret_cast<uint64_t*>(sel_base(bs, slot_of(g.C))) + off_of(g.C);
+      if (z.parts > 1 && !gather_parts(z, (blockIdx.x + i * gridDim.x) / split, split, ZEPI, warp - 2, scratch, tickets, hi, lo)) continue;
+      // the finished 32 x 32 block
 #pragma unroll
       for (int cb = 0; cb < 32; cb += 16) {
         if (PAIR) {
-#pragma unroll
-          for (int i = 0; i < 16; ++i)
-            stg[lane * 16 + (i ^ (lane & 15))] =
-                ((uint64_t)__float_as_uint(lo[cb + i]) << 32) | (uint64_t)__float_as_uint(hi[cb + i]);
+          store_block16(
+              stg,
+              [&](int k) {
+                return ((uint64_t)__float_as_uint(lo[cb + k]) << 32) | (uint64_t)__float_as_uint(hi[cb + k]);
+              },
+              reinterpret_cast<uint64_t*>(z.C), z.ldc, z.m0 + 32 * q, z.n0 + 32 * h + cb, z.M, z.N, false);
         } else {
+          double v[16];
 #pragma unroll
-          for (int i = 0; i < 16; ++i)
-            stg[lane * 16 + (i ^ (lane & 15))] =
-                (uint64_t)__double_as_longlong((double)hi[cb + i] + (double)lo[cb + i]);
+          for (int k = 0; k < 16; ++k) v[k] = dbl_of_pair(hi[cb + k], lo[cb + k]);
+          store_block16(stg, [&](int k) { return (uint64_t)__double_as_longlong(v[k]); },
+                        reinterpret_cast<double*>(z.C), z.ldc, z.m0 + 32 * q, z.n0 + 32 * h + cb, z.M, z.N, z.flags & 1);
         }
-        __syncwarp();
-        const int col = tl.n0 + 32 * h + cb + c_l;
-        for (int rr = lane >> 4; rr < 32; rr += 2) {
-          const int grow = tl.m0 + 32 * q + rr;
-          if (grow < g.M && col < g.N) {
-            const long long o = (long long)grow * g.ldc + col;
-            const uint64_t bits = stg[rr * 16 + (c_l ^ (rr & 15))];
-            if (PAIR || !accum) {
-              Cb[o] = bits;
-            } else {
-              double* Cp = reinterpret_cast<double*>(Cb + o);
-              *Cp += __longlong_as_double((long long)bits);
-            }
-          }
-        }
-        __syncwarp();
       }
     }
   }
@@ -495,7 +387,9 @@ size_t tcz_smem_bytes() { return (size_t)ZRING_BYTES + ZSTG_BYTES + 1024; }
 int tcz_split(int ntiles, int max_segs) {
   if (ntiles <= 0) return 1;
   const int room = sm_count_z() / ntiles;
-  return room < 2 || max_segs < 4 ? 1 : (room < max_segs / 2 ? room : max_segs / 2);
+  // at least four segments to a part: with two, six ladders stepped side by side
+  // (each CTA takes a whole SM) lost 4 % to the larger grids
+  return room < 2 || max_segs < 8 ? 1 : (room < max_segs / 4 ? room : max_segs / 4);
 }
 size_t tcz_scratch_bytes(int ntiles, int split) { return split > 1 ? (size_t)ntiles * split * ZBM * ZBN * 8 : 0; }
 size_t tcz_tickets(int ntiles) { return (size_t)ntiles * ZEPI; }
