@@ -608,7 +608,7 @@ def main():
                      "householder_fallbacks_per_step": s["qr_fallbacks"] / nprof,
                      "gemm_ms_per_step": s["qr_gemm_ms"] / nprof,
                      "gemm_tflops": (s["qr_gemm_flops"] / (s["qr_gemm_ms"] / 1e3) / 1e12) if s["qr_gemm_ms"] else None,
-                     "gemm_arithmetic": "fp64",
+                     "gemm_arithmetic": "fp64" if prec == 0 else "double-float (FP32 pipe) or fp64, the faster per plan",
                      "cholesky_ms_per_step": s["qr_chol_ms"] / nprof},
         "mixed_vs_fp64": check,
         "autotune": ({"plans_tcgen05_128x128": s["tuned_tc128"], "plans_tcgen05_persistent_128x64": s["tuned_tcp128x64"],

@@ -63,9 +63,9 @@ typedef enum {
                                 float sum.  In both modes the Lanczos vectors,
                                 Krylov exponential, SVD, absorb step,
                                 measurements and log-norm stay FP64; the
-                                CholeskyQR gauge has its GEMMs in FP64 and its
-                                factorisation in double-float (~2^-46), with a
-                                FP64 Householder fallback */
+                                CholeskyQR gauge runs in double-float (~2^-46;
+                                its smaller GEMMs in FP64, which is faster there)
+                                with a FP64 Householder fallback */
   TT_PREC_SPLIT_EXACT = 3    /* exact-accumulation split (Ozaki scheme): the
                                 H_eff and bond applies' operands as four
                                 fixed-point BF16 digits with one exponent per

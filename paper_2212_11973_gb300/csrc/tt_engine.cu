@@ -119,9 +119,10 @@ static std::vector<GTile> tiles64_of(const GemmPlan& p) {
   return tiles;
 }
 
-// The plan's arrays into a stager; the tile lists of the 64 x 64 kernels and, by
-// default, of the FP64 kernel follow when a launch first needs them.
-static void upload(Stager& s, GemmPlan p, DevGemmBuf& o, bool f64list = false) {
+// The plan's arrays into a stager, with the tile list of the kernel it is known
+// to run on (else the lists follow when a launch first needs them).
+enum TileList { TL_LATER = 0, TL_F64 = 1, TL_QR = 2 };  // TL_QR: FP64, and double-float where it is faster
+static void upload(Stager& s, GemmPlan p, DevGemmBuf& o, int list = TL_LATER) {
   s.add(p.groups, &o.d.groups);
   s.add(p.segs, &o.d.segs);
   o.d.ngroups = (int)p.groups.size();
@@ -132,7 +133,13 @@ static void upload(Stager& s, GemmPlan p, DevGemmBuf& o, bool f64list = false) {
   o.tc_checked = o.tc_ok = false;
   o.ntiles128 = o.ntilesp = 0;
   o.d.ntilesf = o.d.tf = 0;
-  if (f64list) {
+  o.d.ntilesd = -1;
+  if (list == TL_QR && df_beats_f64(p)) {
+    const std::vector<FTile> t = f64_tiles(p, df_tile_size());
+    s.add(t, &o.d.tilesd);
+    o.d.ntilesd = (int)t.size();
+  }
+  if (list == TL_F64 || (list == TL_QR && o.d.ntilesd < 0)) {
     const F64Shape sh = f64_shape(p);
     o.d.tf = sh.T;
     o.d.wkf = sh.wk;
@@ -205,6 +212,7 @@ void release(tt_ctx* c, DevGemmBuf& o) {
   dfree(c, o.tcbuf);
   dfree(c, o.tilesf);
   dfree(c, o.tiles64);
+  dfree(c, o.tilesd);
   o.d = DevGemm();
   o.host = GemmPlan();
   o.checked = o.tc_checked = o.tc_ok = false;
@@ -402,7 +410,8 @@ struct Eng {
   // ---- plans --------------------------------------------------------------
   // FP64 plans of site j whatever the precision (the measurement's energy)
   // a site's plans to the device, all in one buffer
-  void stage_site(SiteDev& s, bool f64list) {
+  void stage_site(SiteDev& s, bool fp64) {
+    const int f64list = fp64 ? TL_F64 : TL_LATER;
     Stager g;
     upload(g, s.h.xsplit, s.xs);
     upload(g, s.h.xdig, s.xd);
@@ -532,8 +541,8 @@ struct Eng {
       }
     }
     Stager g;
-    upload(g, std::move(b.h.b1), b.b1, !mixed());
-    upload(g, std::move(b.h.b2), b.b2, !mixed());
+    upload(g, std::move(b.h.b1), b.b1, mixed() ? TL_LATER : TL_F64);
+    upload(g, std::move(b.h.b2), b.b2, mixed() ? TL_LATER : TL_F64);
     if (mixed()) {
       upload(g, b.h.xsplit, b.xs);
       upload(g, b.h.tsplit, b.ts);
@@ -591,8 +600,8 @@ struct Eng {
       for (int p = 0; p < 3; ++p) {
         check_plan(cp.gram[p], cw, "CholQR gram");
         check_plan(cp.app[p], cw, "CholQR apply");
-        upload(g, std::move(cp.gram[p]), q.gram[p], true);
-        upload(g, std::move(cp.app[p]), q.app[p], true);
+        upload(g, std::move(cp.gram[p]), q.gram[p], TL_QR);
+        upload(g, std::move(cp.app[p]), q.app[p], TL_QR);
         for (const CholJob& J : cp.cj[p])
           if (J.g + (int64_t)J.parts * J.n * J.n > wsz || J.parts < 1 || J.r + (int64_t)J.n * J.n > wsz ||
               J.ri + (int64_t)J.n * J.n > wsz || J.pk < 0 || J.pk + (int64_t)J.n * (J.n + 1) / 2 > wsz)
@@ -604,8 +613,8 @@ struct Eng {
       }
       check_plan(cp.tt, cw, "CholQR T");
       check_plan(cp.rf, cw, "CholQR R");
-      upload(g, std::move(cp.tt), q.tt, true);
-      upload(g, std::move(cp.rf), q.rf, true);
+      upload(g, std::move(cp.tt), q.tt, TL_F64);
+      upload(g, std::move(cp.rf), q.rf, TL_F64);
       ensure(c, q.fail, q.h.jobs.size() * sizeof(int) + 16);
     }
     g.commit(c, q.arena);
@@ -617,7 +626,7 @@ struct Eng {
 
   void upload_f64(GemmPlan p, DevGemmBuf& o) {
     Stager s;
-    upload(s, std::move(p), o, true);
+    upload(s, std::move(p), o, TL_F64);
     s.commit(c, o.buf);
   }
   DevGemmBuf& absorb_left_plan(int j) {  // into site j from the bond on its left
@@ -809,7 +818,19 @@ struct Eng {
     }
     CK(launch_gemm_f64(g.d, b, st));
   }
-  // the plan with its list of 64 x 64 tiles (the mma.sync and double-float kernels)
+  // the plan with the double-float kernel's tile list
+  const DevGemm& withdf(DevGemmBuf& g) {
+    if (g.d.ntilesd < 0) {
+      if (r->capturing) throw Err{TT_ERR_STATE, "double-float tile list missing during graph capture"};
+      const std::vector<FTile> t = f64_tiles(g.host, df_tile_size());
+      Stager s;
+      s.add(t, &g.d.tilesd);
+      s.commit(c, g.tilesd);
+      g.d.ntilesd = (int)t.size();
+    }
+    return g.d;
+  }
+  // the plan with its list of 64 x 64 tiles (the mma.sync kernels)
   const DevGemm& with64(DevGemmBuf& g) {
     if (g.d.ntiles64 < 0) {
       if (r->capturing) throw Err{TT_ERR_STATE, "64 x 64 tile list missing during graph capture"};
@@ -948,7 +969,7 @@ struct Eng {
     } else if (f64_kernel == 1) {
       CK(launch_gemm_oz(with64(g), b, st));
     } else if (f64_kernel == 2) {
-      CK(launch_gemm_df(with64(g), b, st));
+      CK(launch_gemm_df(withdf(g), b, st));
     } else {
       f64(g, b);
     }
@@ -1231,9 +1252,15 @@ struct Eng {
       return;
     }
     CK(cudaMemsetAsync(q.fail.p, 0, q.h.jobs.size() * sizeof(int), st));
+    // the mixed modes run the large Gram and apply GEMMs in double-float on the
+    // FP32 pipe (their error budget is far above ~2^-46), the others in FP64
+    auto qr_gemm = [&](DevGemmBuf& g) {
+      if (mixed() && g.d.ntilesd >= 0) CK(launch_gemm_df(g.d, b, st));
+      else f64(g, b);
+    };
     for (int p = 0; p < 3; ++p) {
       long e = prof_begin(11, q.gram[p].d.flops);
-      f64(q.gram[p], b);
+      qr_gemm(q.gram[p]);
       prof_end(e);
       e = prof_begin(12, 0);
       // the mixed modes factorise in double-float (their error budget is far
@@ -1241,7 +1268,7 @@ struct Eng {
       CK(launch_chol_inv(q.cjobs[p], q.ncj[p], dptr(r->ws), (int*)q.fail.p, st, q.maxn[p], mixed()));
       prof_end(e);
       e = prof_begin(11, q.app[p].d.flops);
-      f64(q.app[p], b);
+      qr_gemm(q.app[p]);
       prof_end(e);
       count(3);
     }
@@ -2273,9 +2300,9 @@ struct Eng {
     DBuf arena;
     {
       Stager g;
-      upload(g, std::move(h.s1), s1, !mixed());
+      upload(g, std::move(h.s1), s1, mixed() ? TL_LATER : TL_F64);
       upload(g, h.s2, s2);
-      upload(g, std::move(h.s3), s3, !mixed());
+      upload(g, std::move(h.s3), s3, mixed() ? TL_LATER : TL_F64);
       upload(g, h.xsplit, xs);
       g.commit(c, arena);
     }

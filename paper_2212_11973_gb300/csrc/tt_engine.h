@@ -58,7 +58,7 @@ struct DevGemmBuf {
   DBuf tcbuf;  // tensor maps and both tile lists
   void* maps = nullptr;
   GTile *tiles128 = nullptr, *tilesp = nullptr;
-  DBuf tilesf, tiles64;  // tile lists of the FP64 and the 64 x 64 kernels, where not uploaded with the plan
+  DBuf tilesf, tiles64, tilesd;  // tile lists of the FP64, 64 x 64 and double-float kernels, where not uploaded with the plan
   int ntiles128 = 0, ntilesp = 0;  // 128 x 128 tiles (tc), 128 x 64 tiles (persistent tc)
   // autotuned kernel of a split-BF16 plan: -1 not chosen yet, else a TcKernel
   int choice = -1;

@@ -1,7 +1,7 @@
 // Device kernels of the tanTRG hot path (sm_103a).
 //
-//  * grouped, segmented GEMM (double-float on the FP32 pipe; split-BF16 on the
-//    tensor cores; FP64 in tt_gemm64.cu):
+//  * grouped, segmented GEMM (split-BF16 on the tensor cores; FP64 in
+//    tt_gemm64.cu, double-float in tt_gemmdf.cu):
 //    every contraction of the H_eff apply (Supplement, Fig. "Lanczos": L_i A_i,
 //    then H_i, then R_i), the bond apply (Fig. "optimalB"(d)), the environment
 //    updates and the absorb step is a list of groups C_g = sum_seg A_seg B_seg;
@@ -15,7 +15,6 @@
 #include <cstdint>
 #include <type_traits>
 
-#include "tt_df.h"
 #include "tt_kernels.h"
 
 namespace tt {
@@ -36,96 +35,6 @@ constexpr int VT = 256;
 __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
-}
-
-constexpr int FBM = 64, FBN = 64, FBK = 16;
-
-// ---------------------------------------------------------------------------
-// Grouped GEMM in double-float arithmetic on the FP32 pipe: one 64 x 64 output
-// tile per CTA, 256 threads, 4 x 4 per thread, K staged through shared memory
-// in chunks of 16 (GB300
-// issues ~2 FP64 FMA per clock per SM against 128 FP32): FP64 operands split
-// into float pairs (hi, lo) as they are staged, every product by the FMA
-// TwoProduct with the cross terms, every sum by TwoSum into an unnormalised
-// (hi, lo) accumulator (Dekker; Knuth TAOCP vol. 2, 4.2.2): ~2^-46 relative
-// per operation, K 2^-46 of sum |a| |b| per output.  Output FP64.  Used by the
-// environment updates with env_precision 2.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) gemm_df_kernel(const GGroup* __restrict__ groups, const GSeg* __restrict__ segs,
-                                                      const GTile* __restrict__ tiles, Bases bs) {
-  __shared__ float2 As[FBK][FBM + 1];
-  __shared__ float2 Bs[FBK][FBN + 1];
-  const GTile tl = tiles[blockIdx.x];
-  const GGroup g = groups[tl.g];
-  const int tid = threadIdx.x;
-  const int tx = tid % 16, ty = tid / 16;
-  float ah_[4][4], al_[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) { ah_[i][j] = 0.f; al_[i][j] = 0.f; }
-
-  for (int si = g.seg0; si < g.seg1; ++si) {
-    const GSeg sg = segs[si];
-    const double* A = rptr<const double>(bs, sg.A);
-    const double* B = rptr<const double>(bs, sg.B);
-    for (int k0 = 0; k0 < sg.K; k0 += FBK) {
-      for (int e = tid; e < FBM * FBK; e += 256) {
-        int mm, kk;
-        if (sg.tA) { mm = e % FBM; kk = e / FBM; } else { kk = e % FBK; mm = e / FBK; }
-        const int gm = tl.m0 + mm, gk = k0 + kk;
-        double v = 0.0;
-        if (gm < g.M && gk < sg.K) v = sg.tA ? A[(long long)gk * sg.lda + gm] : A[(long long)gm * sg.lda + gk];
-        As[kk][mm] = df_split(v);
-      }
-      for (int e = tid; e < FBN * FBK; e += 256) {
-        int nn, kk;
-        if (sg.tB) { kk = e % FBK; nn = e / FBK; } else { nn = e % FBN; kk = e / FBN; }
-        const int gn = tl.n0 + nn, gk = k0 + kk;
-        double v = 0.0;
-        if (gn < g.N && gk < sg.K) v = sg.tB ? B[(long long)gn * sg.ldb + gk] : B[(long long)gk * sg.ldb + gn];
-        Bs[kk][nn] = df_split(v);
-      }
-      __syncthreads();
-#pragma unroll 4
-      for (int kk = 0; kk < FBK; ++kk) {
-        float2 a[4], b[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const float p = a[i].x * b[j].x;
-            float e = fmaf(a[i].x, b[j].x, -p);
-            e = fmaf(a[i].x, b[j].y, e);
-            e = fmaf(a[i].y, b[j].x, e);
-            const float s = ah_[i][j] + p;
-            const float bp = s - ah_[i][j];
-            al_[i][j] += ((ah_[i][j] - (s - bp)) + (p - bp)) + e;
-            ah_[i][j] = s;
-          }
-      }
-      __syncthreads();
-    }
-  }
-  double* C = rptr<double>(bs, g.C);
-  const bool accum = g.flags & 1;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int gm = tl.m0 + ty + 16 * i;
-    if (gm >= g.M) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int gn = tl.n0 + tx + 16 * j;
-      if (gn >= g.N) continue;
-      double* c = C + (long long)gm * g.ldc + gn;
-      const double v = (double)ah_[i][j] + (double)al_[i][j];
-      *c = accum ? *c + v : v;
-    }
-  }
 }
 
 // ---------------------------------------------------------------------------
@@ -645,12 +554,6 @@ inline int grid_for(long long n) {
 // host wrappers
 // ---------------------------------------------------------------------------
 int lanczos_nblk() { return NBLK; }
-
-cudaError_t launch_gemm_df(const DevGemm& g, const Bases& b, cudaStream_t s) {
-  if (g.ntiles64 == 0) return cudaSuccess;
-  gemm_df_kernel<<<g.ntiles64, 256, 0, s>>>(g.groups, g.segs, g.tiles64, b);
-  return cudaGetLastError();
-}
 
 cudaError_t launch_gemm_bf16(const DevGemm& g, const Bases& b, int nsplit, cudaStream_t s) {
   if (g.ntiles64 == 0) return cudaSuccess;

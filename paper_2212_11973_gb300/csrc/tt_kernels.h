@@ -40,8 +40,9 @@ struct DevGemm {
   GGroup* groups = nullptr;
   GSeg* segs = nullptr;
   GTile* tiles64 = nullptr;   // 64 x 64 output tiles
+  FTile* tilesd = nullptr;    // double-float kernel's tiles
   FTile* tilesf = nullptr;    // FP64 kernel: tf x tf output tiles on wkf warps
-  int ngroups = 0, nsegs = 0, ntiles64 = 0, ntilesf = 0, tf = 0, wkf = 0;
+  int ngroups = 0, nsegs = 0, ntiles64 = 0, ntilesf = 0, tf = 0, wkf = 0, ntilesd = -1;
   double flops = 0;
 };
 struct DevGather {
@@ -100,7 +101,11 @@ struct F64Shape {
 F64Shape f64_shape(const GemmPlan& p);
 std::vector<FTile> f64_tiles(const GemmPlan& p, int T);
 cudaError_t launch_gemm_f64(const DevGemm& g, const Bases& b, cudaStream_t s);
-// The same in double-float arithmetic on the FP32 pipe (~2^-46 per operation).
+// The same in double-float arithmetic on the FP32 pipe (~2^-46 per operation),
+// on f64_tiles(plan, df_tile_size()).
+int df_tile_size();
+// whether the double-float kernel is the faster one for a plan
+bool df_beats_f64(const GemmPlan& p);
 cudaError_t launch_gemm_df(const DevGemm& g, const Bases& b, cudaStream_t s);
 // Exact-accumulation split GEMM (tt_ozaki.cu): FP64 operands of the FP64
 // plans, four fixed-point BF16 digits per K tile, ~2^-32 normwise.

@@ -523,12 +523,12 @@ QrPlanHost build_lq_right(const SiteLayout& S, const Bond& BL, bool shrink) {
 
 CholQrPlan build_cholqr(const std::vector<QrJob>& jobs, int64_t ws0) {
   // Per sector (m x n, column-major X):
-  //   G = X^T X: only the upper block triangle (row blocks of 64, columns from
+  //   G = X^T X: only the upper block triangle (row blocks of 32, columns from
   //   the block's first row on), K split into `parts` chunks that write
   //   separate partial Gram matrices (summed by the Cholesky kernel);
   //   Xo^T = RI^T X^T: RI is upper triangular, so output row block q0 needs
-  //   K = min(n, q0 + 64) only.
-  constexpr int RB = 64, KCHUNK = 512, MAXPARTS = 16;
+  //   K = min(n, q0 + 32) only.
+  constexpr int RB = 32, KCHUNK = 512, MAXPARTS = 16;
   CholQrPlan P;
   int64_t w = ws0;
   for (size_t sec = 0; sec < jobs.size(); ++sec) {
