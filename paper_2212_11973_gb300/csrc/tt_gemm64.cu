@@ -26,10 +26,11 @@
 // Measured against 64 x 64 DFMA tiles with a K loop per CTA (which padded a
 // sector of 12 to 64 and left most SMs idle behind a few long tiles): FP64
 // beta-step of a 4x8 cylinder at D = 256 961 -> 162 ms (140 -> 135 ms by the
-// one-warp tiles later), of the 2x2 cluster at D = 64 24.3 -> 5.4 ms; measurement and QR factors of a D = 300 exact-split
-// step 249 -> 217 ms.  The mixed modes' CholeskyQR Gram and apply products run
-// here too since: as double-float on 64 x 64 tiles they took 31 ms of a D = 300
-// step and 43 of a D = 512 one, here 4 and 10 (and the same 31 ms at D = 1024).
+// one-warp tiles later), of the 2x2 cluster at D = 64 24.3 -> 5.4 ms;
+// measurement and QR factors of a D = 300 exact-split step 249 -> 217 ms.  The
+// smaller CholeskyQR products of the mixed modes run here too (df_beats_f64
+// draws the line): double-float on 64 x 64 tiles took 31 ms of a D = 300 step
+// and 43 of a D = 512 one, here 4 and 10.
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -211,8 +211,18 @@ static __device__ __forceinline__ uint64_t desc_of(uint32_t saddr) {
   return d;
 }
 
+// Segments of part `part` of `parts`: every parts-th pair of the group's, so that
+// the split-BF16 kernel's fold groups are those of an undivided tile where every
+// segment is one piece.
+static __device__ __forceinline__ int part_count(int nseg, int split) { return max(1, min(split, (nseg + 1) >> 1)); }
+static __device__ __forceinline__ int part_segs(int nseg, int parts, int part) {
+  const int pairs = (nseg + 1) >> 1;
+  if (part >= parts || nseg == 0) return 0;
+  return 2 * ((pairs - part + parts - 1) / parts) - ((nseg & 1) && (pairs - 1) % parts == part ? 1 : 0);
+}
+
 // One part of a tile and what the roles need of its group and first segment:
-// segments seg0, seg0 + parts, ... (n of them).
+// segments seg(0) .. seg(n - 1).
 struct TileItem {
   void* C;                 // output of the group
   const short *pa, *pb;    // row exponents of the first segment's operands (digits)
@@ -220,6 +230,7 @@ struct TileItem {
   int ldc, flags;
   int seg0, parts, part, n;
   int K0, eas, ebs;        // first segment
+  __device__ __forceinline__ int seg(int s) const { return seg0 + (s >> 1) * 2 * parts + (s & 1); }
 };
 static __device__ __forceinline__ const short* exps_ptr(const Bases& bs, Ref r) {
   return reinterpret_cast<const short*>(sel_base(bs, slot_of(r))) + off_of(r);
@@ -231,9 +242,9 @@ static __device__ __forceinline__ TileItem load_item(const GGroup* groups, const
   const GGroup g = groups[tl.g];
   const int nseg = g.seg1 - g.seg0;
   it.part = w % split;
-  it.parts = max(1, min(split, nseg));
-  it.n = it.part < it.parts ? (nseg - it.part + it.parts - 1) / it.parts : 0;
-  it.seg0 = g.seg0 + it.part;
+  it.parts = part_count(nseg, split);
+  it.n = part_segs(nseg, it.parts, it.part);
+  it.seg0 = g.seg0 + 2 * it.part;
   it.C = reinterpret_cast<char*>(sel_base(bs, slot_of(g.C))) + off_of(g.C) * esize;  // esize: bytes of an output
   it.m0 = tl.m0;
   it.n0 = tl.n0;
@@ -270,10 +281,11 @@ static __device__ __forceinline__ void fence_maps(const CUtensorMap* maps, int s
 static __device__ __forceinline__ int first_segments(const GGroup* groups, const GSeg* segs, const GTile* tiles,
                                                      const CUtensorMap* maps, int split) {
   const GGroup g = groups[tiles[blockIdx.x / split].g];
-  const int nseg = g.seg1 - g.seg0, parts = max(1, min(split, nseg)), part = blockIdx.x % split;
-  const int n = part < parts ? (nseg - part + parts - 1) / parts : 0;
+  const int nseg = g.seg1 - g.seg0, parts = part_count(nseg, split), part = blockIdx.x % split;
+  const int n = part_segs(nseg, parts, part);
   if (n == 0) return 0;
-  const int s = g.seg0 + part + min((int)(threadIdx.x & 31), n - 1) * parts;
+  const int at = min((int)(threadIdx.x & 31), n - 1);
+  const int s = g.seg0 + 2 * part + (at >> 1) * 2 * parts + (at & 1);
   fence_maps(maps, s);
   return segs[s].K;
 }

@@ -1,6 +1,6 @@
 // Persistent, warp-specialised split-BF16 grouped GEMM on the 5th-generation
 // tensor cores (sm_103a): operands as NS bf16 levels, the level products l_A +
-// l_B < NS, folded every 128 of K at most into a two-float TwoSum sum.
+// l_B < NS, folded every two pieces of at most 64 of K into a two-float TwoSum sum.
 //
 // Laid out as the digit kernel (tt_tcgen05z.cu): one CTA per SM walks 128 x 64
 // output tiles; warp 0 streams the level tiles by TMA into a ring of
@@ -40,7 +40,7 @@ namespace {
 
 using namespace tcx;
 
-constexpr int PBM = 128, PBN = 64, PFOLD_K = 128;
+constexpr int PBM = 128, PBN = 64, PIECE = 64;  // two pieces to a fold group
 constexpr uint32_t PTMEM_COLS = 512;
 constexpr int PEPI = 8;  // epilogue warps
 constexpr int PTHREADS = 64 + 32 * PEPI;
@@ -55,12 +55,12 @@ struct PCfg {
   static constexpr int STAGES = (int)((PSMEM - PSTG_BYTES - 1024) / STAGE_BYTES);
 };
 
-// K chunks of the tile part: the sum over its segments, by the whole warp
-template <int BK>
-__device__ __forceinline__ int part_chunks(const TileItem& q, const GSeg* segs) {
-  if (q.n <= 1) return (q.K0 + BK - 1) / BK;
+// Pieces (at most PIECE of K each, within a segment) of the tile part: the sum over
+// its segments, by the whole warp
+__device__ __forceinline__ int part_pieces(const TileItem& q, const GSeg* segs) {
+  if (q.n <= 1) return (q.K0 + PIECE - 1) / PIECE;
   int t = 0;
-  for (int s = threadIdx.x & 31; s < q.n; s += 32) t += (segs[q.seg0 + s * q.parts].K + BK - 1) / BK;
+  for (int s = threadIdx.x & 31; s < q.n; s += 32) t += (segs[q.seg(s)].K + PIECE - 1) / PIECE;
   return __reduce_add_sync(0xffffffffu, t);
 }
 
@@ -74,7 +74,7 @@ __global__ void __launch_bounds__(PTHREADS, 1) gemm_tcp_kernel(const GGroup* __r
                                                                unsigned* __restrict__ tickets, int* __restrict__ err,
                                                                long long wait_ns) {
   using C = PCfg<NS, BK>;
-  constexpr int S = C::STAGES, FOLD = PFOLD_K / BK;  // chunks per fold group
+  constexpr int S = C::STAGES;
   constexpr int BUF = 64 * NS;                       // TMEM columns of one accumulator buffer
   static_assert(S >= 2 && 2 * BUF <= (int)PTMEM_COLS, "stages and accumulators");
   extern __shared__ uint8_t smem_raw[];
@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(PTHREADS, 1) gemm_tcp_kernel(const GGroup* __r
         if (i == 0 && s0 == 0) {
           kl = kl0;
         } else if (q.n > 1 || i >= TITEMS) {
-          const int sl = q.seg0 + min(s0 + lane, q.n - 1) * q.parts;
+          const int sl = q.seg(min(s0 + lane, q.n - 1));
           kl = segs[sl].K;
           fence_maps(maps, sl);
           __syncwarp();
@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(PTHREADS, 1) gemm_tcp_kernel(const GGroup* __r
         for (int s = s0; s < min(q.n, s0 + 32); ++s) {
           const int K = __shfl_sync(0xffffffffu, kl, s - s0);
           if (lane == 0) {
-            const CUtensorMap* ma = maps + 4 * (q.seg0 + s * q.parts) + 3;
+            const CUtensorMap* ma = maps + 4 * q.seg(s) + 3;
             const CUtensorMap* mb = ma - 1;
             for (int k0 = 0; k0 < K; k0 += BK) {
               const int sg = it % S;
@@ -174,15 +174,15 @@ __global__ void __launch_bounds__(PTHREADS, 1) gemm_tcp_kernel(const GGroup* __r
     bool ok = true;
     for (int i = 0; blockIdx.x + i * gridDim.x < nitems && ok; ++i) {
       const TileItem& q = item(i);
-      int kl = q.K0, c = 0;  // c: chunk within the part; a fold group is FOLD chunks
-      const int T = part_chunks<BK>(q, segs);
+      int kl = q.K0, c = 0;  // c: piece within the part
+      const int T = part_pieces(q, segs);
       for (int s = 0; s < q.n && ok; ++s) {
-        if ((s & 31) == 0 && q.n > 1) kl = segs[q.seg0 + min(s + lane, q.n - 1) * q.parts].K;
+        if ((s & 31) == 0 && q.n > 1) kl = segs[q.seg(min(s + lane, q.n - 1))].K;
         const int K = __shfl_sync(0xffffffffu, kl, s & 31);
         if (lane == 0) {
-          for (int k0 = 0; k0 < K && ok; k0 += BK, ++c) {
+          for (int k0 = 0; k0 < K && ok; k0 += BK) {
             const int b = fg & 1;
-            const bool first = c % FOLD == 0;
+            const bool first = (c & 1) == 0 && k0 % PIECE == 0;
             if (first) {
               ok = wait_ab(&acce[b], ((fg >> 1) & 1) ^ 1, wait_ns, abort_f, err);
               if (!ok) break;
@@ -205,7 +205,9 @@ __global__ void __launch_bounds__(PTHREADS, 1) gemm_tcp_kernel(const GGroup* __r
             umma_commit(&empty_bar[sg]);
             last_commit_s = it;
             ++it;
-            if (c % FOLD == FOLD - 1 || c == T - 1) {
+            if (k0 + BK < K && (k0 + BK) % PIECE != 0) continue;  // the piece goes on
+            ++c;
+            if ((c & 1) == 0 || c == T) {
               umma_commit(&accf[b]);
               last_accf_s = fg;
               ++fg;
@@ -229,7 +231,7 @@ __global__ void __launch_bounds__(PTHREADS, 1) gemm_tcp_kernel(const GGroup* __r
       if (z.part >= z.parts) continue;
 #pragma unroll
       for (int i = 0; i < 32; ++i) { hi[i] = 0.f; lo[i] = 0.f; }
-      const int units = (part_chunks<BK>(z, segs) + FOLD - 1) / FOLD;
+      const int units = (part_pieces(z, segs) + 1) / 2;
       for (int f = 0; f < units; ++f) {
         const int b = fg & 1;
         ok = __all_sync(0xffffffffu, wait_ab(&accf[b], (fg >> 1) & 1, wait_ns, abort_f, err));

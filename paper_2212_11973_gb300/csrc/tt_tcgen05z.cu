@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(ZTHREADS, 1) gemm_tcz_kernel(const GGroup* __r
         if (i == 0 && s0 == 0) {
           kl = kl0;
         } else if (q.n > 1 || i >= TITEMS) {
-          const int sl = q.seg0 + min(s0 + lane, q.n - 1) * q.parts;
+          const int sl = q.seg(min(s0 + lane, q.n - 1));
           kl = segs[sl].K;
           fence_maps(maps, sl);
           __syncwarp();
@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(ZTHREADS, 1) gemm_tcz_kernel(const GGroup* __r
         for (int s = s0; s < min(q.n, s0 + 32); ++s) {
           const int K = __shfl_sync(0xffffffffu, kl, s - s0);
           if (lane == 0) {
-            const CUtensorMap* ma = maps + 4 * (q.seg0 + s * q.parts) + 3;
+            const CUtensorMap* ma = maps + 4 * q.seg(s) + 3;
             const CUtensorMap* mb = ma - 1;
             for (int k0 = 0; k0 < K; k0 += ZBK) {
               const int sg = it % ZSTAGES;
@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(ZTHREADS, 1) gemm_tcz_kernel(const GGroup* __r
       const TileItem& q = item(i);
       int kl = q.K0;
       for (int s = 0; s < q.n && ok; ++s) {
-        if ((s & 31) == 0 && q.n > 1) kl = segs[q.seg0 + min(s + lane, q.n - 1) * q.parts].K;
+        if ((s & 31) == 0 && q.n > 1) kl = segs[q.seg(min(s + lane, q.n - 1))].K;
         const int K = __shfl_sync(0xffffffffu, kl, s & 31);
         if (lane == 0) {
           const int b = fg & 1;
@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(ZTHREADS, 1) gemm_tcz_kernel(const GGroup* __r
       unsigned long long ral = 0, rbl = 0;
       int sal = 0, sbl = 0;
       auto refs = [&](int s) {
-        const GSeg* sp = segs + z.seg0 + min(s + lane, z.n - 1) * z.parts;
+        const GSeg* sp = segs + z.seg(min(s + lane, z.n - 1));
         ral = reinterpret_cast<unsigned long long>(exps_ptr(bs, sp->eA));
         rbl = reinterpret_cast<unsigned long long>(exps_ptr(bs, sp->eB));
         sal = sp->eas;
