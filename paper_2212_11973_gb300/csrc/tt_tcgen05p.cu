@@ -16,7 +16,7 @@
 //
 // What bounds it: the chain of segments (18 to 42 of K = 3 to 180) behind each
 // tile; see the digit kernel.  D = 512, all four launches of an H_eff and a bond
-// apply, average: 29 -> 24 us from one lane fencing and loading each segment's
+// apply, average: 29 -> 25 us from one lane fencing and loading each segment's
 // maps, K chunks of 64 throughout, six MMAs per 16 K and rows stored as they came
 // (S1, whose tiles have one segment each and are bound by their output, 23 us; with
 // the shared-memory reads of the output one by one it took 40).
