@@ -39,31 +39,45 @@ __device__ __forceinline__ double dbl_of_float(float f) {
 }
 
 // hi + lo as FP64 by integer operations (two conversions and an addition on the
-// FP64 pipe cost 192 clocks of an SM sub-partition per warp): renormalised by
-// TwoSum to |t| <= ulp(s) / 2, then the mantissas added, t's truncated at 2^-53 of
-// s.  Infinities and NaN pass through; FP32 subnormals give zero.
-__device__ __forceinline__ double dbl_of_pair(float hi, float lo) {
+// FP64 pipe cost 192 clocks of an SM sub-partition per warp): renormalised by TwoSum
+// to |t| <= ulp(s) / 2, then the mantissas added and rounded at half an ulp of the
+// result (to nearest; of t what lies below half an ulp is dropped, error below 2^-53
+// of the sum).  Sums outside [2^-71, 2^128) set `fp64` (the result is then no use):
+// columns that a state gives no weight go down to FP32 subnormals and beyond, and
+// their direction counts.
+__device__ __forceinline__ double pair_bits(float hi, float lo, bool& fp64) {
   const float s = hi + lo;
   const float bp = s - hi;
   const float t = (hi - (s - bp)) + (lo - bp);
   const unsigned us = __float_as_uint(s), ut = __float_as_uint(t);
-  int es = (us >> 23) & 0xFF;
-  const int et = (ut >> 23) & 0xFF;
-  const unsigned sign = us & 0x80000000u;
-  if (es == 0) return 0.0;
-  if (es == 255)
-    return __hiloint2double((int)(sign | 0x7FF00000u | ((us & 0x7FFFFFu) >> 3)), (int)(us << 29));
-  const unsigned mt = et ? (ut & 0x7FFFFFu) | 0x800000u : 0u;
-  const int sh = es - et - 29;  // >= -5
-  const unsigned T = sh >= 0 ? (sh < 32 ? mt >> sh : 0u) : mt << -sh;
-  unsigned long long m = (unsigned long long)((us & 0x7FFFFFu) | 0x800000u) << 29;
-  m = ((us ^ ut) >> 31) ? m - T : m + T;
-  if (!(m >> 52)) {  // s a power of two, t of the other sign
-    m <<= 1;
-    --es;
+  const int es = (us >> 23) & 0xFF;
+  fp64 = fp64 || ((unsigned)(es - 56) > 198u && s != 0.f);
+  // in units of 2^-53 of s's leading bit: s in bits 30 .. 53, t at es - et >= 24
+  // below it (none of it from 56 on; a zero t has et = 0)
+  const unsigned T = __funnelshift_rc((ut & 0x7FFFFFu) << 6 | 0x20000000u, 0u, es - (int)((ut >> 23) & 0xFF) - 24);
+  const unsigned long long ms = (unsigned long long)((us & 0x7FFFFFu) | 0x800000u) << 30;
+  const unsigned long long m = ((us ^ ut) >> 31) ? ms - T : ms + T;
+  const bool low = !(m >> 53);  // s a power of two, t of the other sign
+  // (53 bits; the leading one, or a carry out of them, goes into the exponent)
+  const unsigned long long v = ((unsigned long long)(es + (low ? 894 : 895)) << 52) + (low ? m : (m + 1) >> 1);
+  return __longlong_as_double(
+      (long long)(((unsigned long long)(us & 0x80000000u) << 32) + (s == 0.f ? 0ull : v)));
+}
+__device__ __forceinline__ double dbl_of_pair(float hi, float lo) {
+  bool fp64 = false;
+  const double v = pair_bits(hi, lo, fp64);
+  return fp64 ? (double)hi + (double)lo : v;
+}
+// of N pairs, with one branch for all of them
+template <int N>
+__device__ __forceinline__ void dbl_of_pairs(const float* hi, const float* lo, double* v) {
+  bool fp64 = false;
+#pragma unroll
+  for (int i = 0; i < N; ++i) v[i] = pair_bits(hi[i], lo[i], fp64);
+  if (fp64) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) v[i] = (double)hi[i] + (double)lo[i];
   }
-  return __longlong_as_double((long long)(((unsigned long long)sign << 32) | ((unsigned long long)(es + 896) << 52) |
-                                          (m & 0xFFFFFFFFFFFFFull)));
 }
 
 }  // namespace tt

@@ -269,8 +269,7 @@ __global__ void __launch_bounds__(PTHREADS, 1) gemm_tcp_kernel(const GGroup* __r
                         reinterpret_cast<float*>(z.C), z.ldc, z.m0 + 32 * q, z.n0 + 32 * h + cb, z.M, z.N, z.flags & 1);
         } else {
           double v[16];
-#pragma unroll
-          for (int k = 0; k < 16; ++k) v[k] = dbl_of_pair(hi[cb + k], lo[cb + k]);
+          dbl_of_pairs<16>(hi + cb, lo + cb, v);
           store_block16(stg, [&](int k) { return (uint64_t)__double_as_longlong(v[k]); },
                         reinterpret_cast<double*>(z.C), z.ldc, z.m0 + 32 * q, z.n0 + 32 * h + cb, z.M, z.N, z.flags & 1);
         }
