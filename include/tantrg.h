@@ -235,7 +235,10 @@ tt_status tt_rho_grow_exp(tt_rho* rho, const tt_mpo* mpo, double ratio, double b
  * D_target / D, within what the neighbouring blocks can hold) with zero-weight
  * orthonormal completions; the state is unchanged, the 1-TDVP manifold larger
  * (the sweeps then populate the new directions).  Used to reach a large D
- * without a two-site sweep at that D.  Canonical centre must be on site 0. */
+ * without a two-site sweep at that D.  Canonical centre must be on site 0.
+ * The next beta-step, in which rounding chooses the null directions, runs in a
+ * fixed order of arithmetic (also after a save and load) and is not captured; a
+ * state that nothing but tt_rho_create has touched is made again in it. */
 tt_status tt_rho_pad(tt_rho* rho, const tt_mpo* mpo, int D_target);
 
 /* n_steps 1-TDVP beta-steps of size dtau (main text, linear stage; one

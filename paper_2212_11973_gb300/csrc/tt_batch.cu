@@ -248,12 +248,13 @@ tt_status tt_batch_pad(tt_batch* b) {
 tt_status tt_batch_step(tt_batch* b, double dtau, int n_steps) {
   if (!b || !(dtau > 0) || n_steps < 0) return TT_ERR_INVALID_ARG;
   int s = 0;
-  if (n_steps > 0 && !parent_current(b, dtau)) {
-    // one step per instance (captures or re-captures the instance graphs),
-    // then the parent graph from them when every instance has one
+  // one step per instance (captures or re-captures the instance graphs), then the
+  // parent graph from them when every instance has one; a second one after a
+  // padding, whose first step is not captured
+  for (int tries = 0; tries < 2 && s < n_steps && !parent_current(b, dtau); ++tries) {
     tt_status r = step_per_instance(b, dtau, 1);
     if (r != TT_OK) return r;
-    s = 1;
+    ++s;
     build_parent(b, dtau);
   }
   if (s == n_steps) return TT_OK;

@@ -68,12 +68,14 @@ __device__ __forceinline__ double dbl_of_pair(float hi, float lo) {
   const double v = pair_bits(hi, lo, fp64);
   return fp64 ? (double)hi + (double)lo : v;
 }
-// of N pairs, with one branch for all of them
+// of N pairs, with one branch for all of them; exact: rounded as an FP64 addition
 template <int N>
-__device__ __forceinline__ void dbl_of_pairs(const float* hi, const float* lo, double* v) {
-  bool fp64 = false;
+__device__ __forceinline__ void dbl_of_pairs(const float* hi, const float* lo, double* v, bool exact) {
+  bool fp64 = exact;
+  if (!exact) {
 #pragma unroll
-  for (int i = 0; i < N; ++i) v[i] = pair_bits(hi[i], lo[i], fp64);
+    for (int i = 0; i < N; ++i) v[i] = pair_bits(hi[i], lo[i], fp64);
+  }
   if (fp64) {
 #pragma unroll
     for (int i = 0; i < N; ++i) v[i] = (double)hi[i] + (double)lo[i];

@@ -30,15 +30,6 @@ __device__ __forceinline__ long long off_of(Ref r) { return (long long)(r & 0x00
 __device__ __forceinline__ int dexp(double v) {
   return (int)((static_cast<unsigned long long>(__double_as_longlong(v)) >> 52) & 0x7FF);
 }
-// biased FP64 exponent of a float (0 for zero / subnormal)
-__device__ __forceinline__ int fexp(float v) {
-  const int e = (__float_as_int(v) >> 23) & 0xFF;
-  return e == 0 ? 0 : e + 896;
-}
-
-// 2^x for -126 <= x <= 127 from the exponent field
-__device__ __forceinline__ float p2f(int x) { return __int_as_float((x + 127) << 23); }
-
 constexpr int DT = 256;
 
 constexpr int GMAXC = 256;  // longest digit row (segment) of the exact path
@@ -54,6 +45,7 @@ constexpr int GMAXC = 256;  // longest digit row (segment) of the exact path
 // Measured with one CTA per part instead of a grid sized by the largest item,
 // and digits by byte permutes: D = 1024 site tensor and environments 32 -> 8 us
 // a launch on average, D = 300 9.1 -> 4.2 us.
+template <bool TOPDOWN>
 __global__ void __launch_bounds__(DT) digit_copy_kernel(const DItem* __restrict__ items,
                                                         const CPart* __restrict__ parts, Bases bs) {
   const CPart part = parts[blockIdx.x];
@@ -86,8 +78,8 @@ __global__ void __launch_bounds__(DT) digit_copy_kernel(const DItem* __restrict_
         const int k = 2 * lane + 64 * i;
         if (k < it.cols) {
           uint32_t d0[4], d1[4];
-          fixed_digit_bits(v[i][0], m, d0);
-          fixed_digit_bits(v[i][1], m, d1);
+          fixed_digit_bits<TOPDOWN>(v[i][0], m, d0);
+          fixed_digit_bits<TOPDOWN>(v[i][1], m, d1);
 #pragma unroll
           for (int lv = 0; lv < 4; ++lv) dst[lv * lo2 + r * drs2 + (k >> 1)] = __byte_perm(d0[lv], d1[lv], 0x7632);
         }
@@ -130,8 +122,8 @@ __global__ void __launch_bounds__(DT) digit_copy_kernel(const DItem* __restrict_
 #pragma unroll
         for (int q = 0; q < 8; q += 2) {
           uint32_t d0[4], d1[4];
-          fixed_digit_bits(v[i][q], e, d0);
-          fixed_digit_bits(v[i][q + 1], e, d1);
+          fixed_digit_bits<TOPDOWN>(v[i][q], e, d0);
+          fixed_digit_bits<TOPDOWN>(v[i][q + 1], e, d1);
 #pragma unroll
           for (int lv = 0; lv < 4; ++lv) stg[lv][lane][4 * warp + q / 2] = __byte_perm(d0[lv], d1[lv], 0x7632);
         }
@@ -147,38 +139,7 @@ __global__ void __launch_bounds__(DT) digit_copy_kernel(const DItem* __restrict_
   }
 }
 
-// two-float c (hi, lo) += coef * (xh + xl), coef split into (ch, cl)
-__device__ __forceinline__ void df_fma(float& sh, float& sl, float ch, float cl, float xh, float xl) {
-  const float p = ch * xh;
-  const float pe = fmaf(ch, xh, -p) + (ch * xl + cl * xh);
-  const float s = sh + p;
-  const float bp = s - sh;
-  const float ap = s - bp;
-  sl += ((sh - ap) + (p - bp)) + pe;
-  sh = s;
-}
-
 constexpr int GMAXK = 64;   // most MPO coefficients of one item (split in shared memory)
-
-// Balanced base-256 digits of round(S + Sl) (a normalised two-float value,
-// |Sl| <= ulp(S) / 2, |S| < 2^31, scaled so that the row's bound is 2^31), in
-// FP32 arithmetic only: every step is exact, the roundings are those of rintf.  Returned as the BF16 bit
-// patterns (the digits are integers of magnitude <= 256, so their FP32 and
-// BF16 forms agree in the upper 16 bits).
-__device__ __forceinline__ void digits_of_pair(float S, float Sl, uint32_t* d) {
-  const float R = rintf(S);
-  const float f = (S - R) + Sl;
-  const float a0 = rintf(R * 5.9604644775390625e-08f);   // R / 2^24
-  const float rem = (R - a0 * 16777216.f) + rintf(f);    // |rem| < 2^24
-  const float a1 = rintf(rem * 1.52587890625e-05f);      // rem / 2^16
-  const float r1 = rem - a1 * 65536.f;
-  const float a2 = rintf(r1 * 0.00390625f);              // r1 / 2^8
-  const float a3 = r1 - a2 * 256.f;
-  d[0] = __float_as_uint(a0);
-  d[1] = __float_as_uint(a1);
-  d[2] = __float_as_uint(a2);
-  d[3] = __float_as_uint(a3);
-}
 
 // One CTA per item (or share of its rows).  Each row is taken by a group of G
 // lanes (G the smallest power of two with 2 G >= cols, at most 32), two adjacent
@@ -328,9 +289,10 @@ __global__ void __launch_bounds__(DT) gather_digits_kernel(const GItem* __restri
 
 }  // namespace
 
-cudaError_t launch_digit_copy(const DevDigit& d, const Bases& b, cudaStream_t s) {
+cudaError_t launch_digit_copy(const DevDigit& d, const Bases& b, cudaStream_t s, bool topdown) {
   if (d.nparts == 0) return cudaSuccess;
-  digit_copy_kernel<<<d.nparts, DT, 0, s>>>(d.items, d.parts, b);
+  if (topdown) digit_copy_kernel<true><<<d.nparts, DT, 0, s>>>(d.items, d.parts, b);
+  else digit_copy_kernel<false><<<d.nparts, DT, 0, s>>>(d.items, d.parts, b);
   return cudaGetLastError();
 }
 

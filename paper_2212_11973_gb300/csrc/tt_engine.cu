@@ -132,14 +132,16 @@ static void upload(Stager& s, GemmPlan p, DevGemmBuf& o, int list = TL_LATER) {
   o.checked = false;
   o.tc_checked = o.tc_ok = false;
   o.ntiles128 = o.ntilesp = 0;
+  o.nordered = o.tordered = 0;
   o.d.ntilesf = o.d.tf = 0;
   o.d.ntilesd = -1;
-  if (list == TL_QR && df_beats_f64(p)) {
+  o.df = list == TL_QR && df_beats_f64(p);
+  if (o.df) {
     const std::vector<FTile> t = f64_tiles(p, df_tile_size());
     s.add(t, &o.d.tilesd);
     o.d.ntilesd = (int)t.size();
   }
-  if (list == TL_F64 || (list == TL_QR && o.d.ntilesd < 0)) {
+  if (list == TL_F64 || (list == TL_QR && !o.df)) {
     const F64Shape sh = f64_shape(p);
     o.d.tf = sh.T;
     o.d.wkf = sh.wk;
@@ -211,6 +213,8 @@ void release(tt_ctx* c, DevGemmBuf& o) {
   dfree(c, o.buf);
   dfree(c, o.tcbuf);
   dfree(c, o.tilesf);
+  dfree(c, o.tileso);
+  o.nordered = o.tordered = 0;
   dfree(c, o.tiles64);
   dfree(c, o.tilesd);
   o.d = DevGemm();
@@ -693,6 +697,7 @@ struct Eng {
   // K extent of the persistent kernels' boxes: 32 where no segment is longer
   // than 64 (digits) or 128 (split-BF16), else 64
   int tc_box(const DevGemmBuf& g) const {
+    if (r->settling && !r->exact) return 64;
     for (const GSeg& sg : g.host.segs)
       if (sg.K > (r->exact ? 64 : 128)) return 64;
     return 32;
@@ -717,7 +722,8 @@ struct Eng {
     bool same = true;
     for (int i = 0; i < 8; ++i)
       if (used & (1u << i)) same = same && g.key_p[i] == b.p[i] && g.key_lo[i] == b.lo[i];
-    if (same && g.tcbuf.p) return true;
+    const int kbox = tc_box(g);
+    if (same && g.tcbuf.p && g.key_box == kbox) return true;
     // a captured step must replay the uploads of the uncaptured one
     if (r->capturing) throw Err{TT_ERR_STATE, "tensor-map operands moved during graph capture"};
     // looked up once per process (thread-safe static initialisation)
@@ -734,7 +740,6 @@ struct Eng {
       g.tc_ok = false;
       return false;
     }
-    const int kbox = tc_box(g);
     const size_t nseg = g.host.segs.size();
     std::vector<CUtensorMap> maps(4 * nseg);
     std::vector<int> seg_group(nseg, 0);
@@ -799,12 +804,31 @@ struct Eng {
     g.ntiles128 = (int)tiles.size();
     g.ntilesp = (int)tp.size();
     for (int i = 0; i < 8; ++i) { g.key_p[i] = b.p[i]; g.key_lo[i] = b.lo[i]; }
+    g.key_box = kbox;
     return true;
   }
 
   // FP64 launch of a plan; the tile lists are built and uploaded when first
   // needed (in the uncaptured step, as for the tensor maps)
   void f64(DevGemmBuf& g, const Bases& b) {
+    if (r->settling) {
+      if (g.tordered == 0) {
+        const F64Shape sh = f64_shape_ordered(g.host);
+        const std::vector<FTile> t = f64_tiles(g.host, sh.T);
+        Stager s;
+        s.add(t, &g.ordered);
+        s.commit(c, g.tileso);
+        g.nordered = (int)t.size();
+        g.tordered = sh.T;
+      }
+      DevGemm d = g.d;
+      d.tilesf = g.ordered;
+      d.ntilesf = g.nordered;
+      d.tf = g.tordered;
+      d.wkf = 1;
+      CK(launch_gemm_f64(d, b, st));
+      return;
+    }
     if (g.d.tf == 0) {
       if (r->capturing) throw Err{TT_ERR_STATE, "FP64 tile list missing during graph capture"};
       const F64Shape sh = f64_shape(g.host);
@@ -855,7 +879,7 @@ struct Eng {
     else if (k == TK_TCP128X64)
       CK(launch_gemm_tcp(g.d.groups, g.d.segs, g.tilesp, g.ntilesp, split_tiles(g), tc_box(g), g.maps, b, r->nsplit,
                          !g.host.groups.empty() && (g.host.groups[0].flags & 2), r->zscr.p, (unsigned*)r->ztick.p,
-                         (int*)r->tcerr.p, c->wait_ns, st));
+                         (int*)r->tcerr.p, c->wait_ns, st, r->settling));
     else
       CK(launch_gemm_bf16(with64(g), b, r->nsplit, st));
   }
@@ -868,7 +892,7 @@ struct Eng {
   // Every candidate overwrites the plan's whole output (no plan here
   // accumulates into C), and the chosen kernel runs last, so the output is
   // the chosen kernel's.  TT_GEMM=tc|tcp|mma forces one kernel.
-  int tune(DevGemmBuf& g, const Bases& b, bool tc) {
+  static int forced_kernel() {
     static const int forced = [] {
       const char* v = std::getenv("TT_GEMM");
       if (!v) return -1;
@@ -877,6 +901,10 @@ struct Eng {
       if (!std::strcmp(v, "mma")) return (int)TK_MMA64;
       return -1;
     }();
+    return forced;
+  }
+  int tune(DevGemmBuf& g, const Bases& b, bool tc) {
+    const int forced = forced_kernel();
     if (forced >= 0) return (forced == TK_MMA64 || tc) ? forced : (int)TK_MMA64;
     if (!tc) return TK_MMA64;
     if (r->capturing) return TK_TCP128X64;  // plans are tuned in the uncaptured step; this is a fallback
@@ -919,6 +947,7 @@ struct Eng {
   // CTAs that share a tile of a persistent tcgen05 kernel, with room for their
   // partial sums (allocated in the uncaptured step, like every buffer)
   int split_tiles(const DevGemmBuf& g) {
+    if (r->settling) return 1;
     int ms = 0;
     for (const GGroup& gg : g.host.groups) ms = std::max(ms, gg.seg1 - gg.seg0);
     const int split = tcz_split(g.ntilesp, ms);
@@ -951,7 +980,16 @@ struct Eng {
       const long e = prof_begin(kind, g.d.flops);
       const int split = split_tiles(g);
       CK(launch_gemm_tcz(g.d.groups, g.d.segs, g.tilesp, g.ntilesp, split, tc_box(g), g.maps, b, r->zscr.p,
-                         (unsigned*)r->ztick.p, (int*)r->tcerr.p, c->wait_ns, pair, st));
+                         (unsigned*)r->ztick.p, (int*)r->tcerr.p, c->wait_ns, pair, st, r->settling));
+      prof_end(e);
+      count();
+      return;
+    }
+    if (use_mixed && r->settling) {  // not a choice that timing makes
+      const bool tc = r->use_tc && prep_tc(g, b);
+      const int k = !tc ? (int)TK_MMA64 : (forced_kernel() >= 0 ? forced_kernel() : (int)TK_TCP128X64);
+      const long e = prof_begin(kind, g.d.flops);
+      launch_split(g, b, k);
       prof_end(e);
       count();
       return;
@@ -967,9 +1005,9 @@ struct Eng {
     if (use_mixed) {
       launch_split(g, b, g.choice);
     } else if (f64_kernel == 1) {
-      CK(launch_gemm_oz(with64(g), b, st));
+      CK(launch_gemm_oz(with64(g), b, st, r->settling));
     } else if (f64_kernel == 2) {
-      CK(launch_gemm_df(withdf(g), b, st));
+      CK(launch_gemm_df(withdf(g), b, st, r->settling));
     } else {
       f64(g, b);
     }
@@ -978,7 +1016,7 @@ struct Eng {
   }
   void gather_digits(const DevGatherBuf& g, const Bases& b) {
     const long e = prof_begin(3, 0);
-    CK(launch_gather_digits(g.d, b, st));
+    CK(r->settling ? launch_gather_digits_rows(g.d, b, st) : launch_gather_digits(g.d, b, st));
     prof_end(e);
     count();
   }
@@ -1025,7 +1063,7 @@ struct Eng {
     b.p[S_X] = v[k].p;
     b.p[S_Y] = vsp[k].p;
     b.lo[S_Y] = (&sz == &r->Lsize ? r->Lpsize : r->Rpsize)[k];
-    if (r->exact) CK(launch_digit_copy(r->edig[k].d, b, st));
+    if (r->exact) CK(launch_digit_copy(r->edig[k].d, b, st, r->settling));
     else CK(launch_split_copy(r->esplit[k].d, b, r->nsplit, st));
     count();
   }
@@ -1035,7 +1073,7 @@ struct Eng {
     b.p[S_X] = (void*)x;
     b.p[S_Y] = r->Xs.p;
     b.lo[S_Y] = s.h.xt_size;
-    if (r->exact) CK(launch_digit_copy(s.xd.d, b, st));
+    if (r->exact) CK(launch_digit_copy(s.xd.d, b, st, r->settling));
     else CK(launch_split_copy(s.xs.d, b, r->nsplit, st));
     count();
   }
@@ -1112,7 +1150,7 @@ struct Eng {
         Bases bx{};
         bx.p[S_X] = (void*)x;
         bx.p[S_Y] = r->Xs.p; bx.lo[S_Y] = bd.h.xt_size;
-        if (r->exact) CK(launch_digit_copy(bd.xd.d, bx, st));
+        if (r->exact) CK(launch_digit_copy(bd.xd.d, bx, st, r->settling));
         else CK(launch_split_copy(bd.xs.d, bx, r->nsplit, st));
         count();
       }
@@ -1124,7 +1162,7 @@ struct Eng {
         Bases bt{};
         bt.p[S_T1] = r->T1.p;
         bt.p[S_Y] = r->T2.p; bt.lo[S_Y] = bd.h.tp_size;
-        if (r->exact) CK(launch_digit_copy(bd.td.d, bt, st));
+        if (r->exact) CK(launch_digit_copy(bd.td.d, bt, st, r->settling));
         else CK(launch_split_copy(bd.ts.d, bt, r->nsplit, st));
         count();
       }
@@ -1214,6 +1252,16 @@ struct Eng {
     double* part = dptr(r->partial);
     KrylovState* ks = (KrylovState*)r->ks.p;
     const int64_t ldq = r->ldq;
+    if (r->settling) {
+      CK(k_settle_begin(x, n, part, ks, Q, st)); count(3);
+      for (int k = 0; k < K; ++k) {
+        apply(Q + (int64_t)k * ldq, w);
+        CK(k_settle_step(Q, ldq, k, K, w, n, part, ks, BREAKDOWN_TOL, st));
+        count(k + 1 < K ? 11 : 10);
+      }
+      CK(k_settle_end(Q, ldq, ks, t, K, x, n, part, (RhoScalars*)r->rs.p, st)); count(4);
+      return;
+    }
     CK(k_lanczos_begin(x, n, part, ks, Q, st)); count(2);
     for (int k = 0; k < K; ++k) {
       apply(Q + (int64_t)k * ldq, w);
@@ -1255,7 +1303,8 @@ struct Eng {
     // the mixed modes run the large Gram and apply GEMMs in double-float on the
     // FP32 pipe (their error budget is far above ~2^-46), the others in FP64
     auto qr_gemm = [&](DevGemmBuf& g) {
-      if (mixed() && g.d.ntilesd >= 0) CK(launch_gemm_df(g.d, b, st));
+      if (mixed() && r->settling) CK(launch_gemm_df(withdf(g), b, st, r->settling));
+      else if (mixed() && g.df) CK(launch_gemm_df(g.d, b, st));
       else f64(g, b);
     };
     for (int p = 0; p < 3; ++p) {
@@ -1265,7 +1314,8 @@ struct Eng {
       e = prof_begin(12, 0);
       // the mixed modes factorise in double-float (their error budget is far
       // above ~2^-46), FP64 mode in FP64
-      CK(launch_chol_inv(q.cjobs[p], q.ncj[p], dptr(r->ws), (int*)q.fail.p, st, q.maxn[p], mixed()));
+      auto chol = r->settling ? launch_chol_rows : launch_chol_inv;
+      CK(chol(q.cjobs[p], q.ncj[p], dptr(r->ws), (int*)q.fail.p, st, q.maxn[p], mixed()));
       prof_end(e);
       e = prof_begin(11, q.app[p].d.flops);
       qr_gemm(q.app[p]);
@@ -1379,7 +1429,7 @@ struct Eng {
   }
 
   // ---- initial state ---------------------------------------------------------
-  void init_state(double beta0) {
+  void init_state(double beta0, bool envs) {
     const Mpo& m = M();
     const int N = m.N;
     // bonds from the MPO channel charges; channel w -> (sector, index)
@@ -1424,8 +1474,10 @@ struct Eng {
     ensure_vec_capacity();
     KrylovState* ks = (KrylovState*)r->ks.p;
     CK(k_normalise_inplace(dptr(r->A[0]), r->lay[0].size, dptr(r->partial), ks, (RhoScalars*)r->rs.p, st));
-    build_boundary_envs();
-    for (int j = N - 1; j >= 1; --j) update_right_env(j);
+    if (envs) {
+      build_boundary_envs();
+      for (int j = N - 1; j >= 1; --j) update_right_env(j);
+    }
     CK(cudaStreamSynchronize(st));
   }
 
@@ -1531,13 +1583,20 @@ struct Eng {
   // rho_0 = sum_{n <= order} (-beta0 H / 2)^n / n! by Horner's rule:
   // P_{order-1} = I - (beta0 / (2 order)) H (the compact first-order state),
   // P_k = I - (beta0 / (2 (k + 1))) H P_{k+1}, rho_0 = P_0.
-  void init_series(double beta0, int order) {
-    init_state(beta0 / order);
+  void init_series(double beta0, int order, bool envs) {
+    init_state(beta0 / order, envs);
     for (int k = order - 2; k >= 0; --k) horner_step(-beta0 / (2.0 * (k + 1)));
     r->beta = beta0;
-    build_boundary_envs();
-    for (int j = r->N - 1; j >= 1; --j) update_right_env(j);
+    if (envs) {
+      build_boundary_envs();
+      for (int j = r->N - 1; j >= 1; --j) update_right_env(j);
+    }
     CK(cudaStreamSynchronize(st));
+  }
+
+  void create(bool envs) {
+    if (r->order == 1) init_state(r->beta0, envs);
+    else init_series(r->beta0, r->order, envs);
   }
 
   void build_boundary_envs() {
@@ -1791,6 +1850,18 @@ struct Eng {
   // zero columns: the state is unchanged, the manifold is larger.
   void pad_bonds(int D_target) {
     const int N = r->N;
+    if (r->fresh) {
+      // the state is still what tt_rho_create made: made again in the arithmetic in
+      // which its null directions will settle
+      bool below = false;
+      for (int k = 1; k < N; ++k) below = below || r->bond[k].total() < D_target;
+      if (below) {
+        r->settling = true;
+        for (int k = 0; k <= N; ++k) invalidate_bond(k);
+        CK(cudaMemsetAsync(r->rs.p, 0, sizeof(RhoScalars), st));
+        create(false);  // (the environments are updated below, the boundary ones stay)
+      }
+    }
     const LocalSpace& ls = M().ls;
     // targets
     std::vector<Bond> tgt = r->bond;
@@ -1899,7 +1970,10 @@ struct Eng {
       r->lay[k] = newk;
       r->lay[k - 1] = newp;
       invalidate_bond(k);
+      r->settling = r->padded = true;
+      r->fresh = false;
     }
+    if (!r->padded) r->settling = false;
     ensure_vec_capacity();
     for (int j = N - 1; j >= 1; --j) update_right_env(j);
     CK(cudaStreamSynchronize(st));
@@ -2671,11 +2745,12 @@ tt_status tt_rho_create(tt_ctx* ctx, const tt_mpo* mpo, double beta0, int taylor
   r->opts = *opts;
   r->N = mpo->mpo.N;
   r->nsplit = opts->growth_precision == 1 ? 2 : (opts->growth_precision == 2 ? 3 : 0);
+  r->beta0 = beta0;
+  r->order = taylor_order;
   tt_status s = guarded(ctx, r, [&] {
     alloc_rho_arrays(r);
-    Eng e(r);
-    if (taylor_order == 1) e.init_state(beta0);
-    else e.init_series(beta0, taylor_order);
+    Eng(r).create(true);
+    r->fresh = true;
   });
   if (s != TT_OK) {
     free_rho(r);
@@ -2704,6 +2779,7 @@ tt_status tt_rho_grow(tt_rho* rho, const tt_mpo* mpo, double dtau, double beta_m
   if (!rho || mpo != rho->mpo || !(dtau > 0)) return TT_ERR_INVALID_ARG;
   return guarded(rho->ctx, rho, [&] {
     Eng e(rho);
+    rho->settling = rho->padded = rho->fresh = false;  // (two-site steps carry no bond along)
     e.set_precision(growth_arith(rho->opts.growth_precision));
     while (rho->beta < beta_max - 1e-12 && !e.saturated()) {
       e.grow_sweep_lr(dtau / 4);
@@ -2720,6 +2796,7 @@ tt_status tt_rho_grow_exp(tt_rho* rho, const tt_mpo* mpo, double ratio, double b
     return TT_ERR_INVALID_ARG;
   return guarded(rho->ctx, rho, [&] {
     Eng e(rho);
+    rho->settling = rho->padded = rho->fresh = false;  // (two-site steps carry no bond along)
     e.set_precision(growth_arith(rho->opts.growth_precision));
     while (rho->beta < beta_max - 1e-12 && !e.saturated()) {
       const double dtau = std::min(rho->beta * (ratio - 1.0), beta_max - rho->beta);
@@ -2736,6 +2813,7 @@ tt_status tt_tdvp_step(tt_rho* rho, const tt_mpo* mpo, double dtau, int n_steps)
   if (!rho || mpo != rho->mpo || !(dtau > 0) || n_steps < 0) return TT_ERR_INVALID_ARG;
   return guarded(rho->ctx, rho, [&] {
     Eng e(rho);
+    if (n_steps > 0) rho->fresh = false;
     e.set_precision(rho->opts.precision);
     e.prepare_all();
     if (!rho->ev0) CK(cudaEventCreate(&rho->ev0));
@@ -2747,7 +2825,17 @@ tt_status tt_tdvp_step(tt_rho* rho, const tt_mpo* mpo, double dtau, int n_steps)
                        rho->graph_buf_gen != rho->ctx->buf_gen || rho->graph_wait_ns != rho->ctx->wait_ns))
       e.drop_graph();
     int s = 0;
-    if (!rho->graph && rho->use_graph && n_steps > 0 && st != nullptr && !rho->stats_pending) {
+    // a padded state's first step, in the arithmetic of tt_settle.cu; not captured
+    if (n_steps > 0 && rho->padded) {
+      e.sweep_lr(dtau / 4);
+      e.sweep_rl(dtau / 4);
+      rho->beta += dtau;
+      ++s;
+      rho->settling = rho->padded = false;
+      rho->capture_due = true;
+    }
+    if (!rho->graph && rho->use_graph && n_steps > s && st != nullptr && (!rho->stats_pending || rho->capture_due)) {
+      rho->capture_due = false;
       // one uncaptured step builds every plan, tensor map and buffer, then one
       // step is captured (no allocation or host synchronisation happens in it)
       e.sweep_lr(dtau / 4);
@@ -3079,6 +3167,22 @@ tt_status tt_layout_sizes_terms(int nw_l, const int* chl_qn, const int* chl_qs, 
   return tt_layout_sizes(&m, 0, nsec_lr, qn, qs, qd, x_size, l_size, r_size);
 }
 
+// whether a column (right bond state) of the site tensor is zero throughout: what
+// padding leaves, and nothing else as a rule
+static bool has_zero_column(const SiteLayout& S, const Bond& B, const std::vector<double>& a) {
+  for (int q = 0; q < B.nsec(); ++q) {
+    const int64_t rows = S.grp_rows[q], n = B.dim[q];
+    if (rows == 0) continue;
+    const double* g = a.data() + S.grp_off[q];
+    for (int64_t c = 0; c < n; ++c) {
+      int64_t i = 0;
+      while (i < rows && g[i * n + c] == 0.0) ++i;
+      if (i == rows) return true;
+    }
+  }
+  return false;
+}
+
 static const char kMagic[8] = {'T', 'T', 'R', 'H', 'O', '0', '0', '1'};
 
 tt_status tt_rho_save(tt_rho* rho, const char* path) {
@@ -3159,6 +3263,7 @@ tt_status tt_rho_load(tt_ctx* ctx, const tt_mpo* mpo, const char* path, const tt
     }
     r->lay.assign(N, SiteLayout());
     Eng e(r);
+    bool zero_column = false;  // a padded state that has not made a step yet
     for (int j = 0; j < N; ++j) {
       e.relayout(j);
       int64_t n;
@@ -3167,10 +3272,12 @@ tt_status tt_rho_load(tt_ctx* ctx, const tt_mpo* mpo, const char* path, const tt
       std::vector<double> h(n);
       f.read((char*)h.data(), n * 8);
       if (!f) throw Err{TT_ERR_INVALID_ARG, "truncated checkpoint"};
+      zero_column = zero_column || has_zero_column(r->lay[j], r->bond[j + 1], h);
       e.ensure_site_buf(j);
       CK(cudaMemcpyAsync(r->A[j].p, h.data(), n * 8, cudaMemcpyHostToDevice, ctx->st));
       CK(cudaStreamSynchronize(ctx->st));
     }
+    r->settling = r->padded = zero_column;
     RhoScalars rs{logscale, resid, 0, 0};
     CK(cudaMemcpyAsync(r->rs.p, &rs, sizeof(rs), cudaMemcpyHostToDevice, ctx->st));
     e.ensure_vec_capacity();

@@ -60,6 +60,11 @@ struct DevGemmBuf {
   GTile *tiles128 = nullptr, *tilesp = nullptr;
   DBuf tilesf, tiles64, tilesd;  // tile lists of the FP64, 64 x 64 and double-float kernels, where not uploaded with the plan
   int ntiles128 = 0, ntilesp = 0;  // 128 x 128 tiles (tc), 128 x 64 tiles (persistent tc)
+  DBuf tileso;  // FP64 kernel's one-warp tiles (a padded state's first step)
+  FTile* ordered = nullptr;
+  int nordered = 0, tordered = 0;
+  bool df = false;  // gauge product of a mixed mode that runs in double-float
+  int key_box = 0;  // K extent of the boxes that the maps were made for
   // autotuned kernel of a split-BF16 plan: -1 not chosen yet, else a TcKernel
   int choice = -1;
   void* key_p[8] = {nullptr};
@@ -157,6 +162,14 @@ struct tt_rho {
   std::vector<tt::DevCopyBuf> esplit;     // per bond: FP64 environment -> padded split copy
   std::vector<tt::DevDigitBuf> edig;      // per bond: FP64 environment -> digits (exact mode)
   std::vector<char> esplit_ok;
+  // padding, the first beta-step after it, and the creation of a state that is
+  // padded as it was created run in a fixed arithmetic (tt_settle.cu): settling
+  // until that step, or growth, is done; padded: the state has directions without
+  // weight; fresh: nothing but tt_rho_create(beta0, order) has touched the state
+  bool settling = false, padded = false, fresh = false;
+  double beta0 = 0.0;
+  int order = 0;
+  bool capture_due = false;               // that step is done, the next one may be captured
   bool apply_only = false;                // a single H_eff apply: no sweep buffers or plans
   bool use_tc = true;                     // tcgen05 kernel for eligible split-bf16 GEMMs
   bool use_cholqr = true;                 // CholeskyQR3 gauge (else Householder only)

@@ -211,6 +211,12 @@ F64Shape f64_shape(const GemmPlan& p) {
   return {8, 4};
 }
 
+F64Shape f64_shape_ordered(const GemmPlan& p) {
+  size_t tiles = 0;
+  for (const GGroup& g : p.groups) tiles += (size_t)((g.M + 15) / 16) * ((g.N + 15) / 16);
+  return {tiles >= 4 * 152 ? 16 : 8, 1};
+}
+
 std::vector<FTile> f64_tiles(const GemmPlan& p, int T) {
   std::vector<std::pair<int, int>> order;  // longest K first
   for (size_t g = 0; g < p.groups.size(); ++g) {

@@ -35,7 +35,7 @@ __device__ __forceinline__ int slot_of(Ref r) { return (int)(r >> 56); }
 __device__ __forceinline__ long long off_of(Ref r) { return (long long)(r & 0x00FFFFFFFFFFFFFFull); }
 
 __global__ void __launch_bounds__(DTH) gemm_df_kernel(const FTile* __restrict__ tiles, const GSeg* __restrict__ segs,
-                                                      Bases bs) {
+                                                      Bases bs, bool exact_out) {
   __shared__ float2 As[2][DK][DM + 1];
   __shared__ float2 Bs[2][DK][DN + 1];
   const FTile tl = tiles[blockIdx.x];
@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(DTH) gemm_df_kernel(const FTile* __restrict__ 
       const int r = ty + 16 * i, q = tx + 8 * j;
       if (r >= tl.rows || q >= tl.cols) continue;
       double* c = C + (long long)r * tl.ldc + q;
-      const double v = dbl_of_pair(hi[i][j], lo[i][j]);
+      const double v = exact_out ? (double)hi[i][j] + (double)lo[i][j] : dbl_of_pair(hi[i][j], lo[i][j]);
       *c = accum ? *c + v : v;
     }
 }
@@ -153,9 +153,9 @@ bool df_beats_f64(const GemmPlan& p) {
   return 1.5 * (td > 150 * chain ? td : 150 * chain) + 20000 < 1.3 * f64 / 152 + 5000;
 }
 
-cudaError_t launch_gemm_df(const DevGemm& g, const Bases& b, cudaStream_t s) {
+cudaError_t launch_gemm_df(const DevGemm& g, const Bases& b, cudaStream_t s, bool exact_out) {
   if (g.ntilesd == 0) return cudaSuccess;
-  gemm_df_kernel<<<g.ntilesd, DTH, 0, s>>>(g.tilesd, g.segs, b);
+  gemm_df_kernel<<<g.ntilesd, DTH, 0, s>>>(g.tilesd, g.segs, b, exact_out);
   return cudaGetLastError();
 }
 

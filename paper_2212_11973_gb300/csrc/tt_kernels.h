@@ -99,6 +99,8 @@ struct F64Shape {
   int T, wk;
 };
 F64Shape f64_shape(const GemmPlan& p);
+// one-warp tiles: every output a single sum over ascending K, whatever T
+F64Shape f64_shape_ordered(const GemmPlan& p);
 std::vector<FTile> f64_tiles(const GemmPlan& p, int T);
 cudaError_t launch_gemm_f64(const DevGemm& g, const Bases& b, cudaStream_t s);
 // The same in double-float arithmetic on the FP32 pipe (~2^-46 per operation),
@@ -106,10 +108,12 @@ cudaError_t launch_gemm_f64(const DevGemm& g, const Bases& b, cudaStream_t s);
 int df_tile_size();
 // whether the double-float kernel is the faster one for a plan
 bool df_beats_f64(const GemmPlan& p);
-cudaError_t launch_gemm_df(const DevGemm& g, const Bases& b, cudaStream_t s);
+// exact_out: hi + lo rounded as by an FP64 addition.
+cudaError_t launch_gemm_df(const DevGemm& g, const Bases& b, cudaStream_t s, bool exact_out = false);
 // Exact-accumulation split GEMM (tt_ozaki.cu): FP64 operands of the FP64
-// plans, four fixed-point BF16 digits per K tile, ~2^-32 normwise.
-cudaError_t launch_gemm_oz(const DevGemm& g, const Bases& b, cudaStream_t s);
+// plans, four fixed-point BF16 digits per K tile, ~2^-32 normwise.  topdown: digits
+// rounded from the top level down (tt_fixed.h).
+cudaError_t launch_gemm_oz(const DevGemm& g, const Bases& b, cudaStream_t s, bool topdown = false);
 // nsplit = 2 (3 products) or 3 (6 products); operand level l at offset l * lo[slot]
 cudaError_t launch_gemm_bf16(const DevGemm& g, const Bases& b, int nsplit, cudaStream_t s);
 // in_type / out_type: 0 = double, 1 = float, 2 / 3 = split bf16 with that many levels
@@ -127,10 +131,11 @@ size_t tc_smem_bytes(int nsplit);
 // CTA per SM, TMA ring / MMA warp / fold-and-epilogue warps, the same
 // arithmetic and maps.
 // out32: every group writes FP32 (flags bit 1), else FP64; split, kbox, scratch
-// and tickets as for launch_gemm_tcz below.
+// and tickets as for launch_gemm_tcz below; bylevel: the products of 64 of K level
+// by level into two sums (kbox 64, split 1).
 cudaError_t launch_gemm_tcp(const GGroup* groups, const GSeg* segs, const GTile* tiles128x64, int ntiles, int split,
                             int kbox, const void* maps, const Bases& b, int nsplit, bool out32, void* scratch,
-                            unsigned* tickets, int* err, long long wait_ns, cudaStream_t s);
+                            unsigned* tickets, int* err, long long wait_ns, cudaStream_t s, bool bylevel = false);
 // Exact-accumulation split GEMM on tcgen05 (tt_tcgen05z.cu): digit operands
 // (4 levels + int16 row exponents, GSeg.eA / eB), persistent 128 x 64 tiles,
 // maps with boxes of kbox = 64 (128-byte swizzle) or 32 (64-byte) K;
@@ -146,12 +151,12 @@ size_t tcz_scratch_bytes(int ntiles, int split);
 size_t tcz_tickets(int ntiles);
 cudaError_t launch_gemm_tcz(const GGroup* groups, const GSeg* segs, const GTile* tiles128x64, int ntiles, int split,
                             int kbox, const void* maps, const Bases& b, void* scratch, unsigned* tickets, int* err,
-                            long long wait_ns, bool pair, cudaStream_t s);
+                            long long wait_ns, bool pair, cudaStream_t s, bool exact_out = false);
 // Digit producers (tt_digits.cu): FP64 rows -> digit rows; the W-gather of
 // the exact path (two-float S1 outputs -> digit rows of T2, rows up to
 // gather_digits_max_cols() long, at most gather_digits_max_contribs() MPO
 // terms per item).
-cudaError_t launch_digit_copy(const DevDigit& d, const Bases& b, cudaStream_t s);
+cudaError_t launch_digit_copy(const DevDigit& d, const Bases& b, cudaStream_t s, bool topdown = false);
 cudaError_t launch_gather_digits(const DevGather& g, const Bases& b, cudaStream_t s);
 int gather_digits_max_cols();
 int gather_digits_max_contribs();
@@ -172,6 +177,16 @@ cudaError_t k_lanczos_step(double* Q, int64_t ldq, int k, int K, double* w, int6
                            RhoScalars* rs, double breakdown_tol, double t, cudaStream_t s);
 // y = sum_j ks->c[j] q_j
 cudaError_t k_lanczos_end(const double* Q, int64_t ldq, const KrylovState* ks, double* y, int64_t n, cudaStream_t s);
+
+// The same exponential, the digit gather and the Cholesky factors in the fixed
+// arithmetic of a padded state's first beta-step (tt_settle.cu).
+cudaError_t k_settle_begin(const double* x, int64_t n, double* partial, KrylovState* ks, double* q0, cudaStream_t s);
+cudaError_t k_settle_step(double* Q, int64_t ldq, int k, int K, double* w, int64_t n, double* partial, KrylovState* ks,
+                          double breakdown_tol, cudaStream_t s);
+cudaError_t k_settle_end(const double* Q, int64_t ldq, KrylovState* ks, double t, int K, double* y, int64_t n,
+                         double* partial, RhoScalars* rs, cudaStream_t s);
+cudaError_t launch_gather_digits_rows(const DevGather& g, const Bases& b, cudaStream_t s);
+cudaError_t launch_chol_rows(const CholJob* jobs, int njobs, double* ws, int* fail, cudaStream_t s, int maxn, bool df);
 
 // v /= ||v||, logscale += ln ||v|| (rs->bad set on zero / non-finite norm)
 cudaError_t k_normalise_inplace(double* v, int64_t n, double* partial, KrylovState* ks, RhoScalars* rs, cudaStream_t s);

@@ -117,12 +117,13 @@ __device__ __forceinline__ void row_exponents(const double* v, int tid, int* e) 
 }
 
 // The thread's digits into a tile of ODIG x 64 x (OBK + OPAD)
+template <bool TOPDOWN>
 __device__ __forceinline__ void store_digits(const double* v, int emax, int tid, __nv_bfloat16* tile) {
 #pragma unroll
   for (int i = 0; i < OEL; i += 2) {
     uint32_t d0[ODIG], d1[ODIG];
-    fixed_digit_bits(v[i], emax, d0);
-    fixed_digit_bits(v[i + 1], emax, d1);
+    fixed_digit_bits<TOPDOWN>(v[i], emax, d0);
+    fixed_digit_bits<TOPDOWN>(v[i + 1], emax, d1);
     __nv_bfloat16* at = tile + part_row(tid) * (OBK + OPAD) + pair_k(tid, i >> 1);
 #pragma unroll
     for (int s = 0; s < ODIG; ++s)
@@ -137,6 +138,7 @@ struct OzShared {
   int eA[2][OBM], eB[2][OBN];
 };
 
+template <bool TOPDOWN>
 __global__ void __launch_bounds__(OT) gemm_oz_kernel(const GGroup* __restrict__ groups, const GSeg* __restrict__ segs,
                                                       const GTile* __restrict__ tiles, Bases bs) {
   extern __shared__ __align__(16) unsigned char oz_smem[];
@@ -203,8 +205,8 @@ __global__ void __launch_bounds__(OT) gemm_oz_kernel(const GGroup* __restrict__ 
     __syncthreads();  // exponents complete; every warp done with the last tile's digits
     if (tid < OBM) sh.eA[cur ^ 1][tid] = 0;
     else if (tid < OBM + OBN) sh.eB[cur ^ 1][tid - OBM] = 0;
-    if (rows_a) store_digits(va, sh.eA[cur][part_row(tid)], tid, &sh.As[0][0][0]);
-    if (rows_b) store_digits(vb, sh.eB[cur][part_row(tid)], tid, &sh.Bs[0][0][0]);
+    if (rows_a) store_digits<TOPDOWN>(va, sh.eA[cur][part_row(tid)], tid, &sh.As[0][0][0]);
+    if (rows_b) store_digits<TOPDOWN>(vb, sh.eB[cur][part_row(tid)], tid, &sh.Bs[0][0][0]);
     fetch(stage);  // the values are in registers
     __syncthreads();
     if (!live) continue;
@@ -272,13 +274,16 @@ __global__ void __launch_bounds__(OT) gemm_oz_kernel(const GGroup* __restrict__ 
 
 }  // namespace
 
-cudaError_t launch_gemm_oz(const DevGemm& g, const Bases& b, cudaStream_t s) {
+cudaError_t launch_gemm_oz(const DevGemm& g, const Bases& b, cudaStream_t s, bool topdown) {
   if (g.ntiles64 == 0) return cudaSuccess;
   // 107 KB of shared memory; set on every call, as the attribute is per device
-  cudaError_t e = cudaFuncSetAttribute(gemm_oz_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(OzShared));
-  if (e != cudaSuccess) return e;
-  gemm_oz_kernel<<<g.ntiles64, OT, sizeof(OzShared), s>>>(g.groups, g.segs, g.tiles64, b);
-  return cudaGetLastError();
+  auto run = [&](auto kernel) {
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(OzShared));
+    if (e != cudaSuccess) return e;
+    kernel<<<g.ntiles64, OT, sizeof(OzShared), s>>>(g.groups, g.segs, g.tiles64, b);
+    return cudaGetLastError();
+  };
+  return topdown ? run(gemm_oz_kernel<true>) : run(gemm_oz_kernel<false>);
 }
 
 }  // namespace tt

@@ -64,8 +64,11 @@ __device__ __forceinline__ int part_pieces(const TileItem& q, const GSeg* segs) 
   return __reduce_add_sync(0xffffffffu, t);
 }
 
-// OUT32: every group of the launch writes FP32 (flags bit 1), else FP64
-template <int NS, int BK, bool OUT32>
+// OUT32: every group of the launch writes FP32 (flags bit 1), else FP64.
+// BYLEVEL (BK = 64): the order of a padded state's first beta-step (tt_settle.cu):
+// the level products of a piece one after the other, those of order 0 into one
+// accumulator and all others into a second, both folded by one formula.
+template <int NS, int BK, bool OUT32, bool BYLEVEL>
 __global__ void __launch_bounds__(PTHREADS, 1) gemm_tcp_kernel(const GGroup* __restrict__ groups,
                                                                const GSeg* __restrict__ segs,
                                                                const GTile* __restrict__ tiles, int nitems, int split,
@@ -76,7 +79,7 @@ __global__ void __launch_bounds__(PTHREADS, 1) gemm_tcp_kernel(const GGroup* __r
   using C = PCfg<NS, BK>;
   constexpr int S = C::STAGES;
   constexpr int BUF = 64 * NS;                       // TMEM columns of one accumulator buffer
-  static_assert(S >= 2 && 2 * BUF <= (int)PTMEM_COLS, "stages and accumulators");
+  static_assert(S >= 2 && 2 * BUF <= (int)PTMEM_COLS && (!BYLEVEL || BK == PIECE), "stages and accumulators");
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[S], empty_bar[S], accf[2], acce[2];
   __shared__ uint32_t tmem_base_s;
@@ -194,13 +197,26 @@ __global__ void __launch_bounds__(PTHREADS, 1) gemm_tcp_kernel(const GGroup* __r
             fence_after();
             const uint32_t tb = tmem + BUF * b;
             const uint32_t sa = smem_u32(smem + sg * C::STAGE_BYTES);
-            const int nk = (min(BK, K - k0) + 15) >> 4;  // 16-wide steps with data
-            for (int kk = 0; kk < nk; ++kk) {
-              const uint64_t bd = desc_of<BK>(sa + NS * C::A_BYTES + kk * 32);
+            const uint32_t sb = sa + NS * C::A_BYTES;
+            if (BYLEVEL) {
 #pragma unroll
-              for (int l = 0; l < NS; ++l)
-                umma_f16(tb + 64 * l, desc_of<BK>(sa + l * C::A_BYTES + kk * 32), bd,
-                         idesc0 | ((uint32_t)((PBN * (NS - l)) >> 3) << 17), (!first || kk > 0 || l > 0) ? 1u : 0u);
+              for (int p = 0; p < NS * (NS + 1) / 2; ++p) {
+                const int la = (p == 2 || p == 4) ? 1 : (p == 5 ? 2 : 0), lb = (p == 1 || p == 4) ? 1 : (p == 3 ? 2 : 0);
+#pragma unroll
+                for (int kk = 0; kk < BK / 16; ++kk)
+                  umma_f16(tb + (p ? 64 : 0), desc_of<BK>(sa + la * C::A_BYTES + kk * 32),
+                           desc_of<BK>(sb + lb * C::B_BYTES + kk * 32), idesc0 | ((uint32_t)(PBN >> 3) << 17),
+                           (!first || p > 1 || kk > 0) ? 1u : 0u);
+              }
+            } else {
+              const int nk = (min(BK, K - k0) + 15) >> 4;  // 16-wide steps with data
+              for (int kk = 0; kk < nk; ++kk) {
+                const uint64_t bd = desc_of<BK>(sb + kk * 32);
+#pragma unroll
+                for (int l = 0; l < NS; ++l)
+                  umma_f16(tb + 64 * l, desc_of<BK>(sa + l * C::A_BYTES + kk * 32), bd,
+                           idesc0 | ((uint32_t)((PBN * (NS - l)) >> 3) << 17), (!first || kk > 0 || l > 0) ? 1u : 0u);
+              }
             }
             umma_commit(&empty_bar[sg]);
             last_commit_s = it;
@@ -240,19 +256,33 @@ __global__ void __launch_bounds__(PTHREADS, 1) gemm_tcp_kernel(const GGroup* __r
         const uint32_t tb = tmem + BUF * b + lane_off + 32 * h;
 #pragma unroll
         for (int cb = 0; cb < 32; cb += 16) {
-          uint32_t dv[NS][16];
+          constexpr int ND = BYLEVEL ? 2 : NS;  // accumulators
+          uint32_t dv[ND][16];
 #pragma unroll
-          for (int d = 0; d < NS; ++d) tmem_ld16_nw(tb + 64 * d + cb, dv[d]);
+          for (int d = 0; d < ND; ++d) tmem_ld16_nw(tb + 64 * d + cb, dv[d]);
           tmem_wait_ld16(dv[0]);
 #pragma unroll
-          for (int d = 1; d < NS; ++d) tmem_dep16(dv[d]);
+          for (int d = 1; d < ND; ++d) tmem_dep16(dv[d]);
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
-            float u = __uint_as_float(dv[NS - 1][i]);
+            float u = __uint_as_float(dv[ND - 1][i]);
 #pragma unroll
-            for (int d = NS - 2; d >= 1; --d) u += __uint_as_float(dv[d][i]);
-            two_sum_into(hi[cb + i], lo[cb + i], __uint_as_float(dv[0][i]));
-            lo[cb + i] += u;
+            for (int d = ND - 2; d >= 1; --d) u += __uint_as_float(dv[d][i]);
+            if (BYLEVEL) {
+              const float x = __uint_as_float(dv[0][i]), h0 = hi[cb + i];
+              if (f == 0) {
+                hi[cb + i] = x;
+                lo[cb + i] = u;
+              } else {
+                const float sv = h0 + x;
+                const float bp = sv - h0;
+                lo[cb + i] += ((h0 - (sv - bp)) + (x - bp)) + u;
+                hi[cb + i] = sv;
+              }
+            } else {
+              two_sum_into(hi[cb + i], lo[cb + i], __uint_as_float(dv[0][i]));
+              lo[cb + i] += u;
+            }
           }
         }
         fence_before();
@@ -269,7 +299,7 @@ __global__ void __launch_bounds__(PTHREADS, 1) gemm_tcp_kernel(const GGroup* __r
                         reinterpret_cast<float*>(z.C), z.ldc, z.m0 + 32 * q, z.n0 + 32 * h + cb, z.M, z.N, z.flags & 1);
         } else {
           double v[16];
-          dbl_of_pairs<16>(hi + cb, lo + cb, v);
+          dbl_of_pairs<16>(hi + cb, lo + cb, v, BYLEVEL);
           store_block16(stg, [&](int k) { return (uint64_t)__double_as_longlong(v[k]); },
                         reinterpret_cast<double*>(z.C), z.ldc, z.m0 + 32 * q, z.n0 + 32 * h + cb, z.M, z.N, z.flags & 1);
         }
@@ -311,8 +341,9 @@ int sm_count() {
 
 cudaError_t launch_gemm_tcp(const GGroup* groups, const GSeg* segs, const GTile* tiles, int ntiles, int split,
                             int kbox, const void* maps, const Bases& b, int nsplit, bool out32, void* scratch,
-                            unsigned* tickets, int* err, long long wait_ns, cudaStream_t s) {
+                            unsigned* tickets, int* err, long long wait_ns, cudaStream_t s, bool bylevel) {
   if (ntiles == 0) return cudaSuccess;
+  if (bylevel && (kbox != 64 || split != 1)) return cudaErrorInvalidValue;
   if ((kbox != 32 && kbox != 64) || split < 1 || (split > 1 && (!scratch || !tickets))) return cudaErrorInvalidValue;
   const int nitems = ntiles * split, grid = nitems < sm_count() ? nitems : sm_count();
   auto run = [&](auto kernel) {
@@ -324,8 +355,9 @@ cudaError_t launch_gemm_tcp(const GGroup* groups, const GSeg* segs, const GTile*
   };
   auto pick = [&](auto ns) {
     constexpr int NS = decltype(ns)::value;
-    if (kbox == 64) return out32 ? run(gemm_tcp_kernel<NS, 64, true>) : run(gemm_tcp_kernel<NS, 64, false>);
-    return out32 ? run(gemm_tcp_kernel<NS, 32, true>) : run(gemm_tcp_kernel<NS, 32, false>);
+    if (bylevel) return out32 ? run(gemm_tcp_kernel<NS, 64, true, true>) : run(gemm_tcp_kernel<NS, 64, false, true>);
+    if (kbox == 64) return out32 ? run(gemm_tcp_kernel<NS, 64, true, false>) : run(gemm_tcp_kernel<NS, 64, false, false>);
+    return out32 ? run(gemm_tcp_kernel<NS, 32, true, false>) : run(gemm_tcp_kernel<NS, 32, false, false>);
   };
   if (nsplit == 2) return pick(std::integral_constant<int, 2>{});
   if (nsplit == 3) return pick(std::integral_constant<int, 3>{});

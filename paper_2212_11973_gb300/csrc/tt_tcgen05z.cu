@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(ZTHREADS, 1) gemm_tcz_kernel(const GGroup* __r
                                                                const CUtensorMap* __restrict__ maps, Bases bs,
                                                                uint64_t* __restrict__ scratch,
                                                                unsigned* __restrict__ tickets, int* __restrict__ err,
-                                                               long long wait_ns) {
+                                                               long long wait_ns, bool exact_out) {
   constexpr int ZA_BYTES = ZBM * ZBK * 2, ZB_BYTES = ZBN * ZBK * 2;  // per digit level
   constexpr int ZSTAGE_BYTES = ZDIG * (ZA_BYTES + ZB_BYTES);
   constexpr int ZSTAGES = ZRING_BYTES / ZSTAGE_BYTES;
@@ -304,7 +304,9 @@ __global__ void __launch_bounds__(ZTHREADS, 1) gemm_tcz_kernel(const GGroup* __r
             const int xe = xa + __shfl_sync(0xffffffffu, eb, cb + i);
             const float sc = __int_as_float(min(max(xe, 0), 254) << 23);
             // D_0 + D_1 2^-8 as an exact pair (sv, ev) (TwoSum), D_2 2^-16 and
-            // D_3 2^-24 into ev, then the pair scaled by the power of two sc
+            // D_3 2^-24 into ev, then the pair scaled by the power of two sc (a
+            // product of its own: fused into the sums below, the same but where it
+            // is subnormal, it would round once less)
             const float d0 = __uint_as_float(dv[0][i]);
             const float p1 = __uint_as_float(dv[1][i]) * 0.00390625f;
             const float sv = d0 + p1;
@@ -312,7 +314,7 @@ __global__ void __launch_bounds__(ZTHREADS, 1) gemm_tcz_kernel(const GGroup* __r
             float ev = (d0 - (sv - bp)) + (p1 - bp);
             ev = fmaf(__uint_as_float(dv[2][i]), 1.52587890625e-05f, ev);
             ev = fmaf(__uint_as_float(dv[3][i]), 5.9604644775390625e-08f, ev);
-            const float s2 = sv * sc, e2 = ev * sc;
+            const float s2 = __fmul_rn(sv, sc), e2 = __fmul_rn(ev, sc);
             if (first) {
               hi[cb + i] = s2;
               lo[cb + i] = e2;
@@ -343,7 +345,7 @@ __global__ void __launch_bounds__(ZTHREADS, 1) gemm_tcz_kernel(const GGroup* __r
               reinterpret_cast<uint64_t*>(z.C), z.ldc, z.m0 + 32 * q, z.n0 + 32 * h + cb, z.M, z.N, false);
         } else {
           double v[16];
-          dbl_of_pairs<16>(hi + cb, lo + cb, v);
+          dbl_of_pairs<16>(hi + cb, lo + cb, v, exact_out);
           store_block16(stg, [&](int k) { return (uint64_t)__double_as_longlong(v[k]); },
                         reinterpret_cast<double*>(z.C), z.ldc, z.m0 + 32 * q, z.n0 + 32 * h + cb, z.M, z.N, z.flags & 1);
         }
@@ -395,7 +397,7 @@ size_t tcz_tickets(int ntiles) { return (size_t)ntiles * ZEPI; }
 
 cudaError_t launch_gemm_tcz(const GGroup* groups, const GSeg* segs, const GTile* tiles, int ntiles, int split,
                             int kbox, const void* maps, const Bases& b, void* scratch, unsigned* tickets, int* err,
-                            long long wait_ns, bool pair, cudaStream_t s) {
+                            long long wait_ns, bool pair, cudaStream_t s, bool exact_out) {
   if (ntiles == 0) return cudaSuccess;
   if ((kbox != 32 && kbox != 64) || split < 1 || (split > 1 && (!scratch || !tickets))) return cudaErrorInvalidValue;
   const size_t smem = tcz_smem_bytes();
@@ -404,7 +406,7 @@ cudaError_t launch_gemm_tcz(const GGroup* groups, const GSeg* segs, const GTile*
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     kernel<<<grid, ZTHREADS, smem, s>>>(groups, segs, tiles, nitems, split, (const CUtensorMap*)maps, b,
-                                        (uint64_t*)scratch, tickets, err, wait_ns);
+                                        (uint64_t*)scratch, tickets, err, wait_ns, exact_out);
     return cudaGetLastError();
   };
   if (pair) return kbox == 64 ? run(gemm_tcz_kernel<true, 64>) : run(gemm_tcz_kernel<true, 32>);
