@@ -141,9 +141,11 @@ __global__ void __launch_bounds__(ZTHREADS, 1) gemm_tcz_kernel(const GGroup* __r
   if (warp == 0) {
     // ---------------- producer ----------------
     int it = 0;
-    for (int i = 0; blockIdx.x + i * gridDim.x < nitems && !*abort_f; ++i) {
+    bool stop = false;  // the abort flag, read once for the whole warp: lanes that saw
+                        // it at different times would wait for each other in item()
+    for (int i = 0; blockIdx.x + i * gridDim.x < nitems && !stop; ++i) {
       const TileItem& q = item(i);
-      for (int s0 = 0; s0 < q.n; s0 += 32) {
+      for (int s0 = 0; s0 < q.n && !stop; s0 += 32) {
         int kl = q.K0;
         if (i == 0 && s0 == 0) {
           kl = kl0;
@@ -153,7 +155,7 @@ __global__ void __launch_bounds__(ZTHREADS, 1) gemm_tcz_kernel(const GGroup* __r
           fence_maps(maps, sl);
           __syncwarp();
         }
-        for (int s = s0; s < min(q.n, s0 + 32); ++s) {
+        for (int s = s0; s < min(q.n, s0 + 32) && !stop; ++s) {
           const int K = __shfl_sync(0xffffffffu, kl, s - s0);
           if (lane == 0) {
             const CUtensorMap* ma = maps + 4 * q.seg(s) + 3;
@@ -172,10 +174,8 @@ __global__ void __launch_bounds__(ZTHREADS, 1) gemm_tcz_kernel(const GGroup* __r
               issued_s = it;
             }
           }
-          __syncwarp();
-          if (*abort_f) break;
+          stop = __any_sync(0xffffffffu, *abort_f);
         }
-        if (*abort_f) break;
       }
     }
   } else if (warp == 1) {
