@@ -62,6 +62,7 @@ struct CholF64 {
   // a - b c, accumulated
   static __device__ __forceinline__ Acc open(T a) { return a; }
   static __device__ __forceinline__ void fnms(Acc& a, T b, T c) { a = fma(-b, c, a); }
+  static __device__ __forceinline__ void tidy(Acc&) {}
   static __device__ __forceinline__ T close(Acc a) { return a; }
   // 1 / sqrt(d): float seed y of the mantissa's (1 - d y^2 = e below 2^-21),
   // y (1 + e/2 + 3 e^2 / 8) leaves ~e^3
@@ -80,69 +81,32 @@ struct CholF64 {
 struct CholDF {
   using T = float2;  // value x + y, |y| <= ulp(x) / 2
   using D = float;
-  using Acc = float2;  // not normalised
+  using Acc = float2;  // not normalised between fnms and tidy or close
   static constexpr double u = 1.4210854715202004e-14;  // 2^-46
   static __device__ __forceinline__ T of(double v) { return df_split(v); }
   // one FP64 addition (the conversions are integer operations)
   static __device__ __forceinline__ double dbl(T a) { return dbl_of_float(a.x) + dbl_of_float(a.y); }
   static __device__ __forceinline__ T zero() { return make_float2(0.f, 0.f); }
   static __device__ __forceinline__ T neg(T a) { return make_float2(-a.x, -a.y); }
-  static __device__ __forceinline__ T two_sum(float s, float t) {
-    const float h = s + t;
-    const float bp = h - s;
-    return make_float2(h, (s - (h - bp)) + (t - bp));
-  }
   static __device__ __forceinline__ T add(T a, double v) {
     const float2 b = df_split(v);
     const float s = a.x + b.x;
     const float bp = s - a.x;
     const float t = ((a.x - (s - bp)) + (b.x - bp)) + (a.y + b.y);
-    return two_sum(s, t);
+    return df_two_sum(s, t);
   }
   static __device__ __forceinline__ D dev(T a, double target) { return fabsf((a.x - (float)target) + a.y); }
-  static __device__ __forceinline__ T mul(T a, T b) {
-    const float p = a.x * b.x;
-    float e = fmaf(a.x, b.x, -p);
-    e = fmaf(a.x, b.y, e);
-    e = fmaf(a.y, b.x, e);
-    return two_sum(p, e);
-  }
+  static __device__ __forceinline__ T mul(T a, T b) { return df_mul(a, b); }
   static __device__ __forceinline__ bool positive(T a) { return a.x >= 1.17549435e-38f && isfinite(a.x); }
   static __device__ __forceinline__ T shfl(T a, int l) {
     return make_float2(__shfl_sync(0xffffffffu, a.x, l), __shfl_sync(0xffffffffu, a.y, l));
   }
   static __device__ __forceinline__ Acc open(T a) { return a; }
-  static __device__ __forceinline__ void fnms(Acc& a, T b, T c) {
-    const float p = b.x * c.x;
-    float e = fmaf(b.x, c.x, -p);  // b.x c.x = p + e exactly
-    e = fmaf(b.x, c.y, e);
-    e = fmaf(b.y, c.x, e);
-    const float s = a.x - p;  // a.x - p = s + t exactly
-    const float bp = s - a.x;
-    const float t = (a.x - (s - bp)) + (-p - bp);
-    a.y += t - e;
-    a.x = s;
-  }
-  static __device__ __forceinline__ T close(Acc a) { return two_sum(a.x, a.y); }
-  // y (1 + e/2 + 3 e^2 / 8) with y the float rsqrt and e = 1 - d y^2 taken in
-  // double-float (|e| < 2^-21, known to ~2^-45)
-  static __device__ __forceinline__ T rsqrt(T d) {
-    const float y = rsqrtf(d.x);
-    const float qh = y * y, ql = fmaf(y, y, -qh);
-    const float th = d.x * qh;
-    float tl = fmaf(d.x, qh, -th);
-    tl = fmaf(d.x, ql, tl);
-    tl = fmaf(d.y, qh, tl);
-    const float e = (1.f - th) - tl;
-    return two_sum(y, y * (e * fmaf(0.375f, e, 0.5f)));
-  }
-  // sqrt(d) from ip = 1 / sqrt(d): s = d ip, corrected by (d - s^2) ip / 2
-  static __device__ __forceinline__ T sqrt_of(T d, T ip) {
-    const T s = mul(d, ip);
-    Acc r = open(d);
-    fnms(r, s, s);
-    return two_sum(s.x, fmaf((r.x + r.y) * 0.5f, ip.x, s.y));
-  }
+  static __device__ __forceinline__ void fnms(Acc& a, T b, T c) { df_fnms(a, b, c); }
+  static __device__ __forceinline__ void tidy(Acc& a) { df_tidy(a); }
+  static __device__ __forceinline__ T close(Acc a) { return df_two_sum(a.x, a.y); }
+  static __device__ __forceinline__ T rsqrt(T d) { return df_rsqrt(d); }
+  static __device__ __forceinline__ T sqrt_of(T d, T ip) { return df_sqrt(d, ip); }
 };
 
 // t[e1] -= sum_s p1[s] x[s] and the same at e2 (skipped below zero; fresh: from
@@ -161,6 +125,8 @@ __device__ __forceinline__ void rank8(T* t, int e1, int e2, const T* p1, const T
   for (int s = 0; s < NB; ++s) {
     A::fnms(c1, q1[s], x[s]);
     A::fnms(c2, q2[s], x[s]);
+    A::tidy(c1);
+    A::tidy(c2);
   }
   if (e1 >= 0) t[e1] = A::close(c1);
   if (e2 >= 0) t[e2] = A::close(c2);
@@ -288,7 +254,10 @@ __global__ void __launch_bounds__(CHOL_T, 1) chol_inv_kernel(const CholJob* __re
           const T ri = P[(k0 + min(i, kb - 1)) * NB + t];
 #pragma unroll
           for (int q = 0; q < 2; ++q)
-            if (i <= j0 + q && j0 + q < kb) A::fnms(c[q], ri, P[(k0 + j0 + q) * NB + t]);
+            if (i <= j0 + q && j0 + q < kb) {
+              A::fnms(c[q], ri, P[(k0 + j0 + q) * NB + t]);
+              A::tidy(c[q]);
+            }
         }
       }
       a[0] = A::close(c[0]);

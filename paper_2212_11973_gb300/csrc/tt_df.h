@@ -82,4 +82,62 @@ __device__ __forceinline__ void dbl_of_pairs(const float* hi, const float* lo, d
   }
 }
 
+// Arithmetic on normalised pairs (|lo| <= ulp(hi) / 2), ~2^-46 relative.
+__device__ __forceinline__ float2 df_two_sum(float s, float t) {
+  const float h = s + t;
+  const float bp = h - s;
+  return make_float2(h, (s - (h - bp)) + (t - bp));
+}
+__device__ __forceinline__ float2 df_mul(float2 a, float2 b) {
+  const float p = a.x * b.x;
+  float e = fmaf(a.x, b.x, -p);
+  e = fmaf(a.x, b.y, e);
+  e = fmaf(a.y, b.x, e);
+  return df_two_sum(p, e);
+}
+// a - b c; the result is not normalised
+__device__ __forceinline__ void df_fnms(float2& a, float2 b, float2 c) {
+  const float p = b.x * c.x;
+  float e = fmaf(b.x, c.x, -p);  // b.x c.x = p + e exactly
+  e = fmaf(b.x, c.y, e);
+  e = fmaf(b.y, c.x, e);
+  const float s = a.x - p;  // a.x - p = s + t exactly
+  const float bp = s - a.x;
+  const float t = (a.x - (s - bp)) + (-p - bp);
+  a.y += t - e;
+  a.x = s;
+}
+// normalises in three operations (Dekker's order: the high part is the larger, or
+// both are rounding errors of what cancelled).  Without it after each of 8 terms
+// the low part grows, and a Cholesky factor of n = 180 is 1.5 times further from
+// its matrix (rms of R^T R - G: 1.6e-15 against 1.1e-15 of the diagonal).
+__device__ __forceinline__ void df_tidy(float2& a) {
+  const float h = a.x + a.y;
+  a.y = a.y - (h - a.x);
+  a.x = h;
+}
+// 1 / sqrt(d): y the float rsqrt and e = 1 - d y^2 as a pair (|e| < 2^-20), then
+// y (1 + e / 2 + 3 e^2 / 8) with the product by e / 2 as a pair: 2^-46.9 (in one FP32
+// term: 2^-44)
+__device__ __forceinline__ float2 df_rsqrt(float2 d) {
+  const float y = rsqrtf(d.x);
+  const float qh = y * y, ql = fmaf(y, y, -qh);
+  const float th = d.x * qh;
+  float tl = fmaf(d.x, qh, -th);
+  tl = fmaf(d.x, ql, tl);
+  tl = fmaf(d.y, qh, tl);
+  const float2 e = df_two_sum(1.f - th, -tl);
+  const float g = 0.5f * y, p = g * e.x;
+  const float q = fmaf(y, fmaf(0.375f * e.x, e.x, 0.5f * e.y), fmaf(g, e.x, -p));
+  const float2 r = df_two_sum(y, p);
+  return df_two_sum(r.x, r.y + q);
+}
+// sqrt(d) from ip = 1 / sqrt(d): s = d ip, corrected by (d - s^2) ip / 2
+__device__ __forceinline__ float2 df_sqrt(float2 d, float2 ip) {
+  const float2 s = df_mul(d, ip);
+  float2 r = d;
+  df_fnms(r, s, s);
+  return df_two_sum(s.x, fmaf((r.x + r.y) * 0.5f, ip.x, s.y));
+}
+
 }  // namespace tt

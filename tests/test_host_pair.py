@@ -34,6 +34,7 @@ def pairs(tmp_path_factory):
         lib.h_pairs(hi.ctypes.data_as(f), lo.ctypes.data_as(f), v.ctypes.data_as(d), C.c_int64(hi.size))
         return v
 
+    run.lib = lib
     return run
 
 
@@ -78,3 +79,46 @@ def test_edges(pairs):
     sub = (rng.integers(-2 ** 23, 2 ** 23, 200000) * 2.0 ** -149).astype(np.float32)
     near = (rng.integers(-2 ** 27, 2 ** 27, sub.size) * 2.0 ** -149).astype(np.float32)
     _same(pairs(near, sub), near, sub)
+
+
+def _f64(a):
+    return a.ctypes.data_as(C.POINTER(C.c_double))
+
+
+@pytest.fixture(scope="module")
+def lib(pairs):
+    return pairs.lib
+
+
+def test_roots_of_pairs(lib):
+    """1 / sqrt(d) and sqrt(d) of a pair from a float seed up to 2 ulp off: e = 1 - d
+    y^2 is known to 2^-48 (three roundings of terms below 2^-24), half of it and the
+    roundings of the last two sums (2^-48 each) and of d to a pair (2^-47, half of it
+    in the root): 2^-46 in all."""
+    n = 200000
+    d = np.exp(np.random.default_rng(4).uniform(-20, 20, n))
+    root = np.sqrt(d.astype(np.longdouble))
+    for off in range(-2, 3):
+        r, rl, s, sl = (np.empty(n) for _ in range(4))
+        lib.h_roots(_f64(d), off, _f64(r), _f64(rl), _f64(s), _f64(sl), C.c_int64(n))
+        assert np.abs((r.astype(np.longdouble) + rl) * root - 1).max() <= 2.0 ** -46
+        assert np.abs((s.astype(np.longdouble) + sl) / root - 1).max() <= 2.0 ** -46
+
+
+def test_rank8_update(lib):
+    """a - sum of 8 products on pairs of exact 46-bit values, normalised after each
+    term: the low part stays below 2^-24 of the partial sum and takes three roundings
+    a term, each of rms 2^-24 2^-24 / sqrt(12) of the largest of them: sqrt(24) of
+    them give 2^-48.5 of the largest, 2^-50 of the sum of the magnitudes (8 terms
+    of like size); doubled for the seven partial sums above the mean.  Left
+    unnormalised, the low part grows with the terms: 2^-48.8."""
+    rng = np.random.default_rng(5)
+    n = 200000
+    a, b, c = (np.rint(rng.standard_normal(k) * 2.0 ** 42) * 2.0 ** -42 for k in (n, 8 * n, 8 * n))
+    out = np.empty(n)
+    lib.h_rank8(_f64(a), _f64(b), _f64(c), _f64(out), C.c_int64(n))
+    x = np.longdouble
+    want = a.astype(x) - (b.astype(x) * c.astype(x)).reshape(n, 8).sum(1)
+    scale = np.abs(a) + np.abs(b * c).reshape(n, 8).sum(1)
+    err = ((out - want) / scale).astype(float)
+    assert np.sqrt((err ** 2).mean()) <= 2.0 ** -49
