@@ -11,8 +11,8 @@
 // memory, or for sectors too large for it in the job's workspace scratch, and
 // factorised and then inverted in place in blocks of NB = 8 rows:
 //   factor, from the top:    one warp factorises the diagonal block in registers
-//     (a column per lane) and inverts it; a thread per column solves the block
-//     row; every warp updates trailing rows with all 8 pivot rows at once;
+//     (two columns of a row per lane) and inverts it; a thread per column solves the
+//     block row; every warp updates trailing rows with all 8 pivot rows at once;
 //   inverse, from the bottom (S holds - sum R X): block row X = D S with the
 //     diagonal block's inverse D, then every row above takes its rank-8 update,
 //     with the block's columns of R copied aside first.
@@ -22,8 +22,8 @@
 // What bounds it: the chain of n pivots on one CTA.  Row by row (one pivot with
 // a square root and a division in FP64, three barriers and a pass over the
 // trailing triangle each) a step took ~2.8 us; in blocks of 8 a pivot's scalar
-// is a float rsqrt and one Newton step (~1000 clocks with the exchange of its
-// row), there are 4 barriers per 8 rows, the next diagonal block is factorised
+// is a float rsqrt and one third-order correction (~1000 clocks with the exchange
+// of its row), there are 4 barriers per 8 rows, the next diagonal block is factorised
 // while the trailing triangle is updated, and a trailing element is loaded and
 // stored once per 8 multiply-adds whose other operands sit in registers or are
 // one broadcast load.  Measured, double-float, one sector with its partial
@@ -42,6 +42,17 @@ namespace {
 
 constexpr int CHOL_T = 512, CHOL_W = CHOL_T / 32, NB = 8;
 constexpr size_t CHOL_SMEM = 226 * 1024;
+
+// elements of a job's packed triangle, to a 16-byte boundary, and the largest n whose
+// triangle and n x 8 copies fit shared memory together (232)
+__host__ __device__ constexpr int tri_elems(int n) { return (n * (n + 1) / 2 + 1) & ~1; }
+constexpr size_t chol_bytes(int n) { return ((size_t)tri_elems(n) + (size_t)NB * n) * 8; }
+constexpr int chol_max_n() {
+  int n = 0;
+  while (chol_bytes(n + 1) <= CHOL_SMEM) ++n;
+  return n;
+}
+constexpr int CHOL_MAXN = chol_max_n();
 
 __device__ __forceinline__ int pk(int i, int j, int n) { return i * n - (i * (i - 1)) / 2 + (j - i); }
 
@@ -134,7 +145,7 @@ __device__ __forceinline__ void rank8(T* t, int e1, int e2, const T* p1, const T
 
 template <class A>
 __global__ void __launch_bounds__(CHOL_T, 1) chol_inv_kernel(const CholJob* __restrict__ jobs, double* __restrict__ ws,
-                                                             int* __restrict__ fail, int smax, int tri) {
+                                                             int* __restrict__ fail) {
   using T = typename A::T;
   using D = typename A::D;
   extern __shared__ __align__(16) unsigned char chol_raw[];
@@ -146,18 +157,18 @@ __global__ void __launch_bounds__(CHOL_T, 1) chol_inv_kernel(const CholJob* __re
   }
   if (fail[J.sec]) return;
   // the packed triangle: shared memory, or the job's workspace scratch (L2
-  // resident) for the sectors too large for it; then n x 8: a block's columns or rows of R, for broadcast
-  // loads
-  T* sm = n <= smax ? reinterpret_cast<T*>(chol_raw) : reinterpret_cast<T*>(ws + J.pk);
-  T* P = reinterpret_cast<T*>(chol_raw) + tri;
+  // resident) for the sectors too large for it; then n x 8: a block's columns or rows
+  // of R, for broadcast loads
+  const bool in_smem = n <= CHOL_MAXN;
+  T* sm = in_smem ? reinterpret_cast<T*>(chol_raw) : reinterpret_cast<T*>(ws + J.pk);
+  T* P = reinterpret_cast<T*>(chol_raw) + (in_smem ? tri_elems(n) : 0);
   const double* G = ws + J.g;
   double* R = ws + J.r;
   double* Ri = ws + J.ri;
   const long long nn = (long long)n * n;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   __shared__ D red[CHOL_W];
-  __shared__ T dg[NB][NB];    // diagonal block (rows of R) and its inverse
-  __shared__ T dgi[NB][NB];
+  __shared__ T dg[NB][NB];    // diagonal block (rows of R)
   __shared__ T dip[NB];       // reciprocals of its pivots
   __shared__ int bad;
   // G: the partial matrices of one element all in flight (one load at a time, a
@@ -416,13 +427,10 @@ __global__ void __launch_bounds__(CHOL_T, 1) chol_inv_kernel(const CholJob* __re
 
 cudaError_t launch_chol_inv(const CholJob* jobs, int njobs, double* ws, int* fail, cudaStream_t s, int maxn, bool df) {
   if (njobs == 0) return cudaSuccess;
-  // the column copy, and the triangle of every sector that fits beside it
-  const size_t copy = (size_t)NB * maxn * 8;
+  // every job's own triangle and copies (of a sector too large for it the copies)
+  const size_t copy = (size_t)NB * maxn * 8, small = chol_bytes(maxn < CHOL_MAXN ? maxn : CHOL_MAXN);
   if (copy > CHOL_SMEM) return cudaErrorInvalidValue;
-  int smax = 0;
-  while (smax < maxn && ((size_t)(smax + 1) * (smax + 2) / 2 + 1) * 8 + copy <= CHOL_SMEM) ++smax;
-  const int tri = (smax * (smax + 1) / 2 + 1) & ~1;  // (16-byte rows after it)
-  const size_t smem = (size_t)tri * 8 + copy;
+  const size_t smem = copy > small ? copy : small;
   // once per process (thread-safe static initialisation): the largest size
   static const cudaError_t e1 =
       cudaFuncSetAttribute(chol_inv_kernel<CholF64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CHOL_SMEM);
@@ -430,8 +438,8 @@ cudaError_t launch_chol_inv(const CholJob* jobs, int njobs, double* ws, int* fai
       cudaFuncSetAttribute(chol_inv_kernel<CholDF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CHOL_SMEM);
   if (e1 != cudaSuccess) return e1;
   if (e2 != cudaSuccess) return e2;
-  if (df) chol_inv_kernel<CholDF><<<njobs, CHOL_T, smem, s>>>(jobs, ws, fail, smax, tri);
-  else chol_inv_kernel<CholF64><<<njobs, CHOL_T, smem, s>>>(jobs, ws, fail, smax, tri);
+  if (df) chol_inv_kernel<CholDF><<<njobs, CHOL_T, smem, s>>>(jobs, ws, fail);
+  else chol_inv_kernel<CholF64><<<njobs, CHOL_T, smem, s>>>(jobs, ws, fail);
   return cudaGetLastError();
 }
 

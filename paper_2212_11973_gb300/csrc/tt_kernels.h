@@ -209,8 +209,8 @@ cudaError_t launch_qr_job(const QrJob& job, double* ws, cudaStream_t s);
 cudaError_t launch_qr_masked(const QrJob* jobs, int njobs, double* ws, const int* only, int* nrun, cudaStream_t s);
 // Cholesky + triangular inverse per job (shifted on request); fail[sec] set on
 // a non-positive pivot.
-// maxn: the largest n of the jobs (shared-memory variant up to 230); df: that
-// variant in double-float arithmetic (~2^-46) instead of FP64.
+// maxn: the largest n of the jobs (those up to 232 in shared memory); df:
+// double-float arithmetic (~2^-46) instead of FP64.
 cudaError_t launch_chol_inv(const CholJob* jobs, int njobs, double* ws, int* fail, cudaStream_t s, int maxn = 0,
                             bool df = false);
 // Sign fix diag(R) >= 0 done inside launch_qr.
