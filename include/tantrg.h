@@ -363,8 +363,10 @@ tt_status tt_layout_sizes_terms(int nw_l, const int* chl_qn, const int* chl_qs, 
  * A_i = A_i^L S_i by QR): A = Q R for a column-major m x n matrix (ld = m,
  * 1 <= n <= min(m, 2048)), Householder in FP64, sign convention diag(R) >= 0.
  * A, Q (m x n, column-major) and R (n x n, column-major, upper triangular) are
- * device pointers; A is not modified.  Scratch comes from the context
- * allocator.  Synchronises the context stream. */
+ * device pointers; A is not modified (Q and R may overlap it and each other, on
+ * one CTA).  Scratch comes from the context allocator.  Synchronises the context
+ * stream.  Waits between the columns' CTAs keep to tt_ctx_set_wait_limit; where one
+ * runs out, one CTA factorises instead. */
 tt_status tt_qr_device(tt_ctx* ctx, const double* A, int m, int n, double* Q, double* R);
 
 /* The same QR without any device allocation, for callers that may not allocate

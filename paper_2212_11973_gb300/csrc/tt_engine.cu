@@ -3317,18 +3317,22 @@ tt_status tt_qr_device(tt_ctx* ctx, const double* A, int m, int n, double* Q, do
   tt_status st = guarded(ctx, nullptr, [&] {
     const int64_t mn = (int64_t)m * n;
     auto apart = [](const double* a, int64_t na, const double* b, int64_t nb) { return a + na <= b || b + nb <= a; };
-    if (apart(A, mn, Q, mn) && apart(A, mn, R, (int64_t)n * n) && apart(Q, mn, R, (int64_t)n * n)) {
+    int ctas = 0;
+    if (apart(A, mn, Q, mn) && apart(A, mn, R, (int64_t)n * n) && apart(Q, mn, R, (int64_t)n * n))
+      CK(qr_grid_ctas(m, n, &ctas));
+    if (ctas > 0) {
       ensure(ctx, ws, qr_grid_scratch(m, n));
       int *err = nullptr, timed_out = 0;
       bool done = false;
-      // a budget of its own: the factorisation is accepted under every wait limit of the context
-      CK(launch_qr_grid(A, m, n, Q, R, ws.p, 2000000000ll, ctx->st, &err, &done));
+      CK(launch_qr_grid(A, m, n, ctas, Q, R, ws.p, ctx->wait_ns, ctx->st, &err, &done));
       if (done) {
         CK(cudaMemcpyAsync(&timed_out, err, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
         CK(cudaStreamSynchronize(ctx->st));
-        if (timed_out) throw Err{TT_ERR_TIMEOUT, "tt_qr_device: a wait between the columns' CTAs ran out"};
-        return;
+        if (!timed_out) return;
       }
+      // refused, or given up (A is as it was): one CTA, which waits for nobody.  (The
+      // scratch is given back first: growing a buffer would drop captured steps.)
+      dfree(ctx, ws);
     }
     ensure(ctx, ws, (size_t)(2 * mn + (int64_t)n * n) * sizeof(double));
     ensure(ctx, job, sizeof(QrJob));

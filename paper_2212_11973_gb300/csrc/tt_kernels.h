@@ -195,12 +195,13 @@ cudaError_t k_normalise_inplace(double* v, int64_t n, double* partial, KrylovSta
 cudaError_t launch_qr(const QrJob* jobs, int njobs, double* ws, cudaStream_t s);
 // The same factorisation of one matrix over the whole GPU (tt_qrgrid.cu): A, Q
 // (m x n) and R (n x n) column-major, not overlapping; scratch of
-// qr_grid_scratch(m, n) bytes.  *done is false where the kernel does not apply
-// (nothing launched); otherwise *err points at a device int that is set when a
-// bounded wait (wait_ns) ran out.
+// qr_grid_scratch(m, n) bytes.  qr_grid_ctas: the CTAs it takes, 0 where it does not
+// apply.  *done is false where the device refused the launch; otherwise *err points
+// at a device int that is set when a bounded wait (wait_ns) ran out.
+cudaError_t qr_grid_ctas(int m, int n, int* ctas);
 size_t qr_grid_scratch(int m, int n);
-cudaError_t launch_qr_grid(const double* A, int m, int n, double* Q, double* R, void* scratch, long long wait_ns,
-                           cudaStream_t s, int** err, bool* done);
+cudaError_t launch_qr_grid(const double* A, int m, int n, int ctas, double* Q, double* R, void* scratch,
+                           long long wait_ns, cudaStream_t s, int** err, bool* done);
 // one job passed by value (the record is a kernel argument, not device memory)
 cudaError_t launch_qr_job(const QrJob& job, double* ws, cudaStream_t s);
 // the same, only for the jobs whose only[job] != 0

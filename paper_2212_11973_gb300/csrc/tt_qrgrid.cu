@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(GT, 1) qr_grid_kernel(const double* __restrict
                                                         double* __restrict__ R, long long wait_ns) {
   extern __shared__ __align__(16) double sm[];
   __shared__ double red[2][GW][2];
-  __shared__ double bc[2];
+  __shared__ double ws_s;
   __shared__ int stop;
   const int c = blockIdx.x, G = gridDim.x, tid = threadIdx.x;
   const int ncol = (n - c + G - 1) / G;  // own columns c, c + G, ...
@@ -145,14 +145,13 @@ __global__ void __launch_bounds__(GT, 1) qr_grid_kernel(const double* __restrict
         }
         if (tid == 0) {
           const double w = q < ncol ? tau * fma(scale, sd.y, cj[k]) : 0.0;
-          bc[0] = w;
-          bc[1] = w * scale;
+          ws_s = w * scale;
           if (q < ncol) cj[k] -= w;
         }
       }
       __syncthreads();
       if (q < ncol) {
-        const double ws = bc[1];
+        const double ws = ws_s;
 #pragma unroll
         for (int e = 0; e < E; ++e) {
           const int i = tid + e * GT;
@@ -219,29 +218,33 @@ __global__ void __launch_bounds__(GT, 1) qr_grid_kernel(const double* __restrict
 // CTAs for an m x n matrix, or 0 where the kernel does not apply (a column
 // longer than its register tile, or more of them per CTA than shared memory
 // holds: the one-CTA kernel's case)
-static int qr_grid_ctas(int m, int n, int sms) {
+static int ctas_of(int m, int n, int sms) {
   if (m > GT * GE) return 0;
   const int G = std::min(n, sms), cp = (n + G - 1) / G;
   return ((size_t)cp * m + 2 * (size_t)n) * sizeof(double) <= GSMEM ? G : 0;
 }
 
-size_t qr_grid_scratch(int m, int n) { return (size_t)m * n * sizeof(double) + ((size_t)n + 1) * sizeof(int); }
-
-cudaError_t launch_qr_grid(const double* A, int m, int n, double* Q, double* R, void* scratch, long long wait_ns,
-                           cudaStream_t s, int** err, bool* done) {
-  *done = false;
-  *err = nullptr;
+cudaError_t qr_grid_ctas(int m, int n, int* ctas) {
+  *ctas = 0;
   int dev = 0, sms = 0, coop = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-  if (e != cudaSuccess) return e;
-  const int G = coop ? qr_grid_ctas(m, n, sms) : 0;
-  if (G == 0) return cudaSuccess;
+  if (e == cudaSuccess && coop) *ctas = ctas_of(m, n, sms);
+  return e;
+}
+
+size_t qr_grid_scratch(int m, int n) { return (size_t)m * n * sizeof(double) + ((size_t)n + 1) * sizeof(int); }
+
+cudaError_t launch_qr_grid(const double* A, int m, int n, int ctas, double* Q, double* R, void* scratch,
+                           long long wait_ns, cudaStream_t s, int** err, bool* done) {
+  *done = false;
+  *err = nullptr;
+  const int G = ctas;
   double* V = (double*)scratch;
   int* flag = (int*)(V + (size_t)m * n);
   int* er = flag + n;
-  e = cudaMemsetAsync(flag, 0, ((size_t)n + 1) * sizeof(int), s);
+  cudaError_t e = cudaMemsetAsync(flag, 0, ((size_t)n + 1) * sizeof(int), s);
   if (e != cudaSuccess) return e;
   const size_t smem = ((size_t)((n + G - 1) / G) * m + 2 * (size_t)n) * sizeof(double);
   const int el = (m + GT - 1) / GT;
@@ -252,6 +255,10 @@ cudaError_t launch_qr_grid(const double* A, int m, int n, double* Q, double* R, 
   if (e != cudaSuccess) return e;
   void* args[] = {(void*)&A, &m, &n, &V, &flag, &er, &Q, &R, &wait_ns};
   e = cudaLaunchCooperativeKernel(k, dim3(G), dim3(GT), args, smem, s);
+  if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {  // (a share of the GPU only)
+    cudaGetLastError();
+    return cudaSuccess;
+  }
   if (e != cudaSuccess) return e;
   *err = er;
   *done = true;
