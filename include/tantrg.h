@@ -249,7 +249,8 @@ tt_status tt_rho_pad(tt_rho* rho, const tt_mpo* mpo, int D_target);
  * next as a CUDA graph; later steps replay it (re-captured after a change of
  * dtau, of the profiling mode or of any device buffer).  Set the environment
  * variable TT_CUDA_GRAPH=0 to launch every kernel directly; TT_QR=householder
- * selects the one-CTA Householder QR for every sector. */
+ * selects the one-CTA Householder QR for every sector, TT_QR_GEMM=df or f64 the
+ * kernel of the gauge's products in the mixed modes (else the faster per plan). */
 tt_status tt_tdvp_step(tt_rho* rho, const tt_mpo* mpo, double dtau, int n_steps);
 
 /* Observables at the canonical centre (site 0 after a step).  Synchronises the

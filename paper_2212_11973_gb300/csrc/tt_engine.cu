@@ -121,7 +121,7 @@ static std::vector<GTile> tiles64_of(const GemmPlan& p) {
 
 // The plan's arrays into a stager, with the tile list of the kernel it is known
 // to run on (else the lists follow when a launch first needs them).
-enum TileList { TL_LATER = 0, TL_F64 = 1, TL_QR = 2 };  // TL_QR: FP64, and double-float where it is faster
+enum TileList { TL_LATER = 0, TL_F64 = 1, TL_DF = 2, TL_QR = 3 };  // TL_QR: the faster of the two
 static void upload(Stager& s, GemmPlan p, DevGemmBuf& o, int list = TL_LATER) {
   s.add(p.groups, &o.d.groups);
   s.add(p.segs, &o.d.segs);
@@ -135,7 +135,7 @@ static void upload(Stager& s, GemmPlan p, DevGemmBuf& o, int list = TL_LATER) {
   o.nordered = o.tordered = 0;
   o.d.ntilesf = o.d.tf = 0;
   o.d.ntilesd = -1;
-  o.df = list == TL_QR && df_beats_f64(p);
+  o.df = list == TL_DF || (list == TL_QR && df_beats_f64(p));
   if (o.df) {
     const std::vector<FTile> t = f64_tiles(p, df_tile_size());
     s.add(t, &o.d.tilesd);
@@ -604,8 +604,8 @@ struct Eng {
       for (int p = 0; p < 3; ++p) {
         check_plan(cp.gram[p], cw, "CholQR gram");
         check_plan(cp.app[p], cw, "CholQR apply");
-        upload(g, std::move(cp.gram[p]), q.gram[p], TL_QR);
-        upload(g, std::move(cp.app[p]), q.app[p], TL_QR);
+        upload(g, std::move(cp.gram[p]), q.gram[p], r->qr_list);
+        upload(g, std::move(cp.app[p]), q.app[p], r->qr_list);
         for (const CholJob& J : cp.cj[p])
           if (J.g + (int64_t)J.parts * J.n * J.n > wsz || J.parts < 1 || J.r + (int64_t)J.n * J.n > wsz ||
               J.ri + (int64_t)J.n * J.n > wsz || J.pk < 0 || J.pk + (int64_t)J.n * (J.n + 1) / 2 > wsz)
@@ -2529,6 +2529,8 @@ void alloc_rho_arrays(tt_rho* r) {
     r->use_graph = !(gg && std::strcmp(gg, "0") == 0);
     const char* gq = std::getenv("TT_QR");
     r->use_cholqr = !(gq && std::strcmp(gq, "householder") == 0);
+    const char* gp = std::getenv("TT_QR_GEMM");  // gauge products of the mixed modes
+    r->qr_list = gp && !std::strcmp(gp, "df") ? TL_DF : (gp && !std::strcmp(gp, "f64") ? TL_F64 : TL_QR);
   }
   r->sp.assign(N, SiteDev());
   r->sp64.assign(N, SiteDev());

@@ -173,6 +173,7 @@ struct tt_rho {
   bool apply_only = false;                // a single H_eff apply: no sweep buffers or plans
   bool use_tc = true;                     // tcgen05 kernel for eligible split-bf16 GEMMs
   bool use_cholqr = true;                 // CholeskyQR3 gauge (else Householder only)
+  int qr_list = 0;                        // tile lists of its products (TileList)
   std::vector<tt::SiteDev> sp;
   std::vector<tt::SiteDev> sp64;
   unsigned long long graph_buf_gen = 0;  // FP64 site plans used by the measurement in mixed mode
