@@ -604,8 +604,9 @@ struct Eng {
       for (int p = 0; p < 3; ++p) {
         check_plan(cp.gram[p], cw, "CholQR gram");
         check_plan(cp.app[p], cw, "CholQR apply");
-        upload(g, std::move(cp.gram[p]), q.gram[p], r->qr_list);
-        upload(g, std::move(cp.app[p]), q.app[p], r->qr_list);
+        // (FP64 mode runs no double-float product)
+        upload(g, std::move(cp.gram[p]), q.gram[p], mixed() ? r->qr_list : TL_F64);
+        upload(g, std::move(cp.app[p]), q.app[p], mixed() ? r->qr_list : TL_F64);
         for (const CholJob& J : cp.cj[p])
           if (J.g + (int64_t)J.parts * J.n * J.n > wsz || J.parts < 1 || J.r + (int64_t)J.n * J.n > wsz ||
               J.ri + (int64_t)J.n * J.n > wsz || J.pk < 0 || J.pk + (int64_t)J.n * (J.n + 1) / 2 > wsz)
