@@ -73,11 +73,6 @@ void ensure(tt_ctx* c, DBuf& b, size_t bytes) {
   b.bytes = want;
 }
 
-template <class T>
-static size_t align_up(size_t x) {
-  return (x + 255) / 256 * 256 + 0 * sizeof(T);
-}
-
 // Arrays of one or more plans gathered on the host and sent to the device in one
 // allocation and one copy: a site has ten plans of several arrays each, and an
 // allocation, a pageable copy and a synchronisation apiece took longer than
@@ -2545,7 +2540,7 @@ void alloc_rho_arrays(tt_rho* r) {
   r->meas.assign(N, MeasDev());
   if (r->apply_only) return;
   tt_ctx* c = r->ctx;
-  ensure(c, r->partial, (size_t)lanczos_nblk() * 17 * 8);
+  ensure(c, r->partial, (size_t)VEC_CTAS * VEC_SUMS * 8);
   ensure(c, r->ks, sizeof(KrylovState));
   CK(cudaMemsetAsync(r->ks.p, 0, sizeof(KrylovState), c->st));
   ensure(c, r->rs, sizeof(RhoScalars));

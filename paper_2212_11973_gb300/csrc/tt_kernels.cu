@@ -29,7 +29,6 @@ __device__ __forceinline__ T* rptr(const Bases& b, Ref r) {
   return reinterpret_cast<T*>(sel_base(b, slot_of(r))) + off_of(r);
 }
 
-constexpr int NBLK = 304;  // 2 x 152 SMs for the vector reductions
 constexpr int VT = 256;
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -344,17 +343,17 @@ __global__ void sumsq_kernel(const double* __restrict__ v, long long n, double* 
   if (threadIdx.x == 0) {
     double t = 0.0;
     for (int q = 0; q < VT / 32; ++q) t += red[q];
-    partial[blockIdx.x * 17] = t;
+    partial[blockIdx.x * VEC_SUMS] = t;
   }
 }
 
-// out[j] = sum_b partial[b * 17 + j] in a fixed order (deterministic)
+// out[j] = sum_b partial[b * VEC_SUMS + j] in a fixed order (deterministic)
 __device__ void finalize_sums(const double* partial, int nblk, int nv, double* out) {
   // called by one warp
   const int lane = threadIdx.x & 31;
   for (int j = 0; j < nv; ++j) {
     double s = 0.0;
-    for (int b = lane; b < nblk; b += 32) s += partial[b * 17 + j];
+    for (int b = lane; b < nblk; b += 32) s += partial[b * VEC_SUMS + j];
     s = warp_sum(s);
     if (lane == 0) out[j] = s;
   }
@@ -493,7 +492,7 @@ __global__ void __launch_bounds__(VT) dot_kernel(const double* __restrict__ x, c
   if (threadIdx.x == 0) {
     double t = 0.0;
     for (int q = 0; q < VT / 32; ++q) t += red[q];
-    partial[blockIdx.x * 17] = t;
+    partial[blockIdx.x * VEC_SUMS] = t;
   }
 }
 
@@ -543,7 +542,7 @@ __global__ void scale_rc_kernel(double* __restrict__ a, long long ld, int rows, 
 
 inline int grid_for(long long n) {
   long long g = (n + VT - 1) / VT;
-  if (g > NBLK) g = NBLK;
+  if (g > VEC_CTAS) g = VEC_CTAS;
   if (g < 1) g = 1;
   return (int)g;
 }
@@ -553,8 +552,6 @@ inline int grid_for(long long n) {
 // ---------------------------------------------------------------------------
 // host wrappers
 // ---------------------------------------------------------------------------
-int lanczos_nblk() { return NBLK; }
-
 cudaError_t launch_gemm_bf16(const DevGemm& g, const Bases& b, int nsplit, cudaStream_t s) {
   if (g.ntiles64 == 0) return cudaSuccess;
   if (nsplit == 2) gemm_bf16_split_kernel<2><<<g.ntiles64, 128, 0, s>>>(g.groups, g.segs, g.tiles64, b);

@@ -166,8 +166,10 @@ cudaError_t launch_gemm_tc(const GGroup* groups, const GSeg* segs, const GTile* 
 
 // Lanczos exponential on flat FP64 vectors of length n (tt_lanczos.cu).  Q holds
 // the Krylov basis with leading dimension ldq; `partial` is scratch of
-// lanczos_nblk() * 17 doubles; ks->ticket must be zero before the first use.
-int lanczos_nblk();
+// VEC_CTAS * VEC_SUMS doubles; ks->ticket must be zero before the first use.
+// Most CTAs of a vector reduction (2 x 152 SMs), and sums per CTA of one
+// (Krylov dimension 16 and one): kernels and their scratch go by these.
+constexpr int VEC_CTAS = 304, VEC_SUMS = 17;
 // ks reset, ks->nb = |x|, q0 = x / |x|
 cudaError_t k_lanczos_begin(const double* x, int64_t n, double* partial, KrylovState* ks, double* q0, cudaStream_t s);
 // step k of K after w = H q_k: alpha_k, beta_k and q_{k+1} (in Q); the last

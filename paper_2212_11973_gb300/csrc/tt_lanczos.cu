@@ -35,10 +35,9 @@ namespace tt {
 
 namespace {
 
-constexpr int LBLK = 304;  // 2 x 152 SMs
 constexpr int LT = 256;
 constexpr int LW = LT / 32;
-constexpr int LMAX = 17;  // values per partial record
+constexpr int LMAX = VEC_SUMS;  // values per partial record
 
 // sums of a[0..V-1] over the warp: value i ends in every lane with
 // lane >> (5 - log2 V) == i
@@ -373,7 +372,7 @@ __global__ void __launch_bounds__(LT) lanczos_combine(const double* __restrict__
 
 int lgrid(int64_t n) {
   const int64_t g = (n + LT - 1) / LT;
-  return (int)(g > LBLK ? LBLK : (g < 1 ? 1 : g));
+  return (int)(g > VEC_CTAS ? VEC_CTAS : (g < 1 ? 1 : g));
 }
 
 }  // namespace

@@ -53,7 +53,7 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// this CTA's sum of acc to partial[blockIdx.x * 17]
+// this CTA's sum of acc to partial[blockIdx.x * VEC_SUMS]
 __device__ __forceinline__ void publish(double acc, double* __restrict__ partial) {
   __shared__ double red[VT / 32];
   const double s = warp_sum(acc);
@@ -62,16 +62,16 @@ __device__ __forceinline__ void publish(double acc, double* __restrict__ partial
   if (threadIdx.x == 0) {
     double t = 0.0;
     for (int q = 0; q < VT / 32; ++q) t += red[q];
-    partial[blockIdx.x * 17] = t;
+    partial[blockIdx.x * VEC_SUMS] = t;
   }
 }
 
-// out[j] = sum_b partial[b * 17 + j], by one warp
+// out[j] = sum_b partial[b * VEC_SUMS + j], by one warp
 __device__ void finalize_sums(const double* partial, int nblk, int nv, double* out) {
   const int lane = threadIdx.x & 31;
   for (int j = 0; j < nv; ++j) {
     double s = 0.0;
-    for (int b = lane; b < nblk; b += 32) s += partial[b * 17 + j];
+    for (int b = lane; b < nblk; b += 32) s += partial[b * VEC_SUMS + j];
     s = warp_sum(s);
     if (lane == 0) out[j] = s;
   }
@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(VT) multidot_kernel(const double* __restrict__
   if (threadIdx.x < nv) {
     double s = 0.0;
     for (int q = 0; q < VT / 32; ++q) s += red[q][threadIdx.x];
-    partial[blockIdx.x * 17 + threadIdx.x] = s;
+    partial[blockIdx.x * VEC_SUMS + threadIdx.x] = s;
   }
 }
 
@@ -580,8 +580,8 @@ __global__ void __launch_bounds__(VT) gather_digits_rows_kernel(const GItem* __r
 }
 
 int grid_for(long long n) {
-  const long long g = (n + VT - 1) / VT, most = lanczos_nblk();
-  return (int)(g > most ? most : (g < 1 ? 1 : g));
+  const long long g = (n + VT - 1) / VT;
+  return (int)(g > VEC_CTAS ? VEC_CTAS : (g < 1 ? 1 : g));
 }
 
 }  // namespace
