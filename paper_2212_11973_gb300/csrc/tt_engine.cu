@@ -126,6 +126,9 @@ static void upload(Stager& s, GemmPlan p, DevGemmBuf& o, int list = TL_LATER) {
   o.d.flops = p.flops;
   o.checked = false;
   o.tc_checked = o.tc_ok = false;
+  o.out32 = !p.groups.empty() && (p.groups[0].flags & 2) ? 1 : 0;
+  for (const GGroup& g : p.groups)
+    if (((g.flags & 2) ? 1 : 0) != o.out32) o.out32 = -1;
   o.ntiles128 = o.ntilesp = 0;
   o.nordered = o.tordered = 0;
   o.d.ntilesf = o.d.tf = 0;
@@ -704,7 +707,8 @@ struct Eng {
   bool prep_tc(DevGemmBuf& g, const Bases& b) {
     if (!g.tc_checked) {
       g.tc_checked = true;
-      g.tc_ok = !g.host.segs.empty();
+      // (the persistent kernels write one output form per launch)
+      g.tc_ok = !g.host.segs.empty() && g.out32 >= 0;
       for (const GSeg& sg : g.host.segs) {
         const int64_t oa = (int64_t)(sg.A & 0x00FFFFFFFFFFFFFFull), ob = (int64_t)(sg.B & 0x00FFFFFFFFFFFFFFull);
         if (sg.tA != 0 || sg.tB != 1 || sg.lda % 8 || sg.ldb % 8 || oa % 8 || ob % 8) g.tc_ok = false;
@@ -874,7 +878,7 @@ struct Eng {
                         (int*)r->tcerr.p, c->wait_ns, st));
     else if (k == TK_TCP128X64)
       CK(launch_gemm_tcp(g.d.groups, g.d.segs, g.tilesp, g.ntilesp, split_tiles(g), tc_box(g), g.maps, b, r->nsplit,
-                         !g.host.groups.empty() && (g.host.groups[0].flags & 2), r->zscr.p, (unsigned*)r->ztick.p,
+                         g.out32 != 0, r->zscr.p, (unsigned*)r->ztick.p,
                          (int*)r->tcerr.p, c->wait_ns, st, r->settling));
     else
       CK(launch_gemm_bf16(with64(g), b, r->nsplit, st));
@@ -960,6 +964,7 @@ struct Eng {
 
   void gemm(DevGemmBuf& g, const Bases& b, bool use_mixed, int kind = 4) {
     if (use_mixed && r->exact) {
+      if (g.out32 < 0) throw Err{TT_ERR_STATE, "exact split: mixed output forms in one GEMM plan"};
       if (!r->use_tc || !prep_tc(g, b))
         throw Err{TT_ERR_INVALID_ARG, "exact split: a GEMM plan is not eligible for the tcgen05 digit kernel"};
       for (const GSeg& sg : g.host.segs)
@@ -969,14 +974,10 @@ struct Eng {
         ensure(c, r->tcerr, 16);
         CK(cudaMemsetAsync(r->tcerr.p, 0, 16, st));
       }
-      // one output form per launch (the digit kernel is specialised on it)
-      const bool pair = !g.host.groups.empty() && (g.host.groups[0].flags & 2);
-      for (const GGroup& gg : g.host.groups)
-        if (((gg.flags & 2) != 0) != pair) throw Err{TT_ERR_STATE, "exact split: mixed output forms in one GEMM plan"};
       const long e = prof_begin(kind, g.d.flops);
       const int split = split_tiles(g);
       CK(launch_gemm_tcz(g.d.groups, g.d.segs, g.tilesp, g.ntilesp, split, tc_box(g), g.maps, b, r->zscr.p,
-                         (unsigned*)r->ztick.p, (int*)r->tcerr.p, c->wait_ns, pair, st, r->settling));
+                         (unsigned*)r->ztick.p, (int*)r->tcerr.p, c->wait_ns, g.out32 != 0, st, r->settling));
       prof_end(e);
       count();
       return;

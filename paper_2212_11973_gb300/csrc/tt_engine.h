@@ -63,6 +63,7 @@ struct DevGemmBuf {
   DBuf tileso;  // FP64 kernel's one-warp tiles (a padded state's first step)
   FTile* ordered = nullptr;
   int nordered = 0, tordered = 0;
+  int out32 = 0;    // flags bit 1 of the groups (FP32 or two-float pairs); -1: not the same in all
   bool df = false;  // gauge product of a mixed mode that runs in double-float
   int key_box = 0;  // K extent of the boxes that the maps were made for
   // autotuned kernel of a split-BF16 plan: -1 not chosen yet, else a TcKernel
