@@ -211,6 +211,7 @@ F64Shape f64_shape(const GemmPlan& p) {
   return {8, 4};
 }
 
+// (16 x 16 where that gives every SM sub-partition a tile)
 F64Shape f64_shape_ordered(const GemmPlan& p) {
   size_t tiles = 0;
   for (const GGroup& g : p.groups) tiles += (size_t)((g.M + 15) / 16) * ((g.N + 15) / 16);

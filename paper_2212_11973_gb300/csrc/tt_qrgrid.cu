@@ -9,7 +9,7 @@
 // of column k + 1 that one first.  A column of Q is H_0 .. H_j e_j: no CTA
 // needs another for it.  Waits are bounded (the cooperative launch makes every
 // CTA resident, so they end; a budget that runs out sets an error flag and the
-// kernel returns).
+// kernel returns, and the caller takes the one-CTA kernel).
 //
 // What bounds it: GB300 does 2 FP64 multiply-adds per clock and SM, so one CTA
 // needs 40 ms for the 1.6e8 of a 2100 x 200 matrix; over the columns they take
